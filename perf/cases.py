@@ -1,0 +1,527 @@
+"""Performance cases of the Enskog-Vlasov lattice Boltzmann library and its learned surrogate.
+
+Each case is work that a program has the library do through its public entry points:
+
+* ``lb``: one window of a lattice run.  The populations restart from the local equilibrium of
+  given fields (``lbm_reset_device``, what the surrogate's fallback does), take ``steps`` time
+  steps (``lbm_step``) and the fields are read back into planar device memory
+  (``lbm_moments_device``).  FP64 contexts have no restart: their windows continue the run.
+* ``ensemble``: many independent domains of uneven sizes advanced by the persistent batch
+  (``Batch.step``), then the fields of every domain collected on the host (``Batch.moments``).
+* ``infer``: one surrogate window of a stack of domains (``Surrogate.infer``).
+* ``train``: one training step (``Surrogate.train_step``) and its gradients on the host
+  (``sur_get_grads``), as a program that logs or clips them reads them.
+
+``exact`` restates the method in FP64 with plain torch operations.
+"""
+import math
+
+import numpy as np
+import torch
+
+import paper_2508_00577_gb300 as ev
+from paper_2508_00577_gb300 import surrogate as S
+
+# Model constants of the Carnahan-Starling fluid and of the van der Waals gas of the
+# coexistence curve; R T / R T_c -> (vapour, liquid density).
+CS = {"a": 0.1, "b": 4.0, "RTc": 0.009432870313372378, "mid": 0.14437,
+      "rho": {0.8: (0.0217232, 0.3071957), 0.85: (0.0315818, 0.2792621), 0.9: (0.0454212, 0.2480842)}}
+VDW = {"a": 9 / 392 / 16, "b": 2 / 21, "RTc": 0.004464285714285715, "mid": 3.5,
+       "rho": {0.85: (1.1190549, 6.3249911), 0.9: (1.4900957, 5.8004457), 0.95: (2.0265522, 5.1160457)}}
+KAPPA = {"cs": 0.116, "vdw": 0.0020592501694759154, "cs3d": 0.05373155671706404, "ensemble": 0.2}
+TAU = 0.3
+PRECISION = {"f64": ev.LBM_FP64, "f32": ev.LBM_FP32, "f16": ev.LBM_FP16_DEV, "bf16": ev.LBM_BF16_DEV}
+
+# Normalisation of the surrogate's fields (rho, u_x, u_y, T) and of their increment per window.
+NORM = ((0.12, 0.0, 0.0, 0.0075), (0.1, 0.01, 0.01, 0.0006), (0.002, 0.001, 0.001, 8e-5))
+
+
+# ---------------------------------------------------------------------------
+# The cases
+# ---------------------------------------------------------------------------
+
+def _lb(name, q, nx, ny, nz, steps, precision="f32", thermal=True, eos="cs", tune=False):
+    c = {"kind": "lb", "q": q, "nx": nx, "ny": ny, "nz": nz, "steps": steps, "precision": precision,
+         "thermal": thermal, "eos": eos, "tune": tune}
+    return dict(c, name=name) if name else c
+
+
+def listed():
+    return [
+        # The FP64 reference run of a small planar slab, which every other type is judged by.
+        _lb("slab_f64", 9, 64, 64, 1, 20, precision="f64"),
+        # One point of the isothermal van der Waals coexistence curve: the smallest lattice.
+        _lb("coexistence_iso", 9, 384, 4, 1, 50, thermal=False, eos="vdw"),
+        # A few droplets on an odd lattice, launch shape left to the library.
+        _lb("droplets_ragged", 9, 331, 203, 2, 50),
+        # A stack of 256^2 domains over one surrogate window of 50 steps: training data, fallback.
+        _lb("window_256x16", 9, 256, 256, 16, 50),
+        # The droplet sweep of the Laplace law, nine 1024^2 layers, autotuned as a long run is.
+        _lb("sweep_f32", 9, 1024, 1024, 9, 20, tune=True),
+        # The same with 16-bit storage.
+        _lb("sweep_f16", 9, 1024, 1024, 9, 10, precision="f16", tune=True),
+        # A small three-dimensional lattice with odd sides.
+        _lb("spinodal_ragged", 27, 75, 50, 61, 20),
+        # The 256^3 spinodal decomposition, FP32 and 16-bit storage.
+        _lb("spinodal_f32", 27, 256, 256, 256, 8, tune=True),
+        _lb("spinodal_bf16", 27, 256, 256, 256, 4, precision="bf16", tune=True),
+        # Uneven droplet-pair domains (64..512 per side) advanced together.
+        {"name": "ensemble_32", "kind": "ensemble", "domains": 32, "side_max": 512, "steps": 400, "layout": 1},
+        # A surrogate window of the rollout's 32 domains, and a training step of a batch of 16.
+        {"name": "infer_256x32", "kind": "infer", "h": 256, "w": 256, "batch": 32},
+        {"name": "train_256x16", "kind": "train", "h": 256, "w": 256, "batch": 16},
+    ]
+
+
+def _log(rng, lo, hi):
+    return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
+
+
+def draw(rng):
+    kind = rng.choice(["lb2", "lb2", "lb2", "lb3", "lb3", "ensemble", "infer", "train"])
+    if kind == "lb2":
+        nx, ny = _log(rng, 24, 1400), _log(rng, 4, 1400)
+        nz = _log(rng, 1, max(1, min(24, 9_000_000 // (nx * ny))))
+        precision = rng.choice(["f32", "f32", "f32", "f16", "bf16", "f64"])
+        thermal = rng.random() < 0.7
+        most = {"f32": 160_000_000, "f16": 80_000_000, "bf16": 80_000_000, "f64": 16_000_000}[precision]
+        if precision == "f64":
+            nx, ny, nz = min(nx, 400), min(ny, 400), min(nz, 4)
+        steps = max(2, min(rng.choice([10, 20, 50]), most // (nx * ny * nz)))
+        eos = "cs" if thermal else rng.choice(["cs", "vdw"])
+        return _lb(None, 9, nx, ny, nz, steps, precision, thermal, eos, rng.random() < 0.4)
+    if kind == "lb3":
+        nx, ny, nz = (_log(rng, 12, 200) for _ in range(3))
+        precision = rng.choice(["f32", "f32", "f16", "bf16"])
+        steps = max(2, min(20, 40_000_000 // (nx * ny * nz)))
+        return _lb(None, 27, nx, ny, nz, steps, precision, rng.random() < 0.8, "cs", rng.random() < 0.5)
+    if kind == "ensemble":
+        return {"kind": "ensemble", "domains": rng.randint(3, 24), "side_max": rng.choice([160, 288, 512]),
+                "steps": rng.randint(50, 300), "layout": rng.randint(2, 1 << 20)}
+    h, w = rng.choice([16, 32, 64, 128, 256]), rng.choice([32, 64, 128, 256])
+    most = max(1, (1 << 21 if kind == "infer" else 1 << 20) // (h * w))
+    return {"kind": kind, "h": h, "w": w, "batch": _log(rng, 1, min(48, most))}
+
+
+# ---------------------------------------------------------------------------
+# Inputs, made on the GPU from the seed
+# ---------------------------------------------------------------------------
+
+def _gen(seed, salt=0):
+    g = torch.Generator(device="cuda")
+    g.manual_seed((int(seed) * 1000003 + salt) & 0x7FFFFFFF)
+    return g
+
+
+def _uniform(g, n, lo, hi):
+    return (lo + (hi - lo) * torch.rand(n, generator=g, device="cuda", dtype=torch.float64)).tolist()
+
+
+def _flow(g, shape, amplitude):
+    """One velocity component: three long periodic waves, [nz][ny][nx]."""
+    out = torch.zeros(shape, device="cuda")
+    for _ in range(3):
+        phase = torch.full((1, 1, 1), _uniform(g, 1, 0.0, 6.28)[0], device="cuda")
+        for axis, n in enumerate(shape):
+            k = int(_uniform(g, 1, 1.0, 3.0)[0])
+            x = torch.arange(n, device="cuda") * (2 * math.pi * k / n)
+            phase = phase + x.reshape([-1 if a == axis else 1 for a in range(3)])
+        out += amplitude * torch.sin(phase)
+    return out
+
+
+def _periodic(n, centre):
+    d = torch.arange(n, device="cuda", dtype=torch.float32) - centre
+    return d - n * torch.round(d / n)
+
+
+def _droplets(g, nx, ny, nz, eos, thermal_states, width=6.0):
+    """Planar fields [4][nz*ny*nx] of layers with one droplet each (a slab where the layer is
+    too flat for one), coexisting densities, a slow long-wave flow."""
+    fields = torch.empty((4, nz, ny, nx), device="cuda")
+    for z in range(nz):
+        cx, cy, r, pick = _uniform(g, 4, 0.0, 1.0)
+        tr = thermal_states[int(pick * len(thermal_states)) % len(thermal_states)]
+        rv, rl = eos["rho"][tr]
+        dx, dy = _periodic(nx, cx * nx), _periodic(ny, cy * ny)
+        if min(nx, ny) < 40:
+            d = (0.25 * nx - dx.abs()).reshape(1, -1).expand(ny, nx)
+        else:
+            d = (0.15 + 0.15 * r) * min(nx, ny) - torch.hypot(dx.reshape(1, -1), dy.reshape(-1, 1))
+        fields[0, z] = rv + 0.5 * (rl - rv) * (1.0 + torch.tanh(2.0 * d / width))
+        fields[3, z] = tr * eos["RTc"]
+    fields[1:3] = torch.stack([_flow(g, (nz, ny, nx), 0.002) for _ in range(2)])
+    return fields.reshape(4, -1)
+
+
+def _lb_fields(case, seed):
+    g = _gen(seed)
+    nx, ny, nz = case["nx"], case["ny"], case["nz"]
+    if case["q"] == 9:
+        eos = VDW if case["eos"] == "vdw" else CS
+        # The isothermal fluid needs wide interfaces and a temperature near the critical one.
+        states = (0.85, 0.9) if case["thermal"] else (0.9,)
+        return _droplets(g, nx, ny, nz, eos, states, width=6.0 if case["thermal"] else 8.0)
+    fields = torch.empty((5, nz, ny, nx), device="cuda")
+    noise = torch.rand((nz, ny, nx), generator=g, device="cuda")
+    fields[0] = CS["mid"] * (1.0 + 0.02 * (noise - 0.5))
+    for a in range(3):
+        fields[1 + a] = _flow(g, (nz, ny, nx), 0.002)
+    fields[4] = 0.85 * CS["RTc"]
+    return fields.reshape(5, -1)
+
+
+def _lb_model(case):
+    m = VDW if case["eos"] == "vdw" else CS
+    kappa = KAPPA["cs3d"] if case["q"] == 27 else KAPPA[case["eos"]]
+    if case["q"] == 9 and case["eos"] == "cs" and not case["thermal"]:
+        kappa = 0.14                              # 8-node interfaces at 0.9 of the critical temperature
+    return {"a": m["a"], "b": m["b"], "kappa": kappa, "eos": case["eos"], "thermal": case["thermal"]}
+
+
+def _ensemble_sizes(case):
+    """Sides in steps of 16 between 64 and side_max: the layout belongs to the case."""
+    r = np.random.default_rng(case["layout"])
+    sides = np.arange(64, case["side_max"] + 1, 16)
+    return [(int(r.choice(sides)), int(r.choice(sides))) for _ in range(case["domains"])]
+
+
+def _ensemble_fields(case, seed):
+    g = _gen(seed, 1)
+    return [_droplets(g, nx, ny, 1, CS, (0.85, 0.9)) for nx, ny in _ensemble_sizes(case)]
+
+
+def _sur_fields(case, seed):
+    g = _gen(seed, 2)
+    x = _droplets(g, case["w"], case["h"], case["batch"], CS, (0.8, 0.85, 0.9))
+    inc = torch.randn(x.shape, generator=g, device="cuda")
+    return x.contiguous(), (x + inc * torch.tensor(NORM[2], device="cuda").reshape(4, 1)).contiguous()
+
+
+def _sur_params(seed):
+    """Weights as after an initialisation: uniform in +-sqrt(6 / fan_in), small biases."""
+    g = _gen(seed, 3)
+    layout, n = S.param_layout()
+    p = torch.zeros(n, device="cuda")
+    for name, off, shape in layout:
+        k = int(np.prod(shape))
+        if name.endswith(".b"):
+            p[off:off + k] = 0.02 * (torch.rand(k, generator=g, device="cuda") - 0.5)
+            continue
+        i = int(name[4:-2]) if name.startswith("conv") else -1
+        if i >= 0:
+            cin = S.CONV_IO[i][0]
+            used, fan = 9 * cin, 9 * (4 if i == 0 else cin)
+            w = math.sqrt(6 / fan) * (2 * torch.rand(used, shape[1], generator=g, device="cuda") - 1)
+            if i == 0:
+                w.reshape(9, 8, shape[1])[:, 4:] = 0
+            p[off:off + used * shape[1]] = w.reshape(-1)
+        else:
+            w = math.sqrt(6 / shape[1]) * (2 * torch.rand(k, generator=g, device="cuda") - 1)
+            p[off:off + k] = (0.1 if name.startswith("head") else 1.0) * w
+    return p
+
+
+_stream = None
+
+
+def _sur_stream():
+    """The stream all models of this process share."""
+    global _stream
+    if _stream is None:
+        _stream = torch.cuda.Stream()
+    return _stream.cuda_stream
+
+
+# ---------------------------------------------------------------------------
+# prepare / run
+# ---------------------------------------------------------------------------
+
+def prepare(case, seed):
+    if case["kind"] == "lb":
+        fields = _lb_fields(case, seed).contiguous()
+        m = _lb_model(case)
+        p = ev.lbm_params.make(lattice=ev.LBM_D2Q9 if case["q"] == 9 else ev.LBM_D3Q27, nx=case["nx"], ny=case["ny"],
+                               nz=case["nz"], eos=ev.LBM_EOS_VDW if case["eos"] == "vdw" else ev.LBM_EOS_CS,
+                               a=m["a"], b=m["b"], kappa=m["kappa"], tau=TAU, thermal=1 if case["thermal"] else 0,
+                               precision=PRECISION[case["precision"]])
+        host = fields.double().cpu().numpy()
+        lat = ev.Lattice(p, host[0], host[1:-1], host[-1])
+        if case["tune"]:
+            ev.lbm_autotune(lat.ctx, 3)
+        return {"case": case, "lat": lat, "in": fields, "out": torch.empty_like(fields), "N": p.N}
+    if case["kind"] == "ensemble":
+        fields = [f.double().cpu().numpy() for f in _ensemble_fields(case, seed)]
+        p = ev.lbm_params.make(eos=ev.LBM_EOS_CS, a=CS["a"], b=CS["b"], kappa=KAPPA["ensemble"], tau=TAU)
+        bt = ev.Batch(p, _ensemble_sizes(case), [f[0] for f in fields], [f[1:3] for f in fields],
+                      [f[3] for f in fields])
+        bt.autotune(4)
+        return {"case": case, "batch": bt, "out": np.empty((4, bt.nodes()), np.float32)}
+    x, y = _sur_fields(case, seed)
+    model = S.Surrogate(case["h"], case["w"], seed=0, stream=_sur_stream())
+    model.set_norm(*NORM)
+    model.set_params(_sur_params(seed).cpu().numpy())
+    st = {"case": case, "model": model, "x": x, "y": y}
+    if case["kind"] == "infer":
+        st["out"] = torch.empty_like(x)
+    else:
+        st["grads"] = torch.empty(model.n, dtype=torch.float32).pin_memory().numpy()
+    torch.cuda.synchronize()
+    return st
+
+
+def run(state):
+    case = state["case"]
+    if case["kind"] == "lb":
+        ctx, N = state["lat"].ctx, state["N"]
+        T = 4 * (state["in"].shape[0] - 1) * N        # byte offset of the temperature
+        if case["precision"] != "f64":
+            src = state["in"].data_ptr()
+            ev.lbm_reset_device(ctx, src, src + 4 * N, src + T)
+        ev.lbm_step(ctx, case["steps"])
+        dst = state["out"].data_ptr()
+        ev.lbm_moments_device(ctx, dst, dst + 4 * N, dst + T)
+        return state["out"]
+    if case["kind"] == "ensemble":
+        bt, out = state["batch"], state["out"]
+        bt.step(case["steps"])
+        at = 0
+        for d, (nx, ny) in enumerate(bt.sizes):
+            rho, u, T = bt.moments(d)
+            sl = slice(at, at + nx * ny)
+            out[0, sl], out[1:3, sl], out[3, sl] = rho, u, T
+            at += nx * ny
+        return out
+    m = state["model"]
+    if case["kind"] == "infer":
+        m.infer(state["x"].data_ptr(), state["out"].data_ptr(), case["batch"])
+        return state["out"]
+    loss = m.train_step(state["x"].data_ptr(), state["y"].data_ptr(), case["batch"], 1e-4)
+    S.sur_get_grads(m.m, state["grads"])
+    return {"loss": loss, "grads": state["grads"]}
+
+
+# ---------------------------------------------------------------------------
+# work
+# ---------------------------------------------------------------------------
+
+# Floating-point operations of a lattice update with the stencils and equilibria factored.
+FLOPS_PER_UPDATE = {(9, True): 700, (9, False): 330, (27, True): 2400, (27, False): 1100}
+UNET_FLOPS_PER_PIXEL = 17.93e9 / 65536
+
+
+def work(case):
+    if case["kind"] == "lb":
+        N = case["nx"] * case["ny"] * case["nz"]
+        # A step reads and writes every population (and, in 16 bits, the 24-byte record) once.
+        size = {"f64": 8, "f32": 4, "f16": 2, "bf16": 2}[case["precision"]]
+        per = 2 * case["q"] * size * (2 if case["thermal"] else 1) + (48 if size == 2 else 0)
+        fields = 4 * (5 if case["q"] == 27 else 4) * (1 if case["precision"] == "f64" else 2)
+        return {"bytes": N * (per * case["steps"] + fields),
+                "flops": N * case["steps"] * FLOPS_PER_UPDATE[case["q"], case["thermal"]]}
+    if case["kind"] == "ensemble":
+        N = sum(nx * ny for nx, ny in _ensemble_sizes(case))
+        return {"bytes": N * (144 * case["steps"] + 16), "flops": N * case["steps"] * FLOPS_PER_UPDATE[9, True]}
+    pixels = case["h"] * case["w"] * case["batch"]
+    _, n = S.param_layout()
+    if case["kind"] == "infer":
+        return {"bytes": pixels * 32 + 2 * n, "flops": pixels * UNET_FLOPS_PER_PIXEL}
+    # Training reads the parameters and Adam's moments and writes them and the gradients.
+    return {"bytes": pixels * 32 + 28 * n, "flops": 3 * pixels * UNET_FLOPS_PER_PIXEL}
+
+
+# ---------------------------------------------------------------------------
+# FP64 restatement with plain torch operations
+# ---------------------------------------------------------------------------
+
+class _Exact:
+    """The lattice Boltzmann step in FP64 on fields [nz][ny][nx]; velocity i = (cx, cy, cz)."""
+
+    def __init__(self, q, m, RT):
+        self.q, self.m, self.RT0 = q, m, RT
+        self.D = 2 if q == 9 else 3
+        self.c = [(i % 3 - 1, (i // 3) % 3 - 1, i // 9 - 1 if q == 27 else 0) for i in range(q)]
+        self.w = [math.prod((2 / 3 if c == 0 else 1 / 6) for c in ci[:self.D]) for ci in self.c]
+        beta = 1.0 / (2.0 * TAU + 1.0)
+        self.ceq, self.cst = 2.0 * beta, 1.0 - beta
+
+    @staticmethod
+    def at(phi, c):
+        """phi(x + c)."""
+        dims = [2 - a for a in range(3) if c[a]]
+        return torch.roll(phi, [-c[a] for a in range(3) if c[a]], dims) if dims else phi
+
+    def grad(self, phi, a):
+        return 3.0 * sum(w * c[a] * self.at(phi, c) for w, c in zip(self.w, self.c) if c[a])
+
+    def diff(self, phi, a):
+        e = [0, 0, 0]
+        e[a] = 1
+        return 0.5 * (self.at(phi, e) - self.at(phi, [-v for v in e]))
+
+    def eos(self, rho):
+        if self.m["eos"] == "vdw":
+            Z = 1.0 / (1.0 - self.m["b"] * rho)
+            dln = self.m["b"] * rho * Z
+        else:
+            e = self.m["b"] * rho / 4.0
+            num, om = 1.0 + e + e * e - e ** 3, 1.0 - e
+            Z = num / om ** 3
+            dln = e * (4.0 + 4.0 * e - 2.0 * e * e) / (om * num)
+        return Z, (1.0 + dln + 2.0 / 3.0 * Z if self.m["thermal"] else 1.0 + dln)
+
+    @staticmethod
+    def psi(a0, a1, a2):
+        """The factors of c = -1, 0, 1."""
+        return (0.5 * (a2 - a1), a0 - a2, 0.5 * (a2 + a1))
+
+    def feq(self, rho, u, zeta):
+        P = [self.psi(1.0, u[a], zeta[a]) for a in range(self.D)]
+        return [rho * math.prod(P[a][c[a] + 1] for a in range(self.D)) for c in self.c]
+
+    def geq(self, rho, u, th, RT):
+        P = [self.psi(1.0, v, th + v * v) for v in u]
+        T = [self.psi(0.5 * v * v, th * v + 0.5 * v ** 3, th * th + 2.5 * th * v * v + 0.5 * v ** 4) for v in u]
+        out = []
+        for c in self.c:
+            s = 1.5 * RT * math.prod(P[a][c[a] + 1] for a in range(self.D))
+            for b in range(self.D):
+                s = s + math.prod((T if a == b else P)[a][c[a] + 1] for a in range(self.D))
+            out.append(rho * s)
+        return out
+
+    def start(self, rho, u, RT):
+        Z, _ = self.eos(rho)
+        th = RT * Z
+        f = torch.stack(self.feq(rho, u, [th + v * v for v in u]))
+        return f, (torch.stack(self.geq(rho, u, th, RT)) if self.m["thermal"] else None)
+
+    def macro(self, f, g):
+        fs = [self.at(f[i], [-v for v in c]) for i, c in enumerate(self.c)]
+        gs = [self.at(g[i], [-v for v in c]) for i, c in enumerate(self.c)] if g is not None else None
+        rho = sum(fs)
+        a, kappa = self.m["a"], self.m["kappa"]
+        gr = [self.grad(rho, k) for k in range(self.D)]
+        lap = 6.0 * sum(w * (self.at(rho, c) - rho) for w, c in zip(self.w, self.c))
+        s = -a * rho * rho - kappa * rho * lap - 0.5 * kappa * sum(v * v for v in gr)
+        F = []
+        for p in range(self.D):
+            F.append(-sum(self.grad((s if p == r else 0.0) + kappa * gr[p] * gr[r], r) for r in range(self.D)))
+        j = [sum(c[k] * fs[i] for i, c in enumerate(self.c) if c[k]) for k in range(self.D)]
+        u = [(j[k] + 0.5 * F[k]) / rho for k in range(self.D)]
+        if gs is None:
+            return fs, gs, rho, u, self.RT0, F
+        E = (sum(gs) + 0.5 * sum(x * y for x, y in zip(u, F))) / rho
+        return fs, gs, rho, u, 2.0 / 3.0 * (E - 0.5 * sum(v * v for v in u)), F
+
+    def step(self, f, g):
+        """Advances f and g in place."""
+        fs, gs, rho, u, RT, F = self.macro(f, g)
+        Z, g0 = self.eos(rho)
+        th = RT * Z
+        P0 = rho * th
+        Phi1 = P0 * (5.0 / 3.0 - g0) * sum(self.diff(u[k], k) for k in range(self.D))
+        Phi = [Phi1 - self.diff(rho * v * (v * v + 3.0 * th - 1.0), k) for k, v in enumerate(u)]
+        us = [v + x / rho for v, x in zip(u, F)]
+        feq = self.feq(rho, u, [th + v * v for v in u])
+        fst = self.feq(rho, us, [th + v * v + x / rho for v, x in zip(us, Phi)])
+        for i in range(self.q):
+            f[i].copy_(fs[i] + self.ceq * (feq[i] - fs[i]) + self.cst * (fst[i] - feq[i]))
+        if gs is None:
+            return
+        q = [P0 * self.diff(th - RT, k) + u[k] * Phi1 for k in range(self.D)]
+        geq = self.geq(rho, u, th, RT)
+        gst = self.geq(rho, us, th, RT - sum(v * v for v in F) / (3.0 * rho * rho))
+        for i, c in enumerate(self.c):
+            if sum(v * v for v in c) == 1:
+                gst[i] = gst[i] + 0.5 * sum(c[k] * q[k] for k in range(self.D))
+            g[i].copy_(gs[i] + self.ceq * (geq[i] - gs[i]) + self.cst * (gst[i] - geq[i]))
+
+
+def _exact_lb(q, m, fields, shape, steps):
+    """Planar FP64 fields after `steps` steps from the local equilibrium of planar `fields`."""
+    F = fields.double().reshape((-1,) + shape)
+    rho, u, RT = F[0].clone(), [v.clone() for v in F[1:-1]], F[-1].clone()
+    x = _Exact(q, m, RT)
+    f, g = x.start(rho, u, RT)
+    if steps * math.prod(shape) < 200_000_000 and steps > 60:      # many small steps: replay one of them
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            x.step(f, g)
+        torch.cuda.current_stream().wait_stream(side)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            x.step(f, g)
+        for _ in range(steps - 1):
+            graph.replay()
+        torch.cuda.synchronize()
+    else:
+        for _ in range(steps):
+            x.step(f, g)
+    _, _, rho, u, RT, _ = x.macro(f, g)
+    return torch.stack([rho, *u, RT]).reshape(fields.shape)
+
+
+def _exact_unet(case, seed):
+    layout, n = S.param_layout()
+    p = _sur_params(seed)
+    view, leaf = {}, p.double()
+    for name, off, shape in layout:                  # the convolutions' weights are BF16 by definition
+        k = int(np.prod(shape))
+        if name.endswith(".w") and not name.startswith("head"):
+            leaf[off:off + k] = p[off:off + k].bfloat16().double()
+    leaf.requires_grad_(case["kind"] == "train")
+    for name, off, shape in layout:
+        view[name] = leaf[off:off + int(np.prod(shape))].reshape(shape)
+    B, H, W = case["batch"], case["h"], case["w"]
+    x, y = (v.double() for v in _sur_fields(case, seed))
+    mean, scale, out_scale = (torch.tensor(v, device="cuda").double() for v in NORM)
+    nhwc = lambda v: v.reshape(4, B, H, W).permute(1, 2, 3, 0)  # noqa: E731
+
+    def conv(i, t):
+        cin, cout = S.CONV_IO[i]
+        wt = view[f"conv{i}.w"][:9 * cin].reshape(9, cin, cout)
+        z = view[f"conv{i}.b"]
+        for k in range(9):
+            z = z + torch.roll(t, (1 - k // 3, 1 - k % 3), (1, 2)) @ wt[k]
+        return z * torch.sigmoid(z)
+
+    def pool(t):
+        b, h, w, c = t.shape
+        return t.reshape(b, h // 2, 2, w // 2, 2, c).mean((2, 4))
+
+    def up(j, t):
+        b, h, w, cin = t.shape
+        cout = S.UP_IO[j][1]
+        o = (t @ view[f"up{j}.w"].T).reshape(b, h, w, 2, 2, cout) + view[f"up{j}.b"]
+        return o.permute(0, 1, 3, 2, 4, 5).reshape(b, 2 * h, 2 * w, cout)
+
+    t = torch.cat([(nhwc(x) - mean) / scale, torch.zeros((B, H, W, 4), device="cuda", dtype=torch.float64)], 3)
+    y0 = conv(1, conv(0, t))
+    y1 = conv(3, conv(2, pool(y0)))
+    y2 = conv(5, conv(4, pool(y1)))
+    t = conv(7, conv(6, pool(y2)))
+    t = conv(9, conv(8, torch.cat([y2, up(0, t)], 3)))
+    t = conv(11, conv(10, torch.cat([y1, up(1, t)], 3)))
+    t = conv(13, conv(12, torch.cat([y0, up(2, t)], 3)))
+    o = t @ view["head.w"].T + view["head.b"]
+    if case["kind"] == "infer":
+        return x + (o * out_scale).permute(3, 0, 1, 2).reshape(4, -1)
+    loss = (o - nhwc(y - x) / out_scale).square().mean()
+    loss.backward()
+    return {"loss": float(loss), "grads": leaf.grad.cpu().numpy()}
+
+
+def exact(case, seed):
+    if case["kind"] == "lb":
+        with torch.no_grad():
+            return _exact_lb(case["q"], _lb_model(case), _lb_fields(case, seed),
+                             (case["nz"], case["ny"], case["nx"]), case["steps"])
+    if case["kind"] == "ensemble":
+        m = {"a": CS["a"], "b": CS["b"], "kappa": KAPPA["ensemble"], "eos": "cs", "thermal": True}
+        with torch.no_grad():
+            out = [_exact_lb(9, m, f, (1, ny, nx), case["steps"]) for f, (nx, ny)
+                   in zip(_ensemble_fields(case, seed), _ensemble_sizes(case))]
+        return torch.cat(out, 1).cpu().numpy()
+    return _exact_unet(case, seed)
