@@ -290,14 +290,18 @@ int lbm_step(lbm_ctx *c, int n_steps)
         int rc = ensure_scratch(c);
         if (rc) return rc;
     }
+    // The launch shape is settled once per call (small lattices are bound by the launches).
+    KParams K = c->K;
+    if (fused && K.tile_w <= 0) evlbm::fused2d_default_tile(K, &K.tile_w, &K.tile_h);
+    if (fused3 && K.tile_h <= 0) K.tile_h = evlbm::fused3d_default_chunk(c->P.precision, K);
     for (int s = 0; s < n_steps; ++s) {
         const int nx = c->cur ^ 1;
         cudaError_t e;
         if (fused)
-            e = evlbm::fused2d_step(c->P.precision, c->K, c->f[c->cur], c->g[c->cur], c->f[nx], c->g[nx], c->RT_iso,
+            e = evlbm::fused2d_step(c->P.precision, K, c->f[c->cur], c->g[c->cur], c->f[nx], c->g[nx], c->RT_iso,
                                     c->R[c->cur], c->R[nx], c->stream);
         else if (fused3)
-            e = evlbm::fused3d_step(c->P.precision, c->K, c->f[c->cur], c->g[c->cur], c->f[nx], c->g[nx], c->RT_iso,
+            e = evlbm::fused3d_step(c->P.precision, K, c->f[c->cur], c->g[c->cur], c->f[nx], c->g[nx], c->RT_iso,
                                     c->R[c->cur], c->R[nx], c->stream);
         else if (fp64(c))
             e = evlbm::ref_step_f64(c->Q, c->K, c->scratch, c->RT_iso, c->f[c->cur], c->g[c->cur], c->f[nx],
@@ -481,19 +485,25 @@ static int autotune3d(lbm_ctx *c, int probe_steps, int *tile_w, int *tile_h)
     cudaEvent_t e0, e1;
     CK(c, cudaEventCreate(&e0));
     CK(c, cudaEventCreate(&e1));
-    const int heights[] = {8, 16, 32, 64, 128, 256};
+    // The powers of two and the default of the lattice's size.
+    int heights[7], nh = 0;
+    for (int h : {evlbm::fused3d_default_chunk(c->P.precision, c->K), 8, 16, 32, 64, 128, 256}) {
+        const int H = h < c->P.nz ? h : c->P.nz;
+        bool seen = false;
+        for (int k = 0; k < nh; ++k) seen = seen || heights[k] == H;
+        if (!seen) heights[nh++] = H;
+    }
     const int nx = c->cur ^ 1;
-    float tmin[6] = {1e30f, 1e30f, 1e30f, 1e30f, 1e30f, 1e30f};
+    float tmin[7];
+    for (int hi = 0; hi < nh; ++hi) tmin[hi] = 1e30f;
     KParams K = c->K;
     cudaError_t e = cudaSuccess;
     // Two rounds over the candidates, each keeping its faster time: a single probe of a
     // few launches is not repeatable to the few per cent that separate neighbouring chunks.
     for (int round = 0; round < kAutotuneRounds; ++round)
-    for (int hi = 0; hi < 6 && e == cudaSuccess; ++hi) {
-        const int H = heights[hi] < c->P.nz ? heights[hi] : c->P.nz;
-        if (hi > 0 && H == (heights[hi - 1] < c->P.nz ? heights[hi - 1] : c->P.nz)) continue;
+    for (int hi = 0; hi < nh && e == cudaSuccess; ++hi) {
         K.tile_w = evlbm::fused3d_tile_w(c->P.precision);
-        K.tile_h = H;
+        K.tile_h = heights[hi];
         for (int s = 0; s <= probe_steps && e == cudaSuccess; ++s) {
             if (s == 1) e = cudaEventRecord(e0, c->stream);
             if (e == cudaSuccess)
@@ -511,10 +521,10 @@ static int autotune3d(lbm_ctx *c, int probe_steps, int *tile_w, int *tile_h)
     if (e != cudaSuccess) return cuda_fail(c, e, "lbm_autotune");
     int bh = 0;
     float best = 1e30f;
-    for (int hi = 0; hi < 6; ++hi)
+    for (int hi = 0; hi < nh; ++hi)
         if (tmin[hi] < best) {
             best = tmin[hi];
-            bh = heights[hi] < c->P.nz ? heights[hi] : c->P.nz;
+            bh = heights[hi];
         }
     c->K.tile_w = evlbm::fused3d_tile_w(c->P.precision);
     c->K.tile_h = bh;
@@ -533,17 +543,22 @@ int lbm_autotune(lbm_ctx *c, int probe_steps, int *tile_w, int *tile_h)
     cudaEvent_t e0, e1;
     CK(c, cudaEventCreate(&e0));
     CK(c, cudaEventCreate(&e1));
-    const int heights[] = {16, 32, 64, 128, 256, LBM_TILE_BALANCED};
+    // Last candidate of its width: the default shape of the lattice's size.
+    int dw = 0, dh = 0;
+    evlbm::fused2d_default_tile(c->K, &dw, &dh);
+    constexpr int kH = 7;
+    const int heights[kH] = {16, 32, 64, 128, 256, LBM_TILE_BALANCED, dh};
     const int nx = c->cur ^ 1;
-    std::vector<float> tmin(evlbm::kFusedWidthCount * 6, 1e30f);
+    std::vector<float> tmin(evlbm::kFusedWidthCount * kH, 1e30f);
     KParams K = c->K;
     cudaError_t e = cudaSuccess;
     for (int round = 0; round < kAutotuneRounds; ++round)
     for (int wi = 0; wi < evlbm::kFusedWidthCount && e == cudaSuccess; ++wi) {
         const int W = evlbm::kFusedWidths[wi];
         if (W > 2 * c->P.nx && W != evlbm::kFusedWidths[0]) continue;
-        for (int hi = 0; hi < 6 && e == cudaSuccess; ++hi) {
+        for (int hi = 0; hi < kH && e == cudaSuccess; ++hi) {
             const int H = heights[hi] < c->P.ny ? heights[hi] : c->P.ny;    // the balanced grid stays -1
+            if (hi == kH - 1 && (W != dw || dh == LBM_TILE_BALANCED)) continue;
             if (hi > 0 && hi < 5 && H == (heights[hi - 1] < c->P.ny ? heights[hi - 1] : c->P.ny)) continue;
             K.tile_w = W;
             K.tile_h = H;
@@ -558,7 +573,7 @@ int lbm_autotune(lbm_ctx *c, int probe_steps, int *tile_w, int *tile_h)
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
             float ms = 0.f;
             if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-            if (e == cudaSuccess && ms < tmin[wi * 6 + hi]) tmin[wi * 6 + hi] = ms;
+            if (e == cudaSuccess && ms < tmin[wi * kH + hi]) tmin[wi * kH + hi] = ms;
         }
     }
     cudaEventDestroy(e0);
@@ -567,9 +582,9 @@ int lbm_autotune(lbm_ctx *c, int probe_steps, int *tile_w, int *tile_h)
     int bw = 0, bh = 0;
     float best = 1e30f;
     for (int wi = 0; wi < evlbm::kFusedWidthCount; ++wi)
-        for (int hi = 0; hi < 6; ++hi)
-            if (tmin[wi * 6 + hi] < best) {
-                best = tmin[wi * 6 + hi];
+        for (int hi = 0; hi < kH; ++hi)
+            if (tmin[wi * kH + hi] < best) {
+                best = tmin[wi * kH + hi];
                 bw = evlbm::kFusedWidths[wi];
                 bh = heights[hi] < c->P.ny ? heights[hi] : c->P.ny;
             }

@@ -54,6 +54,7 @@ bool fused2d_supported(int prec, int Q, const KParams &p);
 // columns is fused3d_tile_w(prec) wide (32 x 8 for FP32, 16 x 16 for 16-bit storage),
 // tile_h is the z-chunk height (0 = default).
 int fused3d_tile_w(int prec);
+int fused3d_default_chunk(int prec, const KParams &p);
 bool fused3d_supported(int prec, int Q, const KParams &p);
 cudaError_t fused3d_step(int prec, const KParams &p, const void *f, const void *g, void *fo, void *go,
                          const void *RT_iso, const void *Rin, void *Rout, cudaStream_t st);

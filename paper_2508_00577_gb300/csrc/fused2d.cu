@@ -17,11 +17,60 @@ bool fused2d_supported(int prec, int Q, const KParams &p)
            (long long)9 * p.N < (1LL << 31);
 }
 
+// Default launch shape: the candidate with the least estimated time.  A CTA that marches p
+// row pairs runs p + 5 iterations per tile (the pipeline of four stages fills first), and the
+// time of one iteration depends on the strip width and on how many CTAs share an SM.  The
+// measured times of an iteration (us, thermal FP32; the ratios hold for the isothermal kernel
+// and 16-bit storage):
+//   CTAs per SM       1     2     3     4
+//   W =  64         1.28  1.60  2.20  2.90
+//   W =  96         1.20  2.25
+//   W = 128         1.50  2.35
+// so few row pairs per CTA win as long as the GPU is not full, and beyond that the wide
+// strips of the balanced grid.  Against the former rule (strips of 128 columns, 128 rows a
+// CTA), us per step: 331 x 203 x 2 104.8 -> 13.2, 512^2 104.5 -> 18.7, 256^2 x 16 123.2 ->
+// 48.9, 1024^2 122.6 -> 45.5, 256^2 x 64 161.7 -> 154.5, 64^2 45.5 -> 8.5, 384 x 4 isothermal
+// 8.5 -> 6.5 (the spacing of dependent launches).
 void fused2d_default_tile(const KParams &p, int *W, int *H)
 {
-    *W = p.nx >= 128 ? 128 : (p.nx > 64 ? 96 : 64);
-    const int h = p.ny <= 128 ? p.ny : 128;
-    *H = h + (h & 1);
+    static const int widths[3] = {128, 96, 64}, per_sm[3] = {2, 2, 4};
+    static const float iter_us[3][4] = {{1.50f, 2.35f, 0.f, 0.f}, {1.20f, 2.25f, 0.f, 0.f}, {1.28f, 1.60f, 2.20f, 2.90f}};
+    static const int heights[] = {2, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 256};
+    constexpr int kFill = 5;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        sms = 152;
+    const long long P = (p.ny + 1) / 2;                      // row pairs of a layer
+    double best = 1e300;
+    for (int k = 0; k < 3; ++k) {
+        const long long S = (p.nx + widths[k] - 1) / widths[k], slots = (long long)sms * per_sm[k];
+        auto iter = [&](long long ctas) {
+            const long long r = (ctas + sms - 1) / sms;
+            return (double)iter_us[k][r < 1 ? 0 : (r > per_sm[k] ? per_sm[k] : r) - 1];
+        };
+        auto offer = [&](double t, int h) {
+            if (t < best) {
+                best = t;
+                *W = widths[k];
+                *H = h;
+            }
+        };
+        for (int h : heights) {
+            const long long pairs = h / 2 < P ? h / 2 : P, ctas = S * ((P + pairs - 1) / pairs) * p.nz;
+            const long long waves = (ctas + slots - 1) / slots;
+            if ((P + pairs - 1) / pairs <= 65535) offer((double)(waves * (pairs + kFill)) * iter(ctas), h);
+            if (pairs == P) break;
+        }
+        // Balanced grid: equal shares of the strip's row pairs; a share that crosses the end
+        // of a layer fills the pipeline once more.
+        const long long T = P * p.nz;
+        long long parts = slots / S;
+        parts = parts < 1 ? 1 : (parts > T ? T : parts);
+        const long long share = (T + parts - 1) / parts, tiles = 1 + (share + P - 2) / P;
+        const long long waves = (S * parts + slots - 1) / slots;
+        offer((double)(waves * (share + kFill * (p.nz > 1 ? tiles : 1))) * iter(S * parts), kTileBalanced);
+    }
 }
 
 cudaError_t fused2d_step(int prec, const KParams &p, const void *f, const void *g, void *fo, void *go,

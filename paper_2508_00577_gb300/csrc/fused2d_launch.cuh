@@ -125,8 +125,8 @@ inline void launch_shape(const KParams &p, FusedArgs &A, int &W, bool &balanced)
 {
     int H = p.tile_h;
     W = p.tile_w;
-    balanced = W > 0 && H == kTileBalanced;
-    if (W <= 0 || (H <= 0 && !balanced)) fused2d_default_tile(p, &W, &H);
+    if (W <= 0 || (H <= 0 && H != kTileBalanced)) fused2d_default_tile(p, &W, &H);
+    balanced = H == kTileBalanced;
     A.H = balanced ? 0 : H + (H & 1);  // row pairs: chunks of an even number of rows
 }
 
