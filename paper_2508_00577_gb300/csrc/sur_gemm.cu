@@ -63,8 +63,6 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool v
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0));
 }
 
-__device__ __forceinline__ float silu(float z) { return z / (1.f + __expf(-z)); }
-
 // ---------------------------------------------------------------------------
 // Epilogue (shared by both mainloops)
 // ---------------------------------------------------------------------------
@@ -86,14 +84,23 @@ __device__ __forceinline__ void epilogue(const Epi &g, uint32_t tmem, long long 
 {
     const long long row = m0 + warp * 32 + lane;
     const bool rv = row < g.M;
-    long long tg[4];
-    int nt = 0;
-    long long orow = row;
-    if (rv && g.pix) {
-        if (g.epi == SUR_EPI_SHUF) nt = 0;
-        else nt = halo_targets(row, g.lh, g.lw, tg);
-        orow = pad_pix(row, g.lh, g.lw);
-    }
+    const long long orow = rv && g.pix ? pad_pix(row, g.lh, g.lw) : row;
+    // 32 consecutive bias values, as 16-byte loads where the array allows it.
+    auto add_bias = [&](float v[32], const float *b) {
+        if ((reinterpret_cast<uintptr_t>(b) & 15) == 0) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float4 q = __ldg(reinterpret_cast<const float4 *>(b) + j);
+                v[4 * j] += q.x;
+                v[4 * j + 1] += q.y;
+                v[4 * j + 2] += q.z;
+                v[4 * j + 3] += q.w;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] += __ldg(b + j);
+        }
+    };
 #pragma unroll 1
     for (int c0 = 0; c0 < BN; c0 += 32) {
         uint32_t r[32];
@@ -119,21 +126,16 @@ __device__ __forceinline__ void epilogue(const Epi &g, uint32_t tmem, long long 
             for (int j = 0; j < 32; ++j) atomicAdd(o + j, v[j]);
         } else if (g.epi == SUR_EPI_SHUF) {
             const int sidx = col / g.shuf_cout, c = col - sidx * g.shuf_cout;
-#pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] += g.bias[c + j];
+            add_bias(v, g.bias + c);
             // Child s of coarse pixel `row` on the fine grid, with its halo copies.
             const int Hc = 1 << g.lh, Wc = 1 << g.lw;
             const long long b = row >> (g.lh + g.lw);
             const int y = (int)((row >> g.lw) & (Hc - 1)), x = (int)(row & (Wc - 1));
             const long long qf = ((b * 2 * Hc + 2 * y + (sidx >> 1)) << (g.lw + 1)) | (2 * x + (sidx & 1));
-            long long ft[4];
-            const int nf = halo_targets(qf, g.lh + 1, g.lw + 1, ft);
-            for (int i = 0; i < nf; ++i) store32_bf16(g.y + ft[i] * g.ldy + g.cy0 + c, v);
+            for_halo(qf, g.lh + 1, g.lw + 1,
+                     [&](long long t) { store32_bf16(g.y + t * g.ldy + g.cy0 + c, v); });
         } else {
-            if (g.bias) {
-#pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] += g.bias[col + j];
-            }
+            if (g.bias) add_bias(v, g.bias + col);
             if (g.epi == SUR_EPI_F32) {
                 float4 *o = reinterpret_cast<float4 *>(static_cast<float *>(g.out) + orow * g.ldo + g.co0 + col);
 #pragma unroll
@@ -144,7 +146,8 @@ __device__ __forceinline__ void epilogue(const Epi &g, uint32_t tmem, long long 
 #pragma unroll
                     for (int j = 0; j < 32; ++j) v[j] = silu(v[j]);
                     if (g.pix) {
-                        for (int i = 0; i < nt; ++i) store32_bf16(g.y + tg[i] * g.ldy + g.cy0 + col, v);
+                        for_halo(row, g.lh, g.lw,
+                                 [&](long long t) { store32_bf16(g.y + t * g.ldy + g.cy0 + col, v); });
                     } else {
                         store32_bf16(g.y + row * g.ldy + g.cy0 + col, v);
                     }

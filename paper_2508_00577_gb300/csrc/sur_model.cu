@@ -195,15 +195,18 @@ int up_fwd(sur_model *m, int j, int B, const bf16 *Xc, bf16 *cat)
     return evsur::gemm(g, m->status, m->stream);
 }
 
-// dY (ld ldd) -> dZ; bias and weight gradients; dX (ld ldx, may be NULL).
-int conv_bwd(sur_model *m, int i, int B, const bf16 *X, int ldx, const bf16 *dY, int ldd, bf16 *dX, int ldxo)
+// dY (ld ldd), plus the gradient dP of the pooled output where there is one -> dZ; bias and
+// weight gradients; dX (ld ldx, may be NULL).
+int conv_bwd(sur_model *m, int i, int B, const bf16 *X, int ldx, const bf16 *dY, int ldd, bf16 *dX, int ldxo,
+             const bf16 *dP = nullptr)
 {
     const ConvL &L = m->conv[i];
     const int l = kConvLevel[i];
     const long long M = lvl_pix(m, l, B);
     const int H = lvl_h(m, l), W = lvl_w(m, l);
     // dZ and, in the same pass, the bias gradient (its column sums).
-    CK(evsur::silu_bwd(dY, ldd, m->Z[i], M, lvl_lh(m, l), lvl_lw(m, l), L.cout, m->dZ, m->G + L.b, m->stream));
+    CK(evsur::silu_bwd(dY, ldd, dP, m->Z[i], M, lvl_lh(m, l), lvl_lw(m, l), L.cout, m->dZ, m->G + L.b,
+                       m->stream));
     sur_gemm_args g{};
     g.a = gather(SUR_OP_TCONV3, X, ldx, 0, L.cin, 9LL * L.cin, H, W);
     g.b = gather(SUR_OP_TPIX, m->dZ, L.cout, 0, 0, L.cout, H, W);
@@ -271,14 +274,16 @@ int up_bwd(sur_model *m, int j, int B, const bf16 *Xc, const bf16 *dcat, bf16 *d
 
 int refresh_weights(sur_model *m)
 {
+    evsur::WeightCopy w[kConvs + kUps];
     for (int i = 0; i < kConvs; ++i) {
         const ConvL &L = m->conv[i];
-        CK(evsur::conv_weights(m->P + L.w, L.cin, L.cout, L.kp, L.kpo, L.wb, L.wf, m->stream));
+        w[i] = {m->P + L.w, L.wb, L.wf, 0, L.cin, L.cout, L.kp, L.kpo};
     }
     for (int j = 0; j < kUps; ++j) {
         const UpL &U = m->up[j];
-        CK(evsur::up_weights(m->P + U.w, U.cin, U.cout, U.wb, U.wt, m->stream));
+        w[kConvs + j] = {m->P + U.w, U.wb, U.wt, 1, U.cin, U.cout, 0, 0};
     }
+    CK(evsur::copy_weights(w, kConvs + kUps, m->stream));
     return SUR_OK;
 }
 
@@ -393,10 +398,10 @@ int forward(sur_model *m, const float *d_x, int B, bool train)
     return SUR_OK;
 }
 
+// Backward pass from the gradient dY03 of the last convolution's output (the head's, which
+// the callers compute).
 int backward(sur_model *m, int B)
 {
-    const long long M0 = lvl_pix(m, 0, B);
-    CK(evsur::head_bwd(m->Y03, M0, m->lh, m->lw, m->P + m->head_w, m->dO, m->dY03, m->G + m->head_w, m->G + m->head_b, m->stream));
     int rc;
 #define BW(expr)                 \
     if ((rc = (expr)) != SUR_OK) \
@@ -412,14 +417,11 @@ int backward(sur_model *m, int B)
     BW(up_bwd(m, 0, B, m->Y31, m->dcat2, m->dY31));
     BW(conv_bwd(m, 7, B, m->Y30, 256, m->dY31, 256, m->dY30, 256));
     BW(conv_bwd(m, 6, B, m->p2, 128, m->dY30, 256, m->dp2, 128));
-    CK(evsur::unpool2_acc(m->dp2, lvl_pix(m, 3, B), m->lh - 3, m->lw - 3, 128, m->dcat2, 256, m->stream));
-    BW(conv_bwd(m, 5, B, m->Y20, 128, m->dcat2, 256, m->dY20, 128));
+    BW(conv_bwd(m, 5, B, m->Y20, 128, m->dcat2, 256, m->dY20, 128, m->dp2));
     BW(conv_bwd(m, 4, B, m->p1, 64, m->dY20, 128, m->dp1, 64));
-    CK(evsur::unpool2_acc(m->dp1, lvl_pix(m, 2, B), m->lh - 2, m->lw - 2, 64, m->dcat1, 128, m->stream));
-    BW(conv_bwd(m, 3, B, m->Y10, 64, m->dcat1, 128, m->dY10, 64));
+    BW(conv_bwd(m, 3, B, m->Y10, 64, m->dcat1, 128, m->dY10, 64, m->dp1));
     BW(conv_bwd(m, 2, B, m->p0, 32, m->dY10, 64, m->dp0, 32));
-    CK(evsur::unpool2_acc(m->dp0, lvl_pix(m, 1, B), m->lh - 1, m->lw - 1, 32, m->dcat0, 64, m->stream));
-    BW(conv_bwd(m, 1, B, m->Y00, 32, m->dcat0, 64, m->dY00, 32));
+    BW(conv_bwd(m, 1, B, m->Y00, 32, m->dcat0, 64, m->dY00, 32, m->dp0));
     BW(conv_bwd(m, 0, B, m->xin, 8, m->dY00, 32, nullptr, 0));
 #undef BW
     return SUR_OK;
@@ -446,8 +448,8 @@ int fwd_bwd(sur_model *m, const float *d_x, const float *d_y, int B, float *loss
     CK(cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream));
     if ((rc = forward(m, d_x, B, true))) return rc;
     const long long M0 = lvl_pix(m, 0, B);
-    CK(evsur::head(m->Y03, M0, m->lh, m->lw, m->P + m->head_w, m->P + m->head_b, m->norm, d_x, d_y, 0, m->dO, m->loss, nullptr,
-                   m->stream));
+    CK(evsur::head_loss_bwd(m->Y03, M0, m->lh, m->lw, m->P + m->head_w, m->P + m->head_b, m->norm, d_x, d_y, m->loss,
+                            m->dY03, m->G + m->head_w, m->G + m->head_b, m->stream));
     if ((rc = backward(m, B))) return rc;
     if (loss) {
         CK(cudaMemcpyAsync(loss, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream));
@@ -487,14 +489,16 @@ int fwd_bwd_unrolled(sur_model *m, const float *d_x0, const float *d_targets, in
     CK(cudaMemsetAsync(Gx, 0, sizeof(float) * F, m->stream));
     for (int j = 0; j < k; ++j) {
         if ((rc = forward(m, state(j), B, false))) return rc;
-        CK(evsur::head(m->Y03, M0, m->lh, m->lw, m->P + m->head_w, m->P + m->head_b, m->norm, state(j), nullptr, 1,
-                       nullptr, nullptr, state(j + 1), m->stream));
+        CK(evsur::head_next(m->Y03, M0, m->lh, m->lw, m->P + m->head_w, m->P + m->head_b, m->norm, state(j),
+                            state(j + 1), m->stream));
     }
     const float inv = 1.f / (4.f * (float)M0 * (float)k);
     for (int j = k; j >= 1; --j) {
         CK(evsur::unroll_term(state(j), d_targets + (long long)(j - 1) * F, M0, m->norm, inv, Gx, m->dO, m->loss,
                               m->stream));
         if ((rc = forward(m, state(j - 1), B, true))) return rc;
+        CK(evsur::head_bwd(m->Y03, M0, m->lh, m->lw, m->P + m->head_w, m->dO, m->dY03, m->G + m->head_w,
+                           m->G + m->head_b, m->stream));
         if ((rc = backward(m, B))) return rc;
         // backward() leaves the first convolution's dZ in m->dZ.
         if (j > 1)
@@ -759,8 +763,7 @@ int sur_infer(sur_model *m, const float *d_x, float *d_y, int batch)
     if (rc) return rc;
     if ((rc = forward(m, d_x, batch, false))) return rc;
     const long long M0 = lvl_pix(m, 0, batch);
-    CK(evsur::head(m->Y03, M0, m->lh, m->lw, m->P + m->head_w, m->P + m->head_b, m->norm, d_x, nullptr, 1, nullptr, nullptr, d_y,
-                   m->stream));
+    CK(evsur::head_next(m->Y03, M0, m->lh, m->lw, m->P + m->head_w, m->P + m->head_b, m->norm, d_x, d_y, m->stream));
     return SUR_OK;
 }
 
@@ -797,8 +800,8 @@ int sur_rollout(sur_model *m, lbm_ctx *lb, float *d_fields, int batch, const sur
     bool lb_current = false;
     for (int w = 0; w < cfg->windows; ++w) {
         if ((rc = forward(m, d_fields, batch, false))) return rc;
-        CK(evsur::head(m->Y03, N, m->lh, m->lw, m->P + m->head_w, m->P + m->head_b, m->norm, d_fields, nullptr, 1,
-                       nullptr, nullptr, m->next, m->stream));
+        CK(evsur::head_next(m->Y03, N, m->lh, m->lw, m->P + m->head_w, m->P + m->head_b, m->norm, d_fields, m->next,
+                            m->stream));
         if ((rc = measure(m->next, nxt, &bad))) return rc;
         if (cfg->project_mass && !bad) {
             for (int b = 0; b < batch; ++b) delta[b] = (float)((nxt[2 * b] - mass0[b]) / (double)Mb);

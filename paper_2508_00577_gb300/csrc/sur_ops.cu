@@ -1,9 +1,10 @@
 // Elementwise and reduction kernels of the learned surrogate on halo-padded
-// NHWC tensors (see surrogate.cuh): SiLU backward, bias gradients, 2x2 average
-// pooling and its adjoint, input packing, the 1x1 head with the loss or the
-// state update, the loss terms and first-layer input gradient of unrolled
-// training, Adam, the BF16 operand copies of the weights, and the per-domain
-// fallback indicators.
+// NHWC tensors (see surrogate.cuh): SiLU backward (with the pooling's adjoint), bias
+// gradients, 2x2 average pooling, input packing, the 1x1 head with the loss and its
+// gradients or the state update, the loss terms and first-layer input gradient of
+// unrolled training, Adam, the BF16 operand copies of the weights, and the per-domain
+// fallback indicators.  The kernels over activations are bound by HBM: 16-byte accesses,
+// consecutive threads on consecutive bytes, pixel indices by shifts.
 #include <stdint.h>
 
 #include "surrogate.cuh"
@@ -18,12 +19,20 @@ inline int grid_1d(long long n)
     return (int)(g > 8192 ? 8192 : (g < 1 ? 1 : g));
 }
 
-// Kernels that end in per-channel atomics (block_colsum8): at most 512 blocks, so that
-// each channel's accumulator takes at most 512 atomic additions per call.
-inline int grid_red(long long n)
+// Grid of the activation kernels: what is resident at once (per_sm blocks of 256 threads, by
+// registers, on each of the 152 SMs), each block striding over the tensor.  Those that end in
+// per-channel atomics (block_colsum8) so add at most 152 per_sm values to each accumulator.
+inline int grid_res(long long n, int per_sm)
 {
     const int g = grid_1d(n);
-    return g > 512 ? 512 : g;
+    return g > 152 * per_sm ? 152 * per_sm : g;
+}
+
+inline int log2i(int v)
+{
+    int l = 0;
+    while ((1 << l) < v) ++l;
+    return l;
 }
 
 #define GRID_STRIDE(e, total)                                                                    \
@@ -50,50 +59,69 @@ __device__ __forceinline__ void block_colsum8(const float acc[8], int C8, float 
 
 // dZ = dY * silu'(Z), silu'(z) = s (1 + z (1 - s)) with s = 1 / (1 + e^-z);
 // 8 channels per thread; dZ gets its halo copies (it is gathered by the adjoint
-// convolution).  dbias (may be NULL) += the column sums of the stored (BF16) dZ over
-// the interior pixels: the bias gradient, without a second pass over dZ.
-__global__ void __launch_bounds__(256) k_silu_bwd(const bf16 *dY, int ldd, const bf16 *Z, long long M, int lh,
-                                                  int lw, int C, bf16 *dZ, float *dbias)
+// convolution).  dbias += the column sums of the stored (BF16) dZ over the interior
+// pixels: the bias gradient, without a second pass over dZ.  POOL: the layer's output also
+// went into the 2x2 average pooling, whose gradient dP (coarse grid, halo-padded, ld C)
+// adds a quarter to each child; the sum is rounded to BF16 as a stored gradient would be.
+// C8 = C / 8 = 1 << c8s.
+// Bound by HBM: 6 bytes per element (4 + 2), and the divide of s, whose slow-path branch
+// serialised the eight channels, was most of the rest: 71 us at 2^20 pixels x 32 channels
+// with it, 512 blocks, 64-bit divisions and a halo list in local memory.
+template <bool POOL>
+__global__ void __launch_bounds__(256, POOL ? 4 : 5) k_silu_bwd(const bf16 *dY, int ldd, const bf16 *dP, const bf16 *Z, long long M,
+                                                  int lh, int lw, int c8s, bf16 *dZ, float *dbias)
 {
-    const int C8 = C >> 3;
+    const int C8 = 1 << c8s, C = C8 << 3;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    GRID_STRIDE(e, M * C8)
+    GRID_STRIDE(e, M << c8s)
     {
-        const long long m = e / C8;
-        const int c = (int)(e - m * C8) << 3;
+        const long long m = e >> c8s;
+        const int c = (int)(e & (C8 - 1)) << 3;
         const long long p = pad_pix(m, lh, lw);
         const uint4 dv = *reinterpret_cast<const uint4 *>(dY + p * ldd + c);
         const uint4 zv = *reinterpret_cast<const uint4 *>(Z + p * C + c);
         const bf16 *dh = reinterpret_cast<const bf16 *>(&dv), *zh = reinterpret_cast<const bf16 *>(&zv);
-        float o[8];
+        float d[8], o[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) d[j] = __bfloat162float(dh[j]);
+        if constexpr (POOL) {
+            const int H = 1 << lh, W = 1 << lw;
+            const long long b = m >> (lh + lw);
+            const int y = (int)((m >> lw) & (H - 1)), x = (int)(m & (W - 1));
+            const long long pc = (b * (H / 2 + 2) + y / 2 + 1) * (W / 2 + 2) + x / 2 + 1;
+            const uint4 pv = *reinterpret_cast<const uint4 *>(dP + pc * C + c);
+            const bf16 *ph = reinterpret_cast<const bf16 *>(&pv);
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                d[j] = __bfloat162float(__float2bfloat16_rn(d[j] + 0.25f * __bfloat162float(ph[j])));
+        }
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const float z = __bfloat162float(zh[j]);
-            const float s = 1.f / (1.f + __expf(-z));
-            o[j] = __bfloat162float(dh[j]) * s * (1.f + z * (1.f - s));
+            const float s = sigmoid(z);
+            o[j] = d[j] * s * (1.f + z * (1.f - s));
         }
         const uint4 ov = pack8(o);
         const bf16 *oh = reinterpret_cast<const bf16 *>(&ov);
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[j] += __bfloat162float(oh[j]);
-        long long tg[4];
-        const int n = halo_targets(m, lh, lw, tg);
-        for (int i = 0; i < n; ++i) *reinterpret_cast<uint4 *>(dZ + tg[i] * C + c) = ov;
+        for_halo(m, lh, lw, [&](long long t) { *reinterpret_cast<uint4 *>(dZ + t * C + c) = ov; });
     }
     if (dbias) block_colsum8(acc, C8, dbias);
 }
 
 // out[c] += sum over interior pixels of X[pix*ldx + c], c < C (bias gradients), 8
 // channels (16 bytes) per load.
-__global__ void __launch_bounds__(256) k_colsum(const bf16 *X, int ldx, long long M, int lh, int lw, int C,
+__global__ void __launch_bounds__(256) k_colsum(const bf16 *X, int ldx, long long M, int lh, int lw, int c8s,
                                                 float *out)
 {
-    const int C8 = C >> 3;
+    const int C8 = 1 << c8s;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    GRID_STRIDE(e, M * C8)
+#pragma unroll 4
+    GRID_STRIDE(e, M << c8s)
     {
-        const long long m = e / C8;
-        const int c = (int)(e - m * C8) << 3;
+        const long long m = e >> c8s;
+        const int c = (int)(e & (C8 - 1)) << 3;
         const uint4 v = *reinterpret_cast<const uint4 *>(X + pad_pix(m, lh, lw) * ldx + c);
         const bf16 *h = reinterpret_cast<const bf16 *>(&v);
 #pragma unroll
@@ -103,40 +131,32 @@ __global__ void __launch_bounds__(256) k_colsum(const bf16 *X, int ldx, long lon
 }
 
 // 2x2 average pooling: X (fine grid, ld ldx, first C channels) -> Y (coarse grid
-// 2^lh x 2^lw, ld C) with halo copies.
-__global__ void k_pool2(const bf16 *X, int ldx, long long Mc, int lh, int lw, int C, bf16 *Y)
+// 2^lh x 2^lw, ld C) with halo copies; 8 channels per thread (one channel per thread, with
+// 2-byte accesses, took 46 us at 2^18 coarse pixels x 32 channels).
+__global__ void __launch_bounds__(256) k_pool2(const bf16 *X, int ldx, long long Mc, int lh, int lw, int c8s, bf16 *Y)
 {
-    const int Wf2 = 2 * (1 << lw) + 2;
-    GRID_STRIDE(e, Mc * C)
+    const int Wf2 = 2 * (1 << lw) + 2, C8 = 1 << c8s, C = C8 << 3;
+    GRID_STRIDE(e, Mc << c8s)
     {
-        const long long q = e / C;
-        const int c = (int)(e - q * C);
-        const long long f = child0(q, lh, lw);
-        const float s = __bfloat162float(X[f * ldx + c]) + __bfloat162float(X[(f + 1) * ldx + c]) +
-                        __bfloat162float(X[(f + Wf2) * ldx + c]) + __bfloat162float(X[(f + Wf2 + 1) * ldx + c]);
-        const bf16 v = __float2bfloat16_rn(0.25f * s);
-        long long tg[4];
-        const int n = halo_targets(q, lh, lw, tg);
-        for (int i = 0; i < n; ++i) Y[tg[i] * C + c] = v;
-    }
-}
-
-// Adjoint of the pooling, accumulated into the interior: dX[child] += dY[q] / 4.
-__global__ void k_unpool2_acc(const bf16 *dY, long long Mc, int lh, int lw, int C, bf16 *dX, int ldx)
-{
-    const int Wf2 = 2 * (1 << lw) + 2;
-    GRID_STRIDE(e, Mc * C)
-    {
-        const long long q = e / C;
-        const int c = (int)(e - q * C);
-        const float d = 0.25f * __bfloat162float(dY[pad_pix(q, lh, lw) * C + c]);
-        const long long f = child0(q, lh, lw);
-        const long long fs[4] = {f, f + 1, f + Wf2, f + Wf2 + 1};
+        const long long q = e >> c8s;
+        const int c = (int)(e & (C8 - 1)) << 3;
+        const bf16 *f = X + child0(q, lh, lw) * ldx + c;
+        const uint4 v[4] = {*reinterpret_cast<const uint4 *>(f), *reinterpret_cast<const uint4 *>(f + ldx),
+                            *reinterpret_cast<const uint4 *>(f + (long long)Wf2 * ldx),
+                            *reinterpret_cast<const uint4 *>(f + (long long)(Wf2 + 1) * ldx)};
+        float o[8];
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            bf16 *p = dX + fs[s] * ldx + c;
-            *p = __float2bfloat16_rn(__bfloat162float(*p) + d);
+        for (int j = 0; j < 8; ++j) {
+            float s = 0.f;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float t = __bfloat162float(reinterpret_cast<const bf16 *>(&v[k])[j]);
+                s = k ? s + t : t;
+            }
+            o[j] = 0.25f * s;
         }
+        const uint4 ov = pack8(o);
+        for_halo(q, lh, lw, [&](long long t) { *reinterpret_cast<uint4 *>(Y + t * C + c) = ov; });
     }
 }
 
@@ -152,67 +172,142 @@ __global__ void k_pack_in(const float *x, long long M, int lh, int lw, const flo
 #pragma unroll
         for (int c = 4; c < 8; ++c) v[c] = 0.f;
         const uint4 pv = pack8(v);
-        long long tg[4];
-        const int n = halo_targets(m, lh, lw, tg);
-        for (int i = 0; i < n; ++i) *reinterpret_cast<uint4 *>(X + tg[i] * 8) = pv;
+        for_halo(m, lh, lw, [&](long long t) { *reinterpret_cast<uint4 *>(X + t * 8) = pv; });
     }
 }
 
-// 1x1 head (C -> 4) and its use: mode 0 = loss against targets, mode 1 = next state.
+// 1x1 head (32 -> 4 channels) and its use:
 //   o[m][k] = bh[k] + sum_c Y[m][c] Wh[k][c]
-//   mode 0: r = o - (y - x)/out_scale; loss += r^2 / (4M); dO[m][k] = 2 r / (4M)
-//   mode 1: xn[k][m] = x[k][m] + out_scale[k] o[m][k]
-template <int C>
-__global__ void k_head(const bf16 *Y, long long M, int lh, int lw, const float *Wh, const float *bh,
-                       const float *norm, const float *x, const float *yt, int mode, float *dO, float *loss,
-                       float *xn)
+//   kHeadNext: xn[k][m] = x[k][m] + out_scale[k] o[m][k]
+//   kHeadLoss: r = o - (yt - x)/out_scale; loss += r^2 / (4M); dO = 2 r / (4M); then the
+//              head's backward pass on dO
+//   kHeadBwd:  the backward pass on a given dO [M][4]:
+//              dY[m][c] = sum_k dO[m][k] Wh[k][c]; dWh[k][c] += sum_m dO[m][k] Y[m][c];
+//              dbh[k] += sum_m dO[m][k]
+// A block stages the 64-byte rows of 256 pixels in shared memory (80-byte pitch: 16-byte
+// reads of consecutive rows hit distinct banks), so that global accesses are whole lines;
+// thread = pixel for o, lane = channel (a warp on its own 32 pixels) for the backward pass,
+// which overwrites the staged Y with dY.  Bound by HBM: Y read once, dY written once.  As
+// separate kernels, with each thread reading its pixel's 64 bytes itself, loss + backward
+// took 110 + 129 us at 2^20 pixels and the state update 166 us at 2^21.
+enum { kHeadNext, kHeadLoss, kHeadBwd };
+template <int MODE>
+__global__ void __launch_bounds__(256) k_head(const bf16 *Y, long long M, int lh, int lw, const float *Wh,
+                                              const float *bh, const float *norm, const float *x, const float *yt,
+                                              const float *dO, float *loss, float *xn, bf16 *dY, float *dWh,
+                                              float *dbh)
 {
-    __shared__ float w[4 * C + 4];
-    __shared__ float red[256];
-    for (int i = threadIdx.x; i < 4 * C; i += blockDim.x) w[i] = Wh[i];
-    if (threadIdx.x < 4) w[4 * C + threadIdx.x] = bh[threadIdx.x];
-    __syncthreads();
-    const float inv = 1.f / (4.f * (float)M);
-    float acc = 0.f;
-    GRID_STRIDE(m, M)
-    {
-        float o[4] = {w[4 * C], w[4 * C + 1], w[4 * C + 2], w[4 * C + 3]};
-        const bf16 *yr = Y + pad_pix(m, lh, lw) * C;
+    __shared__ uint4 sy[256 * 5];
+    __shared__ float w[4 * 32];
+    __shared__ float4 sd[MODE == kHeadNext ? 1 : 256];
+    const int t = threadIdx.x, lane = t & 31, wi = t >> 5;
+    if (t < 128) w[t] = Wh[t];
+    float o0[4] = {0.f, 0.f, 0.f, 0.f}, wl[4];
 #pragma unroll
-        for (int c8 = 0; c8 < C; c8 += 8) {
-            const uint4 v = *reinterpret_cast<const uint4 *>(yr + c8);
-            const bf16 *h = reinterpret_cast<const bf16 *>(&v);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const float yv = __bfloat162float(h[j]);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) o[k] += yv * w[k * C + c8 + j];
-            }
-        }
-        if (mode == 0) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float r = o[k] - (yt[k * M + m] - x[k * M + m]) / norm[8 + k];
-                acc += r * r;
-                dO[m * 4 + k] = 2.f * r * inv;
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) xn[k * M + m] = x[k * M + m] + norm[8 + k] * o[k];
-        }
+    for (int k = 0; k < 4; ++k) {
+        if (MODE != kHeadBwd) o0[k] = bh[k];
+        wl[k] = Wh[k * 32 + lane];
     }
-    if (mode != 0) return;
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
+    const float inv = 1.f / (4.f * (float)M);
+    float acc = 0.f, gw[4] = {0.f, 0.f, 0.f, 0.f}, gb = 0.f;
+    for (long long base = (long long)blockIdx.x * 256; base < M; base += (long long)gridDim.x * 256) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int px = (t >> 2) + 64 * j, ch = t & 3;
+            if (base + px < M)
+                sy[px * 5 + ch] = *reinterpret_cast<const uint4 *>(Y + pad_pix(base + px, lh, lw) * 32 + ch * 8);
+        }
+        const long long m = base + t;
+        float xv[4], yv[4];
+        float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (m < M) {
+            if (MODE == kHeadBwd) {
+                d = *reinterpret_cast<const float4 *>(dO + m * 4);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    xv[k] = x[k * M + m];
+                    if (MODE == kHeadLoss) yv[k] = yt[k * M + m];
+                }
+            }
+        }
+        __syncthreads();
+        if (MODE != kHeadBwd && m < M) {
+            float o[4] = {o0[0], o0[1], o0[2], o0[3]};
+#pragma unroll
+            for (int c8 = 0; c8 < 4; ++c8) {
+                const uint4 v = sy[t * 5 + c8];
+                const bf16 *h = reinterpret_cast<const bf16 *>(&v);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float f = __bfloat162float(h[j]);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) o[k] += f * w[k * 32 + c8 * 8 + j];
+                }
+            }
+            if (MODE == kHeadLoss) {
+                float r[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    r[k] = o[k] - (yv[k] - xv[k]) / norm[8 + k];
+                    acc += r[k] * r[k];
+                }
+                d = make_float4(2.f * r[0] * inv, 2.f * r[1] * inv, 2.f * r[2] * inv, 2.f * r[3] * inv);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) xn[k * M + m] = xv[k] + norm[8 + k] * o[k];
+            }
+        }
+        if (MODE != kHeadNext) {
+            sd[t] = d;
+            __syncwarp();
+#pragma unroll 8
+            for (int k = 0; k < 32; ++k) {
+                const int px = wi * 32 + k;
+                const float4 dk = sd[px];
+                bf16 *yp = reinterpret_cast<bf16 *>(sy + px * 5) + lane;
+                const float f = base + px < M ? __bfloat162float(*yp) : 0.f;
+                *yp = __float2bfloat16_rn(dk.x * wl[0] + dk.y * wl[1] + dk.z * wl[2] + dk.w * wl[3]);
+                gw[0] += dk.x * f;
+                gw[1] += dk.y * f;
+                gw[2] += dk.z * f;
+                gw[3] += dk.w * f;
+                if (lane < 4) gb += lane == 0 ? dk.x : (lane == 1 ? dk.y : (lane == 2 ? dk.z : dk.w));
+            }
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int px = (t >> 2) + 64 * j, ch = t & 3;
+                if (base + px < M)
+                    *reinterpret_cast<uint4 *>(dY + pad_pix(base + px, lh, lw) * 32 + ch * 8) = sy[px * 5 + ch];
+            }
+        }
         __syncthreads();
     }
-    if (threadIdx.x == 0) atomicAdd(loss, red[0] * inv);
+    if (MODE == kHeadNext) return;
+    // Block sums of the loss and of the gradients: red[warp][channel-major gw, gb], loss in sd.
+    float *red = reinterpret_cast<float *>(sy);
+    float *rl = reinterpret_cast<float *>(sd);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) red[wi * 132 + k * 32 + lane] = gw[k];
+    if (lane < 4) red[wi * 132 + 128 + lane] = gb;
+    rl[t] = acc;
+    __syncthreads();
+    if (t < 132) {
+        float s = 0.f;
+        for (int j = 0; j < 8; ++j) s += red[j * 132 + t];
+        if (t < 128) atomicAdd(dWh + t, s);
+        else atomicAdd(dbh + t - 128, s);
+    }
+    if (MODE == kHeadLoss) {
+        for (int s = 128; s > 0; s >>= 1) {
+            if (t < s) rl[t] += rl[t + s];
+            __syncthreads();
+        }
+        if (t == 0) atomicAdd(loss, rl[0] * inv);
+    }
 }
 
-// Head backward (C = 32): dY[m][c] = sum_k dO[m][k] Wh[k][c]; dWh[k][c] += sum_m dO[m][k] Y[m][c];
-// dbh[k] += sum_m dO[m][k].  One warp per pixel at a time, lane = channel.
 // Unrolled training (k windows, each applied to the previous prediction): the loss
 // term of a prediction x'_j against its target y_j, r = (x'_j - y_j) / out_scale, added
 // to the planar field gradient G = dL/dx'_j as 2 r / out_scale * inv (inv = 1 / (4 M k)),
@@ -285,44 +380,6 @@ __global__ void k_conv0_dx(const bf16 *dZ, const bf16 *Wb, int Kp, long long M, 
     }
 }
 
-__global__ void k_head_bwd(const bf16 *Y, long long M, int lh, int lw, const float *Wh, const float *dO, bf16 *dY,
-                           float *dWh, float *dbh)
-{
-    __shared__ float red[8][4 * 32 + 4];
-    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-    float w[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) w[k] = Wh[k * 32 + lane];
-    float gw[4] = {0, 0, 0, 0}, gb = 0.f;
-    for (long long m = (long long)blockIdx.x * 8 + wi; m < M; m += (long long)gridDim.x * 8) {
-        const float4 d = *reinterpret_cast<const float4 *>(dO + m * 4);
-        const long long p = pad_pix(m, lh, lw) * 32 + lane;
-        const float yv = __bfloat162float(Y[p]);
-        dY[p] = __float2bfloat16_rn(d.x * w[0] + d.y * w[1] + d.z * w[2] + d.w * w[3]);
-        gw[0] += d.x * yv;
-        gw[1] += d.y * yv;
-        gw[2] += d.z * yv;
-        gw[3] += d.w * yv;
-        if (lane < 4) gb += lane == 0 ? d.x : (lane == 1 ? d.y : (lane == 2 ? d.z : d.w));
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) red[wi][k * 32 + lane] = gw[k];
-    if (lane < 4) red[wi][128 + lane] = gb;
-    __syncthreads();
-    if (wi == 0) {
-        for (int k = 0; k < 4; ++k) {
-            float s = 0.f;
-            for (int j = 0; j < 8; ++j) s += red[j][k * 32 + lane];
-            atomicAdd(dWh + k * 32 + lane, s);
-        }
-        if (lane < 4) {
-            float s = 0.f;
-            for (int j = 0; j < 8; ++j) s += red[j][128 + lane];
-            atomicAdd(dbh + lane, s);
-        }
-    }
-}
-
 // Adam with bias correction on FP32 masters (c1 = 1 - b1^t, c2 = 1 - b2^t).
 __global__ void k_adam(float *w, const float *gr, float *m, float *v, long long n, float lr, float b1, float b2,
                        float eps, float c1, float c2)
@@ -338,39 +395,42 @@ __global__ void k_adam(float *w, const float *gr, float *m, float *v, long long 
     }
 }
 
-// BF16 operand copies of a 3x3 convolution from its master Wt [Kp][Cout]:
-//   Wb [Cout][Kp]   (forward B operand, K = tap*Cin + ci)
-//   Wf [Cin][Kpo]   (adjoint B operand, K = tap*Cout + co, taken at the mirrored tap 8 - tap)
-__global__ void k_conv_weights(const float *Wt, int Cin, int Cout, int Kp, int Kpo, bf16 *Wb, bf16 *Wf)
+// BF16 operand copies of every layer's weights in one launch (one launch per layer took
+// 17 x ~4.5 us); block b works on a stretch of kWeightChunk elements of one layer.
+//   3x3 convolution, master W [Kp][Cout]:
+//     fwd [Cout][Kp]   (forward B operand, K = tap*Cin + ci)
+//     adj [Cin][Kpo]   (adjoint B operand, K = tap*Cout + co, taken at the mirrored tap 8 - tap)
+//   transposed convolution, master W [4 Cout][Cin]:
+//     fwd [4 Cout][Cin] (forward B operand), adj [Cin][4 Cout] (adjoint B operand).
+constexpr int kWeightChunk = 1024;
+struct WeightTab {
+    WeightCopy L[kMaxWeightCopies];
+    int first[2 * kMaxWeightCopies + 1];      // first block of each layer's fwd and adj copies
+    int n;
+};
+__global__ void __launch_bounds__(256) k_weights(const __grid_constant__ WeightTab tab)
 {
-    GRID_STRIDE(e, (long long)Cout * Kp)
-    {
-        const int co = (int)(e / Kp), k = (int)(e % Kp);
-        Wb[e] = __float2bfloat16_rn(Wt[(long long)k * Cout + co]);
-    }
-    if (!Wf) return;
-    GRID_STRIDE(e, (long long)Cin * Kpo)
-    {
-        const int ci = (int)(e / Kpo), k = (int)(e % Kpo);
+    int j = 0;
+    while (j + 1 < 2 * tab.n && (int)blockIdx.x >= tab.first[j + 1]) ++j;
+    const WeightCopy &w = tab.L[j >> 1];
+    const bool adj = j & 1;
+    const int total = w.up ? 4 * w.cout * w.cin : (adj ? w.cin * w.kpo : w.cout * w.kp);
+    const int e0 = ((int)blockIdx.x - tab.first[j]) * kWeightChunk;
+    for (int e = e0 + threadIdx.x; e < total && e < e0 + kWeightChunk; e += 256) {
         float v = 0.f;
-        if (k < 9 * Cout) {
-            const int tap = k / Cout, co = k % Cout;
-            v = Wt[(long long)((8 - tap) * Cin + ci) * Cout + co];
+        if (w.up) {
+            v = adj ? w.w[(e % (4 * w.cout)) * w.cin + e / (4 * w.cout)] : w.w[e];
+        } else if (!adj) {
+            const int co = e / w.kp, k = e - co * w.kp;
+            v = w.w[k * w.cout + co];
+        } else {
+            const int ci = e / w.kpo, k = e - ci * w.kpo;
+            if (k < 9 * w.cout) {
+                const int tap = k / w.cout, co = k - tap * w.cout;
+                v = w.w[((8 - tap) * w.cin + ci) * w.cout + co];
+            }
         }
-        Wf[e] = __float2bfloat16_rn(v);
-    }
-}
-
-// BF16 copies of a transposed convolution from its master W [4 Cout][Cin]:
-//   Wb [4 Cout][Cin] (forward B operand), Wt [Cin][4 Cout] (adjoint B operand).
-__global__ void k_up_weights(const float *Wm, int Cin, int Cout, bf16 *Wb, bf16 *Wt)
-{
-    GRID_STRIDE(e, 4LL * Cout * Cin)
-    {
-        const int r = (int)(e / Cin), ci = (int)(e % Cin);
-        const bf16 v = __float2bfloat16_rn(Wm[e]);
-        Wb[e] = v;
-        Wt[(long long)ci * 4 * Cout + r] = v;
+        (adj ? w.adj : w.fwd)[e] = __float2bfloat16_rn(v);
     }
 }
 
@@ -449,30 +509,30 @@ cudaError_t shift_rho(float *rho, int batch, long long Mb, const float *delta, c
     return cudaGetLastError();
 }
 
-cudaError_t silu_bwd(const bf16 *dY, int ldd, const bf16 *Z, long long M, int lh, int lw, int C, bf16 *dZ,
-                     float *dbias, cudaStream_t st)
+cudaError_t silu_bwd(const bf16 *dY, int ldd, const bf16 *dP, const bf16 *Z, long long M, int lh, int lw, int C,
+                     bf16 *dZ, float *dbias, cudaStream_t st)
 {
-    if (C % 8 || C / 8 > 32) return cudaErrorInvalidValue;
-    k_silu_bwd<<<grid_red(M * C / 8), 256, 0, st>>>(dY, ldd, Z, M, lh, lw, C, dZ, dbias);
+    const int s = log2i(C >> 3);
+    if (C != 8 << s || C > 256) return cudaErrorInvalidValue;
+    const int g = grid_res(M << s, dP ? 4 : 5);
+    if (dP) k_silu_bwd<true><<<g, 256, 0, st>>>(dY, ldd, dP, Z, M, lh, lw, s, dZ, dbias);
+    else k_silu_bwd<false><<<g, 256, 0, st>>>(dY, ldd, dP, Z, M, lh, lw, s, dZ, dbias);
     return cudaGetLastError();
 }
 
 cudaError_t colsum(const bf16 *X, int ldx, long long M, int lh, int lw, int C, float *out, cudaStream_t st)
 {
-    if (C % 8 || C / 8 > 32 || ldx % 8 || (reinterpret_cast<uintptr_t>(X) & 15)) return cudaErrorInvalidValue;
-    k_colsum<<<grid_red(M * C / 8), 256, 0, st>>>(X, ldx, M, lh, lw, C, out);
+    const int s = log2i(C >> 3);
+    if (C != 8 << s || C > 256 || ldx % 8 || (reinterpret_cast<uintptr_t>(X) & 15)) return cudaErrorInvalidValue;
+    k_colsum<<<grid_res(M << s, 6), 256, 0, st>>>(X, ldx, M, lh, lw, s, out);
     return cudaGetLastError();
 }
 
 cudaError_t pool2(const bf16 *X, int ldx, long long Mc, int lh, int lw, int C, bf16 *Y, cudaStream_t st)
 {
-    k_pool2<<<grid_1d(Mc * C), 256, 0, st>>>(X, ldx, Mc, lh, lw, C, Y);
-    return cudaGetLastError();
-}
-
-cudaError_t unpool2_acc(const bf16 *dY, long long Mc, int lh, int lw, int C, bf16 *dX, int ldx, cudaStream_t st)
-{
-    k_unpool2_acc<<<grid_1d(Mc * C), 256, 0, st>>>(dY, Mc, lh, lw, C, dX, ldx);
+    const int s = log2i(C >> 3);
+    if (C != 8 << s || ldx % 8 || (reinterpret_cast<uintptr_t>(X) & 15)) return cudaErrorInvalidValue;
+    k_pool2<<<grid_1d(Mc << s), 256, 0, st>>>(X, ldx, Mc, lh, lw, s, Y);
     return cudaGetLastError();
 }
 
@@ -482,19 +542,28 @@ cudaError_t pack_in(const float *x, long long M, int lh, int lw, const float *no
     return cudaGetLastError();
 }
 
-cudaError_t head(const bf16 *Y, long long M, int lh, int lw, const float *Wh, const float *bh, const float *norm,
-                 const float *x, const float *yt, int mode, float *dO, float *loss, float *xn, cudaStream_t st)
+cudaError_t head_next(const bf16 *Y, long long M, int lh, int lw, const float *Wh, const float *bh, const float *norm,
+                      const float *x, float *xn, cudaStream_t st)
 {
-    k_head<32><<<grid_1d(M), 256, 0, st>>>(Y, M, lh, lw, Wh, bh, norm, x, yt, mode, dO, loss, xn);
+    k_head<kHeadNext><<<grid_res(M, 5), 256, 0, st>>>(Y, M, lh, lw, Wh, bh, norm, x, nullptr, nullptr, nullptr, xn,
+                                                   nullptr, nullptr, nullptr);
+    return cudaGetLastError();
+}
+
+cudaError_t head_loss_bwd(const bf16 *Y, long long M, int lh, int lw, const float *Wh, const float *bh,
+                          const float *norm, const float *x, const float *yt, float *loss, bf16 *dY, float *dWh,
+                          float *dbh, cudaStream_t st)
+{
+    k_head<kHeadLoss><<<grid_res(M, 3), 256, 0, st>>>(Y, M, lh, lw, Wh, bh, norm, x, yt, nullptr, loss, nullptr, dY, dWh,
+                                                   dbh);
     return cudaGetLastError();
 }
 
 cudaError_t head_bwd(const bf16 *Y, long long M, int lh, int lw, const float *Wh, const float *dO, bf16 *dY,
                      float *dWh, float *dbh, cudaStream_t st)
 {
-    long long g = (M + 8 * 32 - 1) / (8 * 32);
-    if (g > 2048) g = 2048;
-    k_head_bwd<<<(int)(g < 1 ? 1 : g), 256, 0, st>>>(Y, M, lh, lw, Wh, dO, dY, dWh, dbh);
+    k_head<kHeadBwd><<<grid_res(M, 6), 256, 0, st>>>(Y, M, lh, lw, Wh, nullptr, nullptr, nullptr, nullptr, dO, nullptr,
+                                                  nullptr, dY, dWh, dbh);
     return cudaGetLastError();
 }
 
@@ -520,15 +589,22 @@ cudaError_t adam(float *w, const float *g, float *m, float *v, long long n, floa
     return cudaGetLastError();
 }
 
-cudaError_t conv_weights(const float *Wt, int Cin, int Cout, int Kp, int Kpo, bf16 *Wb, bf16 *Wf, cudaStream_t st)
+cudaError_t copy_weights(const WeightCopy *layers, int n, cudaStream_t st)
 {
-    k_conv_weights<<<grid_1d((long long)Cout * Kp), 256, 0, st>>>(Wt, Cin, Cout, Kp, Kpo, Wb, Wf);
-    return cudaGetLastError();
-}
-
-cudaError_t up_weights(const float *Wm, int Cin, int Cout, bf16 *Wb, bf16 *Wt, cudaStream_t st)
-{
-    k_up_weights<<<grid_1d(4LL * Cout * Cin), 256, 0, st>>>(Wm, Cin, Cout, Wb, Wt);
+    if (n < 1 || n > kMaxWeightCopies) return cudaErrorInvalidValue;
+    WeightTab tab;
+    tab.n = n;
+    int blocks = 0;
+    for (int k = 0; k < n; ++k) {
+        const WeightCopy &w = tab.L[k] = layers[k];
+        const int fwd = w.up ? 4 * w.cout * w.cin : w.cout * w.kp, adj = w.up ? fwd : w.cin * w.kpo;
+        tab.first[2 * k] = blocks;
+        blocks += (fwd + kWeightChunk - 1) / kWeightChunk;
+        tab.first[2 * k + 1] = blocks;
+        blocks += (adj + kWeightChunk - 1) / kWeightChunk;
+    }
+    tab.first[2 * n] = blocks;
+    k_weights<<<blocks, 256, 0, st>>>(tab);
     return cudaGetLastError();
 }
 
