@@ -80,7 +80,8 @@ struct Epi {
 };
 
 template <int BN>
-__device__ __forceinline__ void epilogue(const Epi &g, uint32_t tmem, long long m0, int n0, int warp, int lane)
+__device__ __forceinline__ void epilogue(const Epi &g, uint32_t tmem, long long m0, int n0, int warp, int lane,
+                                         int cbeg = 0, int cend = BN)
 {
     const long long row = m0 + warp * 32 + lane;
     const bool rv = row < g.M;
@@ -102,7 +103,7 @@ __device__ __forceinline__ void epilogue(const Epi &g, uint32_t tmem, long long 
         }
     };
 #pragma unroll 1
-    for (int c0 = 0; c0 < BN; c0 += 32) {
+    for (int c0 = cbeg; c0 < cend; c0 += 32) {
         uint32_t r[32];
         const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + c0;
         asm volatile(
@@ -692,6 +693,182 @@ __global__ void __launch_bounds__(192, 1)
     if (warp == 0) tmem_free(tmem, TCOLS);
 }
 
+
+// ---------------------------------------------------------------------------
+// Row-marching 3x3 convolution (images at least 128 pixels wide)
+// ---------------------------------------------------------------------------
+// The TMA mainloop above reads each input pixel from L2 nine times, once per tap: 100 KB per
+// 128 x 32 output tile, which bound the wide-image layers.  Here a CTA owns a column of 128
+// pixels and walks down its image rows: a ring in shared memory holds the halo-wide input
+// rows (130 pixels x C channels, one or more swizzled boxes each), an output row reads the
+// three rows around it, and a tap's A operand is the row's matrix started (dx + 1) pixels
+// further: the swizzle works on shared-memory addresses, so a descriptor may start at any
+// row of the pattern.  Each input row then comes from L2 once per CTA (plus two per column
+// walked), and the weights (all 9 C x N of them) stay in shared memory.  The products are
+// accumulated in the same K order as there.
+template <int C, int N> struct CfgR {
+    static constexpr int CB = C < 64 ? C : 64, NB = C / CB;       // channels per box, boxes per row
+    static constexpr int RB = CB * 2;                             // bytes of a pixel in a box
+    static constexpr int BOX = (130 * RB + 1023) / 1024 * 1024, ROW = NB * BOX;
+    static constexpr int KB = (9 * C + 63) / 64, WBYTES = KB * N * 128;
+    static constexpr int CTAS = N == 32 && C == 32 ? 3 : (N == 64 && C == 64 ? 1 : 2);
+    static constexpr int NR = C == 32 ? (N == 32 ? 5 : 6) : (N == 32 ? 4 : 8);
+    static constexpr int SMEM = WBYTES + NR * ROW + 1024;
+    static constexpr int EW = N == 32 ? 4 : 8;                    // epilogue warps
+    static_assert(CTAS * (SMEM + 2048) <= 232448, "shared memory per SM");
+};
+
+struct RArgs {
+    int c0, b_c0;         // first channel of A, first K column of B
+    int lh, lw;           // image size
+    int tiles;            // output rows x columns of 128 pixels, all images
+    Epi e;
+};
+
+template <int C, int N>
+__global__ void __launch_bounds__(32 * (CfgR<C, N>::EW + 2), CfgR<C, N>::CTAS)
+    k_conv_rows(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const RArgs g)
+{
+    using Cf = CfgR<C, N>;
+    constexpr int NR = Cf::NR, EW = Cf::EW, TCOLS = 2 * N;
+    extern __shared__ unsigned char dsm_raw[];
+    __shared__ __align__(8) uint64_t full[NR], empty[NR], tfull[2], tempty[2], wbar, done_bar;
+    __shared__ uint32_t tmem_sh;
+    __shared__ int abort_flag;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    volatile int *abort_v = &abort_flag;
+    // This CTA's stretch of the tiles, ordered (image, column, row): neighbours in the ring.
+    const int t0 = (int)((long long)g.tiles * blockIdx.x / gridDim.x);
+    const int t1 = (int)((long long)g.tiles * (blockIdx.x + 1) / gridDim.x);
+    const int H = 1 << g.lh;
+
+    if (warp == 0) tmem_alloc(&tmem_sh, TCOLS);
+    if (t == 0) {
+        for (int s = 0; s < NR; ++s) {
+            mbar_init(smem_u32(&full[s]), 1);
+            mbar_init(smem_u32(&empty[s]), 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&tfull[b]), 1);
+            mbar_init(smem_u32(&tempty[b]), 32 * EW);
+        }
+        mbar_init(smem_u32(&wbar), 1);
+        mbar_init(smem_u32(&done_bar), 1);
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tmem = tmem_sh;
+    const uint32_t wbase = (smem_u32(dsm_raw) + 1023u) & ~1023u, rbase = wbase + Cf::WBYTES;
+
+    if (warp == EW) {
+        if (lane == 0) {
+            // ---------------- TMA producer: the weights, then the input rows ----------------
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&wbar)),
+                         "r"((uint32_t)Cf::WBYTES));
+            for (int kb = 0; kb < Cf::KB; ++kb)
+                tma_load_2d(wbase + (uint32_t)(kb * N * 128), &tmB, g.b_c0 + kb * 64, 0, smem_u32(&wbar));
+            int r = 0;                                            // rows loaded so far
+            bool ok = true;
+            for (int i = t0; i < t1 && ok; ++i) {
+                const int y = i & (H - 1), col = i >> g.lh;
+                const int b = col >> (g.lw - 7), x0 = (col & ((1 << (g.lw - 7)) - 1)) << 7;
+                // Stored rows y .. y + 2 hold the interior rows y - 1 .. y + 1.
+                for (int yy = (i == t0 || y == 0) ? y : y + 2; yy <= y + 2 && ok; ++yy, ++r) {
+                    const int s = r % NR;
+                    if (r >= NR && !mbar_wait(smem_u32(&empty[s]), (uint32_t)((r / NR - 1) & 1), abort_v)) {
+                        *abort_v = 1;
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&full[s])),
+                                 "r"((uint32_t)(Cf::NB * 130 * Cf::RB)));
+#pragma unroll
+                    for (int j = 0; j < Cf::NB; ++j)
+                        tma_load_4d(rbase + (uint32_t)(s * Cf::ROW + j * Cf::BOX), &tmA, g.c0 + j * Cf::CB, x0, yy, b,
+                                    smem_u32(&full[s]));
+                }
+            }
+            // No copy may be in flight when the CTA ends (after a wait gave up, rows that no
+            // MMA waited for).
+            mbar_wait(smem_u32(&wbar), 0);
+            for (int k = r > NR ? r - NR : 0; k < r; ++k) mbar_wait(smem_u32(&full[k % NR]), (uint32_t)((k / NR) & 1));
+        }
+    } else if (warp == EW + 1) {
+        if (lane == 0) {
+            // ---------------- MMA issuer ----------------
+            const uint32_t idesc = make_idesc(N, false, false);
+            bool ok = t1 <= t0 || mbar_wait(smem_u32(&wbar), 0, abort_v);
+            if (!ok) *abort_v = 1;
+            int top = 0, have = 0, lt = 0;                        // ring index of row y - 1, rows waited for
+            for (int i = t0; i < t1 && ok; ++i, ++lt) {
+                const int y = i & (H - 1), buf = lt & 1;
+                if (lt >= 2 && !mbar_wait(smem_u32(&tempty[buf]), (uint32_t)(((lt >> 1) - 1) & 1), abort_v)) {
+                    *abort_v = 1;
+                    break;
+                }
+                for (; have < top + 3 && ok; ++have)
+                    if (!mbar_wait(smem_u32(&full[have % NR]), (uint32_t)((have / NR) & 1), abort_v)) {
+                        *abort_v = 1;
+                        ok = false;
+                    }
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t acc_t = tmem + (uint32_t)(buf * N);
+#pragma unroll 1
+                for (int dy = 0; dy < 3; ++dy) {
+                    const uint32_t ra = rbase + (uint32_t)((top + dy) % NR * Cf::ROW);
+#pragma unroll
+                    for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                        for (int c = 0; c < C; c += 16) {
+                            const int k = (dy * 3 + dx) * C + c;
+                            const uint64_t da = smem_desc(ra + (uint32_t)(c / Cf::CB * Cf::BOX + dx * Cf::RB + c % Cf::CB * 2),
+                                                          16, Cf::RB * 8, Cf::RB == 128 ? 2 : 4);
+                            const uint64_t db = smem_desc(wbase + (uint32_t)((k >> 6) * N * 128 + (k & 63) * 2), 16, 1024, 2);
+                            mma_bf16(acc_t, da, db, idesc, k > 0 ? 1u : 0u);
+                        }
+                }
+                // The next output row of this column still reads rows y and y + 1.
+                const int next = i + 1 < t1 && y != H - 1 ? 1 : 3;
+                for (int k = 0; k < next; ++k) mma_commit(smem_u32(&empty[(top + k) % NR]));
+                top += next;
+                mma_commit(smem_u32(&tfull[buf]));
+            }
+            mma_commit(smem_u32(&done_bar));   // arrives once every MMA above completed
+        }
+    } else {
+        // ---------------- epilogue (EW warps: lane quarter warp % 4, column half warp / 4) ----------------
+        const int half = warp >> 2, cw = N * 4 / EW;
+        int lt = 0;
+        for (int i = t0; i < t1; ++i, ++lt) {
+            const int buf = lt & 1;
+            const bool ready = mbar_wait(smem_u32(&tfull[buf]), (uint32_t)((lt >> 1) & 1), abort_v);
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            if (!__all_sync(0xffffffffu, ready && !*abort_v)) {
+                *abort_v = 1;
+                break;
+            }
+            const int y = i & (H - 1), col = i >> g.lh;
+            const int b = col >> (g.lw - 7), x0 = (col & ((1 << (g.lw - 7)) - 1)) << 7;
+            const long long m0 = ((((long long)b << g.lh) + y) << g.lw) + x0;
+            epilogue<N>(g.e, tmem + (uint32_t)(buf * N), m0, 0, warp & 3, lane, half * cw, (half + 1) * cw);
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[buf])));
+        }
+        // Tensor memory must be idle before it is freed.
+        if (!mbar_wait(smem_u32(&done_bar), 0)) *abort_v = 1;
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    if (t == 0 && *abort_v) atomicExch(g.e.status, 1);
+    if (warp == 0) tmem_free(tmem, TCOLS);
+}
+
 }  // namespace
 
 }  // namespace evsur
@@ -936,6 +1113,61 @@ bool tma_eligible(const sur_gemm_args &a)
     return hw > 0 && a.a.rows % hw == 0;
 }
 
+// Row-marching convolution: eligible shapes (of those tma_eligible accepts) are whole 3x3
+// convolutions over images at least 128 pixels wide with the channel counts instantiated here.
+bool rows_eligible(const sur_gemm_args &a)
+{
+    if (a.a.kind != SUR_OP_CONV3 || a.a.W < 128 || a.K != (9 * a.a.C + 63) / 64 * 64 || a.M != a.a.rows) return false;
+    return (a.a.C == 32 || a.a.C == 64) && (a.N == 32 || a.N == 64);
+}
+
+template <int C, int N>
+int launch_rows(const sur_gemm_args &a, const Epi &e, cudaStream_t st)
+{
+    using Cf = CfgR<C, N>;
+    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+    if (!enc) return -1;
+    const int H = a.a.H, W = a.a.W;
+    const size_t e2 = 2;
+    CUtensorMap ma, mb;
+    cuuint64_t dims[4] = {(cuuint64_t)a.a.ld, (cuuint64_t)(W + 2), (cuuint64_t)(H + 2),
+                          (cuuint64_t)(a.a.rows / ((long long)H * W))};
+    cuuint64_t strides[3] = {a.a.ld * e2, (cuuint64_t)(W + 2) * a.a.ld * e2,
+                             (cuuint64_t)(H + 2) * (W + 2) * a.a.ld * e2};
+    cuuint32_t box[4] = {(cuuint32_t)Cf::CB, 130, 1, 1}, es[4] = {1, 1, 1, 1};
+    if (enc(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(a.a.p), dims, strides, box, es,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, Cf::CB == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return -1;
+    cuuint64_t bdims[2] = {(cuuint64_t)a.b.ld, (cuuint64_t)a.b.rows}, bstr[1] = {a.b.ld * e2};
+    cuuint32_t bbox[2] = {64, (cuuint32_t)N}, bes[2] = {1, 1};
+    if (enc(&mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(a.b.p), bdims, bstr, bbox, bes,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return -1;
+    static int attr_dev = -1, sms = 0;
+    cudaError_t err = set_smem(k_conv_rows<C, N>, Cf::SMEM, attr_dev);
+    if (err != cudaSuccess) return SUR_ECUDA;
+    if (!sms) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return SUR_ECUDA;
+    }
+    RArgs g;
+    g.c0 = a.a.c0;
+    g.b_c0 = a.b.c0;
+    g.lh = ilog2(H);
+    g.lw = ilog2(W);
+    g.tiles = a.M / 128;
+    g.e = e;
+    // At least 8 rows a CTA, so that the two rows it loads beyond its own stay a small part.
+    int ctas = Cf::CTAS * sms;
+    if (g.tiles / 8 < ctas) ctas = g.tiles / 8 > 0 ? g.tiles / 8 : 1;
+    k_conv_rows<C, N><<<ctas, 32 * (Cf::EW + 2), Cf::SMEM, st>>>(ma, mb, g);
+    return cudaGetLastError() == cudaSuccess ? SUR_OK : SUR_ECUDA;
+}
+
 }  // namespace
 
 void set_tma(bool on) { g_tma_enabled = on; }
@@ -1003,6 +1235,11 @@ int gemm(const sur_gemm_args &a, int *status, cudaStream_t st)
             else err = launch_tma<32, 16, true>(ma, mb, tg, mtiles, st);
             return err == cudaSuccess ? SUR_OK : SUR_ECUDA;
         }
+    }
+    if (tma_eligible(a) && rows_eligible(a)) {
+        const int rc = a.a.C == 32 ? (a.N == 32 ? launch_rows<32, 32>(a, e, st) : launch_rows<32, 64>(a, e, st))
+                                   : (a.N == 32 ? launch_rows<64, 32>(a, e, st) : launch_rows<64, 64>(a, e, st));
+        if (rc >= 0) return rc;                // -1: a tensor map was refused
     }
     if (tma_eligible(a)) {
         CUtensorMap ma, mb;
