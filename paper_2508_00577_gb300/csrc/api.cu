@@ -107,14 +107,38 @@ void fill_kparams(lbm_ctx *c)
 
 bool dev16(const lbm_ctx *c) { return c->P.precision == LBM_FP16_DEV || c->P.precision == LBM_BF16_DEV; }
 
+// Macroscopic fields by the fused kernels where a fused step applies: one launch, the fields
+// straight to `o`.  False where it does not (FP64, literal force form, D3Q27 walls).
+bool fused_moments(lbm_ctx *c, const evlbm::MomentOut &o, cudaError_t *e)
+{
+    if (fp64(c)) return false;
+    const void *f = c->f[c->cur], *g = c->g[c->cur], *R = c->R[c->cur];
+    if (evlbm::fused2d_supported(c->P.precision, c->Q, c->K)) {
+        *e = evlbm::fused2d_moments(c->P.precision, c->K, f, g, c->RT_iso, R, o, c->stream);
+        return true;
+    }
+    if (evlbm::fused3d_supported(c->P.precision, c->Q, c->K)) {
+        *e = evlbm::fused3d_moments(c->P.precision, c->K, f, g, c->RT_iso, R, o, c->stream);
+        return true;
+    }
+    return false;
+}
+
 int run_macro(lbm_ctx *c)
 {
     int rc = ensure_scratch(c);
     if (rc) return rc;
-    cudaError_t e = fp64(c) ? evlbm::ref_macro_f64(c->Q, c->K, c->scratch, c->RT_iso, c->f[c->cur], c->g[c->cur],
-                                                  c->stream)
-                            : evlbm::ref_macro_f32(c->P.precision, c->Q, c->K, c->scratch, c->RT_iso,
-                                                   c->f[c->cur], c->g[c->cur], c->R[c->cur], c->stream);
+    cudaError_t e = cudaSuccess;
+    if (!fp64(c)) {
+        // R T, as the scratch field holds it (the caller divides by R on the host).
+        using O = evlbm::FieldOffsets;
+        float *s = static_cast<float *>(c->scratch);
+        if (fused_moments(c, {s + O::rho * c->N, s + O::u * c->N, s + O::RT * c->N, s + O::F * c->N, 1.0}, &e))
+            return e == cudaSuccess ? LBM_OK : cuda_fail(c, e, "moments");
+    }
+    e = fp64(c) ? evlbm::ref_macro_f64(c->Q, c->K, c->scratch, c->RT_iso, c->f[c->cur], c->g[c->cur], c->stream)
+                : evlbm::ref_macro_f32(c->P.precision, c->Q, c->K, c->scratch, c->RT_iso, c->f[c->cur], c->g[c->cur],
+                                       c->R[c->cur], c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "moment stages");
     return LBM_OK;
 }
@@ -350,10 +374,13 @@ int lbm_reset_device(lbm_ctx *c, const float *d_rho, const float *d_u, const flo
 int lbm_moments_device(lbm_ctx *c, float *d_rho, float *d_u, float *d_T)
 {
     if (!c) return LBM_EINVAL;
+    cudaError_t e = cudaSuccess;
+    if (fused_moments(c, {d_rho, d_u, d_T, nullptr, c->P.R}, &e))
+        return e == cudaSuccess ? LBM_OK : cuda_fail(c, e, "lbm_moments_device");
     int rc = run_macro(c);
     if (rc) return rc;
-    cudaError_t e = fp64(c) ? evlbm::ref_export_f64(c->Q, c->K, c->scratch, c->P.R, d_rho, d_u, d_T, c->stream)
-                            : evlbm::ref_export_f32(c->Q, c->K, c->scratch, c->P.R, d_rho, d_u, d_T, c->stream);
+    e = fp64(c) ? evlbm::ref_export_f64(c->Q, c->K, c->scratch, c->P.R, d_rho, d_u, d_T, c->stream)
+                : evlbm::ref_export_f32(c->Q, c->K, c->scratch, c->P.R, d_rho, d_u, d_T, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "lbm_moments_device");
     return LBM_OK;
 }

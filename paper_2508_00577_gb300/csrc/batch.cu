@@ -226,7 +226,9 @@ struct lbm_batch {
     int graph_steps, graph_cur, graph_w, graph_h;
     bool graph_probe;
     long long graph_limit;
-    void *scratch;               // stage-kernel fields for lbm_batch_moments (largest domain)
+    void *scratch;               // device fields of lbm_batch_moments, 4 of the largest domain
+    float *host;                 // their pinned host copy, allocated on first use (NULL: pageable)
+    bool host_tried;
     long long max_nodes;
     long long steps;
     KParams K;                   // common physics (per-domain sizes filled on use)
@@ -375,6 +377,7 @@ void free_batch(lbm_batch *b)
     if (b->d_error) cudaFree(b->d_error);
     if (b->d_probe) cudaFree(b->d_probe);
     if (b->scratch) cudaFree(b->scratch);
+    if (b->host) cudaFreeHost(b->host);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
     b->stream = nullptr;
 }
@@ -485,7 +488,7 @@ int lbm_batch_init(const lbm_params *p, int n_domains, const int *nx, const int 
     if (e == cudaSuccess) e = cudaMalloc(&b->d_error, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_probe, sizeof(int));
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_probe, 0, sizeof(int), b->stream);
-    if (e == cudaSuccess) e = cudaMalloc(&b->scratch, sizeof(float) * evlbm::kRefFieldCount * max_nodes);
+    if (e == cudaSuccess) e = cudaMalloc(&b->scratch, sizeof(float) * 4 * max_nodes);
     float *d_fields = nullptr;
     if (e == cudaSuccess) e = cudaMalloc(&d_fields, sizeof(float) * 4 * max_nodes);
     if (e != cudaSuccess) {
@@ -669,24 +672,30 @@ int lbm_batch_moments(lbm_batch *b, int domain, double *rho, double *u, double *
     const KParams K = domain_kparams(b, domain);
     const BatchDomain &D = b->dom[domain];
     const long long Nd = K.N;
-    cudaError_t e = evlbm::ref_macro_f32(1, 9, K, b->scratch, b->RT_iso + D.foff, b->f[b->cur] + D.off,
-                                         b->P.thermal ? b->g[b->cur] + D.off : nullptr, nullptr, b->stream);
+    // One launch writes the four planar fields, one copy brings them to the host (through
+    // pinned memory of at most 16 bytes per node of the largest domain, kept by the batch).
+    float *d = static_cast<float *>(b->scratch);
+    cudaError_t e = evlbm::fused2d_moments(1, K, b->f[b->cur] + D.off, b->P.thermal ? b->g[b->cur] + D.off : nullptr,
+                                           b->RT_iso + D.foff, nullptr, {d, d + Nd, d + 3 * Nd, nullptr, 1.0}, b->stream);
     if (e != cudaSuccess) return bfail(b, LBM_ECUDA, "lbm_batch_moments: %s", cudaGetErrorString(e));
-    std::vector<float> h(4 * Nd);
-    using O = evlbm::FieldOffsets;
-    const float *s = static_cast<const float *>(b->scratch);
-    BCK(b, cudaMemcpyAsync(h.data(), s + O::rho * Nd, sizeof(float) * Nd, cudaMemcpyDeviceToHost, b->stream));
-    BCK(b, cudaMemcpyAsync(h.data() + Nd, s + O::u * Nd, sizeof(float) * 2 * Nd, cudaMemcpyDeviceToHost, b->stream));
-    BCK(b, cudaMemcpyAsync(h.data() + 3 * Nd, s + O::RT * Nd, sizeof(float) * Nd, cudaMemcpyDeviceToHost, b->stream));
-    BCK(b, cudaStreamSynchronize(b->stream));
-    for (long long k = 0; k < Nd; ++k) {
-        if (rho) rho[k] = h[k];
-        if (u) {
-            u[k] = h[Nd + k];
-            u[Nd + k] = h[2 * Nd + k];
+    if (!b->host_tried) {
+        b->host_tried = true;
+        if (cudaMallocHost(&b->host, sizeof(float) * 4 * b->max_nodes) != cudaSuccess) {
+            cudaGetLastError();
+            b->host = nullptr;
         }
-        if (T) T[k] = double(h[3 * Nd + k]) / b->P.R;
     }
+    std::vector<float> pageable;
+    if (!b->host) pageable.resize(4 * Nd);
+    float *h = b->host ? b->host : pageable.data();
+    BCK(b, cudaMemcpyAsync(h, d, sizeof(float) * 4 * Nd, cudaMemcpyDeviceToHost, b->stream));
+    BCK(b, cudaStreamSynchronize(b->stream));
+    if (rho)
+        for (long long k = 0; k < Nd; ++k) rho[k] = h[k];
+    if (u)
+        for (long long k = 0; k < 2 * Nd; ++k) u[k] = h[Nd + k];
+    if (T)
+        for (long long k = 0; k < Nd; ++k) T[k] = double(h[3 * Nd + k]) / b->P.R;
     return LBM_OK;
 }
 

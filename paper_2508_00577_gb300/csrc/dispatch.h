@@ -40,6 +40,21 @@ struct FieldOffsets {
                                theta0 = 23, P0 = 24, gamma0 = 25, flux = 26, wq = 29, m_in = 30;
 };
 
+// Device outputs of the fused moments kernels (any may be NULL): rho [N], u [D][N], T [N] =
+// R T / R (R = 1: R T itself), F [D][N].
+struct MomentOut {
+    float *rho, *u, *T, *F;
+    double R;
+};
+// Macroscopic fields of the current state on lattices a fused step supports, as that step's
+// own stages compute them.
+cudaError_t fused2d_moments(int prec, const KParams &p, const void *f, const void *g, const void *RT_iso,
+                            const void *Rin, const MomentOut &o, cudaStream_t st);
+cudaError_t fused2d_moments16(int prec, const KParams &p, const void *f, const void *g, const void *RT_iso,
+                              const void *Rin, const MomentOut &o, cudaStream_t st);
+cudaError_t fused3d_moments(int prec, const KParams &p, const void *f, const void *g, const void *RT_iso,
+                            const void *Rin, const MomentOut &o, cudaStream_t st);
+
 // Fused single-pass D2Q9 step (FP32 arithmetic); prec 1/2/3 as above.  The
 // launch shape is a strip of tile_w columns marching over chunks of tile_h rows
 // (KParams::tile_w/tile_h; 0 = default).

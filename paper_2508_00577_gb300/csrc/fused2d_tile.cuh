@@ -83,6 +83,11 @@ template <int W> constexpr size_t smem_of()
     return sizeof(v2) * (size_t)(kFields * kDepth * slots_of<W>() + (4 * 9 + 2 * 9 + kCentre) * W);
 }
 
+// The macroscopic fields alone (fused_tile with MOM) need the density, momentum and stress
+// rings.
+constexpr int kMomentFields = 6;
+template <int W> constexpr size_t moments_smem_of() { return sizeof(v2) * (size_t)(kMomentFields * kDepth * slots_of<W>()); }
+
 struct FusedArgs {
     const float *f, *g;          // FP32 populations, or the raw 16-bit deviations (16-bit storage)
     float *fo, *go;
@@ -95,7 +100,19 @@ struct FusedArgs {
     float a, b, kappa, lambda, c_eq, c_star;
     int walls;                   // 1: the columns x = 0 and x = nx-1 are wall nodes (KParams::walls)
     float wall_uy[2], wall_RT;   // wall velocities (along y) and R T_w
+    // MOM: outputs rho [N], u [2][N], T [N], F [2][N] (any may be NULL); T = R T / R with
+    // R = Rh + Rl and Ri = 1 / R.
+    float *m_rho, *m_u, *m_T, *m_F;
+    float Rh, Rl, Ri;
+    int z0;                      // MOM: first layer of the launch
 };
+
+// RT / R to within a rounding (R = Rh + Rl, Ri ~ 1 / R); exact for R = 1.
+__device__ __forceinline__ float over_R(float RT, float Rh, float Rl, float Ri)
+{
+    const float q = RT * Ri;
+    return fmaf(fmaf(-q, Rl, fmaf(-q, Rh, RT)), Ri, q);
+}
 
 __device__ __forceinline__ int wrap_any(int v, int n)
 {
@@ -175,8 +192,10 @@ __device__ __forceinline__ v2 sum9(const v2 h[9])
 // bz.  smem holds smem_of<kW>() bytes.  CG selects loads that may see populations
 // written by other CTAs of the same launch.  A CTA that runs several tiles must pass a
 // barrier between them (the rings are reused).  WALLS compiles in the wall columns
-// (FusedArgs::walls); without it the kernel has no trace of them.
-template <int kW, bool THERMAL, bool CG, bool WALLS = false, typename ST = float>
+// (FusedArgs::walls); without it the kernel has no trace of them.  MOM stops after stage C
+// and writes the macroscopic fields there: A then runs on 2 halo columns and row pairs, B on
+// 1, C on the strip itself, and smem holds moments_smem_of<kW>() bytes.
+template <int kW, bool THERMAL, bool CG, bool WALLS = false, typename ST = float, bool MOM = false>
 __device__ __forceinline__ void fused_tile(const FusedArgs &A, int bx, int y0, int rows, int bz, v2 *smem)
 {
     // 16-bit deviation storage (ST = __half / __nv_bfloat16): pulls decode, stage D encodes
@@ -210,13 +229,15 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &A, int bx, int y0, i
         if (h < 3) {
             slot = h;
             col = x0 - 3 + h;
-            inB = h >= 1;
-            inC = h == 2;
+            inA = !MOM || h >= 1;
+            inB = h >= (MOM ? 2 : 1);
+            inC = !MOM && h == 2;
         } else if (h < 6) {
             slot = Weff + h;
             col = x0 + Weff + (h - 3);
-            inB = h <= 4;
-            inC = h == 3;
+            inA = !MOM || h <= 4;
+            inB = h <= (MOM ? 3 : 4);
+            inC = !MOM && h == 3;
         } else {
             inA = inB = inC = false;
         }
@@ -256,10 +277,10 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &A, int bx, int y0, i
     // Pair indices: pair q holds rows 2q, 2q+1 (absolute, unwrapped).
     const int q0 = y0 / 2;
     const int qD_end = (y0 + Heff + 1) / 2;              // one past the last collided pair
-    const int qbeg = q0 - 3, qend = qD_end + 2;
+    const int qbeg = q0 - (MOM ? 2 : 3), qend = qD_end + (MOM ? 1 : 2);
     int rA = wrap_any(2 * qbeg, ny);                      // wrapped first row of the next A pair
-    int rC = wrap_any(2 * (q0 - 1), ny);                  // ... of the next C pair
-    int rD = wrap_any(2 * q0, ny);                        // ... of the next D pair
+    int rC = wrap_any(2 * (q0 - (MOM ? 0 : 1)), ny);      // ... of the next C pair
+    int rD = wrap_any(2 * q0, ny);                        // ... of the next D (MOM: output) pair
     int s0 = ((qbeg % 3) + 3) % 3;                        // ring slot of pair q
 
     v2 pf[9], pg[9];
@@ -282,7 +303,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &A, int bx, int y0, i
             fld(RHO, s0)[slot] = sum9(pf);
             fld(JX, s0)[slot] = ((pf[2] + pf[5]) + pf[8]) - ((pf[0] + pf[3]) + pf[6]);
             fld(JY, s0)[slot] = ((pf[6] + pf[7]) + pf[8]) - ((pf[0] + pf[1]) + pf[2]);
-            if (inD) {
+            if (!MOM && inD) {
                 v2 *fr = f9 + (q & 3) * 9 * kW + t;
                 if (WALLS && wallc) {
                     // A wall column keeps, for stage D, the mass streaming into it: the three
@@ -315,7 +336,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &A, int bx, int y0, i
         __syncthreads();
 
         // ---------------- B: Korteweg stress of pair q-1 ----------------
-        if (inB && q - 1 >= q0 - 2) {
+        if (inB && q - 1 >= q0 - (MOM ? 1 : 2)) {
             const v2 *r2 = fld(RHO, sm2), *r1 = fld(RHO, sm1), *r0 = fld(RHO, s0);
             const v2 aW = r2[slot - 1], aC = r2[slot], aE = r2[slot + 1];     // pair q-2
             const v2 bW = r1[slot - 1], bC = r1[slot], bE = r1[slot + 1];     // pair q-1 (centre rows)
@@ -338,7 +359,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &A, int bx, int y0, i
 
         // ---------------- C: force, velocity, temperature, EOS of pair q-2 ----------------
         v2 cprev[kCentre];                                 // centre values of pair q-3 (stage D)
-        if (inC && q - 2 >= q0 - 1) {
+        if (inC && q - 2 >= q0 - (MOM ? 0 : 1)) {
             // Pi of pairs q-3 (slot s0), q-2 (sm2, centre rows), q-1 (sm1).
             const int sw = slot - 1, se = slot + 1;
             const v2 *x3 = fld(PXX, s0), *x2 = fld(PXX, sm2), *x1 = fld(PXX, sm1);
@@ -367,7 +388,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &A, int bx, int y0, i
                 const v2 Gam = sum9(pg);
                 const v2 E = fma2(V(0.5f), fma2(ux, Fx, uy * Fy), Gam) * ir;
                 RT = V(2.f / 3.f) * fma2(V(-0.5f), fma2(ux, ux, uy * uy), E);
-                if (inD) {
+                if (!MOM && inD) {
                     v2 *gr = g9 + (q & 1) * 9 * kW + t;
 #pragma unroll
                     for (int i = 0; i < 9; ++i) gr[i * kW] = pg[i];
@@ -384,6 +405,23 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &A, int bx, int y0, i
                 RT = V(in_bounds(T0 - A.RT_iso, N) ? ldpop<CG>(T0) : 0.f, in_bounds(T1 - A.RT_iso, N) ? ldpop<CG>(T1) : 0.f);
                 rC = next_row(next_row(rC, ny), ny);
             }
+            if constexpr (MOM) {
+                const unsigned o0 = layer + (unsigned)rD * nx + cols[1];
+                const unsigned o1 = layer + (unsigned)next_row(rD, ny) * nx + cols[1];
+                rD = next_row(next_row(rD, ny), ny);
+                const bool second = 2 * (q - 2) + 1 < y0 + Heff;
+                auto put = [&](float *dst, v2 v) {
+                    if (!dst) return;
+                    if (in_bounds(o0, N)) dst[o0] = v.x;
+                    if (second && in_bounds(o1, N)) dst[o1] = v.y;
+                };
+                put(A.m_rho, rho);
+                put(A.m_u, ux);
+                put(A.m_u ? A.m_u + N : nullptr, uy);
+                put(A.m_T, V(over_R(RT.x, A.Rh, A.Rl, A.Ri), over_R(RT.y, A.Rh, A.Rl, A.Ri)));
+                put(A.m_F, Fx);
+                put(A.m_F ? A.m_F + N : nullptr, Fy);
+            } else {
             // EOS in the Enskog gauge: P0 = P_E = rho RT Z, gamma0 = 1 + rho Z'/Z [+ 2/3 Z].
             v2 Z, dlnZ;
             if (A.eos == 0) {
@@ -414,11 +452,14 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &A, int bx, int y0, i
                 cr[0 * kW] = rho; cr[1 * kW] = Fx; cr[2 * kW] = Fy;
                 cr[3 * kW] = RT; cr[4 * kW] = th; cr[5 * kW] = g0;
             }
+            }
         }
         __syncthreads();
 
         // ---------------- D: collide pair q-3 ----------------
-        if (inD && q - 3 >= q0 && wallc) {
+        if (MOM) {
+            // no collision
+        } else if (inD && q - 3 >= q0 && wallc) {
             // Wall nodes (diffuse reflection): the equilibria at the wall velocity (0, U_w) and
             // temperature R T_w (Eqs. feq, geq) with the density rho_w that returns the mass m
             // that streamed in, P_E(rho_w, R T_w) = 2 m.

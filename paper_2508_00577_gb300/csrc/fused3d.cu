@@ -799,6 +799,183 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
     if (t < 32) tmem::dealloc(tm_base_sh, TM_COLS);
 }
 
+// Macroscopic fields of the current state (lbm_moments): stages A to C of the step alone, so
+// the density is needed within two columns of the tile, the stress within one, and momentum
+// and partial forces stay in registers; 13 KB of shared memory.  One pass over the
+// populations (216 + 20 bytes per node, FP32 storage) in place of four stage kernels through
+// ~20 scratch fields per node: at 256^3 those took 2904 us (moments 832, stress 332, macro
+// 1434, export 305), with BF16 storage 9745 us.
+struct MGeo {
+    static constexpr int TX = 32, TY = 8, NT = TX * TY, WA = TX + 4, WB = TX + 2;
+    static constexpr int SA = WA * (TY + 4), SB = WB * (TY + 2);
+    static_assert(SA - NT <= NT && SB <= 2 * NT, "two column passes");
+};
+struct MArgs {
+    float *rho, *u, *T, *F;                       // outputs, any may be NULL
+    float Rh, Rl, Ri;                             // R = Rh + Rl, Ri ~ 1 / R
+};
+
+template <bool THERMAL, typename S>
+__global__ void __launch_bounds__(MGeo::NT, 3) k_moments3d(const Args<S> A, const MArgs M)
+{
+    constexpr bool DEV = Store<S>::dev;
+    constexpr int TX = MGeo::TX, TY = MGeo::TY, NT = MGeo::NT, WA = MGeo::WA, WB = MGeo::WB, SA = MGeo::SA, SB = MGeo::SB;
+    __shared__ float RHO[3 * SA], PI[6 * SB];
+    const int t = threadIdx.x, nx = A.nx, ny = A.ny, nz = A.nz;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    const int z0 = (int)blockIdx.z * A.HZ, zend = min(z0 + A.HZ, nz);
+    const unsigned N = A.N;
+    const float a = A.a, kappa = A.kappa;
+    auto sa = [](int cx, int cy) { return (cy + 2) * WA + (cx + 2); };
+    const int dcx = t % TX, dcy = t / TX;
+    const bool out_of = x0 + dcx >= nx || y0 + dcy >= ny;
+    const Cell cD = cell_of(x0 + dcx, y0 + dcy, nx, ny);
+    // The thread's second column of stage A: two rows above and below the tile, then two
+    // columns left and right of each tile row.
+    int hx, hy;
+    if (t < 2 * WA) { hx = t % WA - 2; hy = t / WA - 2; }
+    else if (t < 4 * WA) { hx = (t - 2 * WA) % WA - 2; hy = TY + (t - 2 * WA) / WA; }
+    else { const int m = (t - 4 * WA) & 3; hy = (t - 4 * WA) >> 2; hx = m < 2 ? m - 2 : TX + m - 2; }
+    float j0[3] = {0.f, 0.f, 0.f}, j1[3] = {0.f, 0.f, 0.f}, j2[3];    // momentum of planes q, q-1, q-2
+    float p1[3] = {0.f, 0.f, 0.f}, p2[3] = {0.f, 0.f, 0.f};            // partial forces of planes q-1, q-2
+
+    for (int q = z0 - 2; q <= zend + 1; ++q) {
+        const int s0 = ((q % 3) + 3) % 3, sm1 = s0 == 0 ? 2 : s0 - 1, sm2 = s0 == 2 ? 0 : s0 + 1;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            j2[m] = j1[m];
+            j1[m] = j0[m];
+        }
+        // A: rho (tile + 2) and j (tile) of plane q
+        unsigned zo[3];
+        plane_offsets(q, nx, ny, nz, zo);
+#pragma unroll 1
+        for (int k = 0; k < 2; ++k) {
+            if (k == 1 && t >= SA - NT) break;
+            const int cx = k ? hx : dcx, cy = k ? hy : dcy;
+            const Cell c = k ? cell_of(x0 + cx, y0 + cy, nx, ny) : cD;
+            float rho = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
+#pragma unroll
+            for (int i = 0; i < 27; ++i) {
+                const unsigned si = src_of(i, c, zo, N);
+                float h = ldc(A.f, si, 27ull * N);
+                if constexpr (DEV) h = decode_f<27>(cxi(i), cyi(i), czi(i), ldrec(A.Rin, si - i * N, N), h);
+                rho += h;
+                if (cxi(i) == 1) jx += h; else if (cxi(i) == -1) jx -= h;
+                if (cyi(i) == 1) jy += h; else if (cyi(i) == -1) jy -= h;
+                if (czi(i) == 1) jz += h; else if (czi(i) == -1) jz -= h;
+            }
+            if (k == 0) {
+                j0[0] = jx;
+                j0[1] = jy;
+                j0[2] = jz;
+            }
+            if (in_bounds(sa(cx, cy), SA)) RHO[s0 * SA + sa(cx, cy)] = rho;
+        }
+        __syncthreads();
+        if (q < z0) continue;                                     // block-uniform
+        // B: Korteweg stress of plane q-1 (tile + 1)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int cb = t + k * NT;
+            if (cb >= SB) continue;
+            const float *r[3] = {RHO + sm2 * SA, RHO + sm1 * SA, RHO + s0 * SA};
+            const int c0 = sa(cb % WB - 1, cb / WB - 1);
+            if (!(in_bounds(c0 - WA - 1, SA) && in_bounds(c0 + WA + 1, SA))) continue;
+            const float rc = r[1][c0];
+            float gx = 0.f, gy = 0.f, gz = 0.f, lap = 0.f;
+#pragma unroll
+            for (int i = 0; i < 27; ++i) {
+                if (i == 13) continue;
+                const float v = r[1 + czi(i)][c0 + cyi(i) * WA + cxi(i)];
+                const float w = wi(i);
+                if (cxi(i)) gx += (cxi(i) * w) * v;
+                if (cyi(i)) gy += (cyi(i) * w) * v;
+                if (czi(i)) gz += (czi(i) * w) * v;
+                lap += w * (v - rc);
+            }
+            gx *= 3.f; gy *= 3.f; gz *= 3.f; lap *= 6.f;
+            const float s = -a * rc * rc - kappa * rc * lap - 0.5f * kappa * (gx * gx + gy * gy + gz * gz);
+            float *pr = PI + cb;
+            pr[0] = s + kappa * gx * gx;
+            pr[SB] = kappa * gx * gy;
+            pr[2 * SB] = kappa * gx * gz;
+            pr[3 * SB] = s + kappa * gy * gy;
+            pr[4 * SB] = kappa * gy * gz;
+            pr[5 * SB] = s + kappa * gz * gz;
+        }
+        __syncthreads();
+        // C: stress plane q-1 folded into the partial forces; fields of plane q-2.  The next
+        // iteration's A rewrites only ring cells B has read and, in the slot of plane q-2, this
+        // thread's own tile cell and cells C does not read.
+        const int b0 = (dcy + 1) * WB + dcx + 1;
+        float T[3] = {0.f, 0.f, 0.f}, Sz[3] = {0.f, 0.f, 0.f}, F[3];
+#pragma unroll
+        for (int oy = -1; oy <= 1; ++oy)
+#pragma unroll
+            for (int ox = -1; ox <= 1; ++ox) {
+                const float w = (ox ? 1.f / 6.f : 2.f / 3.f) * (oy ? 1.f / 6.f : 2.f / 3.f);
+                const float *pp = PI + b0 + oy * WB + ox;
+                if (ox) {
+                    const float cw = ox * w;
+                    T[0] += cw * pp[0];
+                    T[1] += cw * pp[SB];
+                    T[2] += cw * pp[2 * SB];
+                }
+                if (oy) {
+                    const float cw = oy * w;
+                    T[0] += cw * pp[SB];
+                    T[1] += cw * pp[3 * SB];
+                    T[2] += cw * pp[4 * SB];
+                }
+                Sz[0] += w * pp[2 * SB];
+                Sz[1] += w * pp[4 * SB];
+                Sz[2] += w * pp[5 * SB];
+            }
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            F[m] = -3.f * (p2[m] + (1.f / 6.f) * (T[m] + Sz[m]));
+            p2[m] = p1[m] + (2.f / 3.f) * T[m];
+            p1[m] = (1.f / 6.f) * (T[m] - Sz[m]);
+        }
+        if (q - 2 < z0 || out_of) continue;                       // no barrier below
+        const float rho = RHO[sm2 * SA + sa(dcx, dcy)], ir = rcpa(rho);
+        float u[3];
+#pragma unroll
+        for (int m = 0; m < 3; ++m) u[m] = (j2[m] + 0.5f * F[m]) * ir;
+        const unsigned n = (unsigned)(q - 2) * (unsigned)nx * (unsigned)ny + (unsigned)(y0 + dcy) * (unsigned)nx +
+                           (unsigned)(x0 + dcx);
+        if (!in_bounds(n, N)) continue;
+        if (M.T) {
+            float RT;
+            if (THERMAL) {
+                unsigned zc[3];
+                plane_offsets(q - 2, nx, ny, nz, zc);
+                float Gam = 0.f;
+#pragma unroll
+                for (int i = 0; i < 27; ++i) {
+                    const unsigned si = src_of(i, cD, zc, N);
+                    float h = ldc(A.g, si, 27ull * N);
+                    if constexpr (DEV) h = decode_g<27>(cxi(i), cyi(i), czi(i), ldrec(A.Rin, si - i * N, N), h);
+                    Gam += h;
+                }
+                const float E = (Gam + 0.5f * (u[0] * F[0] + u[1] * F[1] + u[2] * F[2])) * ir;
+                RT = (2.f / 3.f) * (E - 0.5f * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
+            } else {
+                RT = ldc(A.RT_iso, n, N);
+            }
+            const float qt = RT * M.Ri;                            // RT / R, exact for R = 1
+            M.T[n] = fmaf(fmaf(-qt, M.Rl, fmaf(-qt, M.Rh, RT)), M.Ri, qt);
+        }
+        if (M.rho) M.rho[n] = rho;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            if (M.u) M.u[(size_t)m * N + n] = u[m];
+            if (M.F) M.F[(size_t)m * N + n] = F[m];
+        }
+    }
+}
+
 template <bool THERMAL, typename S>
 cudaError_t launch(const Args<S> &A, cudaStream_t st)
 {
@@ -888,8 +1065,8 @@ template <class G> int default_chunk(const KParams &p)
 }
 
 template <typename S>
-cudaError_t step_t(const KParams &p, const void *f, const void *g, void *fo, void *go, const void *RT_iso,
-                   const void *Rin, void *Rout, cudaStream_t st)
+Args<S> make_args3(const KParams &p, const void *f, const void *g, void *fo, void *go, const void *RT_iso,
+                   const void *Rin, void *Rout)
 {
     Args<S> A;
     A.f = static_cast<const S *>(f);
@@ -910,6 +1087,39 @@ cudaError_t step_t(const KParams &p, const void *f, const void *g, void *fo, voi
     A.lambda = float(p.lambda);
     A.c_eq = float(p.c_eq);
     A.c_star = float(p.c_star);
+    return A;
+}
+
+template <typename S>
+cudaError_t moments_t(const KParams &p, const void *f, const void *g, const void *RT_iso, const void *Rin,
+                      const MomentOut &o, cudaStream_t st)
+{
+    Args<S> A = make_args3<S>(p, f, g, nullptr, nullptr, RT_iso, Rin, nullptr);
+    MArgs M;
+    M.rho = o.rho;
+    M.u = o.u;
+    M.T = o.T;
+    M.F = o.F;
+    M.Rh = float(o.R);
+    M.Rl = float(o.R - double(M.Rh));
+    M.Ri = float(1.0 / o.R);
+    // Chunks of 32 planes (after 4 that fill the pipeline), shorter while the grid would leave
+    // slots of the GPU (152 SMs x 3) empty.
+    const int gx = (p.nx + MGeo::TX - 1) / MGeo::TX, gy = (p.ny + MGeo::TY - 1) / MGeo::TY;
+    A.HZ = 32;
+    while (A.HZ > 2 && (long long)gx * gy * ((p.nz + A.HZ - 1) / A.HZ) < 456) A.HZ >>= 1;
+    while ((p.nz + A.HZ - 1) / A.HZ > 65535) A.HZ <<= 1;
+    const dim3 grid(gx, gy, (p.nz + A.HZ - 1) / A.HZ);
+    if (p.thermal) k_moments3d<true, S><<<grid, MGeo::NT, 0, st>>>(A, M);
+    else k_moments3d<false, S><<<grid, MGeo::NT, 0, st>>>(A, M);
+    return cudaGetLastError();
+}
+
+template <typename S>
+cudaError_t step_t(const KParams &p, const void *f, const void *g, void *fo, void *go, const void *RT_iso,
+                   const void *Rin, void *Rout, cudaStream_t st)
+{
+    Args<S> A = make_args3<S>(p, f, g, fo, go, RT_iso, Rin, Rout);
     z_chunks(p.tile_h > 0 ? p.tile_h : default_chunk<typename TileOf<S>::G>(p), p.nz, A);
     return p.thermal ? launch<true, S>(A, st) : launch<false, S>(A, st);
 }
@@ -939,6 +1149,14 @@ cudaError_t fused3d_step(int prec, const KParams &p, const void *f, const void *
     if (prec == 2) return step_t<__half>(p, f, g, fo, go, RT_iso, Rin, Rout, st);
     if (prec == 3) return step_t<__nv_bfloat16>(p, f, g, fo, go, RT_iso, Rin, Rout, st);
     return step_t<float>(p, f, g, fo, go, RT_iso, Rin, Rout, st);
+}
+
+cudaError_t fused3d_moments(int prec, const KParams &p, const void *f, const void *g, const void *RT_iso,
+                            const void *Rin, const MomentOut &o, cudaStream_t st)
+{
+    if (prec == 2) return moments_t<__half>(p, f, g, RT_iso, Rin, o, st);
+    if (prec == 3) return moments_t<__nv_bfloat16>(p, f, g, RT_iso, Rin, o, st);
+    return moments_t<float>(p, f, g, RT_iso, Rin, o, st);
 }
 
 }  // namespace evlbm
