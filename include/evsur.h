@@ -109,8 +109,9 @@ typedef struct sur_gemm_args {
 } sur_gemm_args;
 
 /* One GEMM on the tensor cores (128 x {32,64,128} CTA tiles, 64-deep K blocks,
- * one thread issuing tcgen05.mma into a TMEM accumulator).  A CONV3 or PIX A
- * operand with a DENSE B operand and no split is fed by TMA (swizzled
+ * one thread issuing tcgen05.mma into a TMEM accumulator).  A CONV3, PIX or UPADJ
+ * A operand with a DENSE B operand and no split, and a TCONV3, TUP or TPIX A operand
+ * with a TPIX B operand over whole images, are fed by TMA (swizzled
  * cp.async.bulk.tensor boxes); every other form by a cp.async pipeline.
  * d_status (device int) is set to 1 if a wait gave up. */
 int sur_gemm(const sur_gemm_args *g, int *d_status, void *stream);

@@ -8,13 +8,14 @@
 // Activations are NHWC matrices stored halo-padded: [B][H+2][W+2][C], the
 // border rows and columns holding periodic copies, so a 3x3 tap is a plain
 // shifted window of the stored tensor.  Two mainloops feed the tensor core:
-//   * TMA: the forward convolutions.  Each 64-deep K block of A is one (or,
-//     for 32- and 8-channel inputs, 2 or 8) cp.async.bulk.tensor boxes of 128
-//     pixels of the shifted window, swizzled 128/64 B (none for 8 channels); B
-//     (the weights) is one swizzled box.  One thread issues the copies, one the
-//     MMAs, four warps run the epilogue.
-//   * cp.async: every other operand form (the adjoint gathers and the MN-major
-//     weight-gradient operands); four producer warps, one MMA warp.
+//   * TMA: the convolutions and their input and weight gradients.  Each 64-deep K
+//     block of A is one (or, for 32- and 8-channel inputs, 2 or 8)
+//     cp.async.bulk.tensor boxes of 128 pixels of the shifted window, swizzled
+//     128/64 B (none for 8 channels); B (the weights) is one swizzled box.  The
+//     children of the coarse pixels (UPADJ, TUP) are boxes of a five-dimensional
+//     view of the fine tensor.  One thread issues the copies, one the MMAs, four
+//     warps run the epilogue.
+//   * cp.async: every other operand form; four producer warps, one MMA warp.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <stdint.h>
@@ -421,7 +422,8 @@ __global__ void __launch_bounds__(160, 1) k_gemm_cpasync(const KArgs g)
 struct TArgs {
     int nkb;
     int mtiles, ntiles;   // tile grid (the launch grid is smaller: CTAs loop over tiles)
-    int kind;          // SUR_OP_CONV3 or SUR_OP_PIX
+    int kind;          // SUR_OP_* of A
+    int ld;            // row stride of A, elements (UPADJ, TUP)
     int lc, c0;        // log2 channels of the gathered tensor, first channel
     int lh, lw;        // interior grid of A
     int boxw, boxh;    // pixels of one box row, box rows (a tile is boxw * boxh * boxs pixels)
@@ -450,6 +452,16 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map
         "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
         "%5}], [%6];" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
+        : "memory");
+}
+
+__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2, int c3,
+                                            int c4, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+        "%5, %6}], [%7];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
         : "memory");
 }
 
@@ -573,6 +585,13 @@ __global__ void __launch_bounds__(192, 1)
                         (void)boxw;
                         for (int sg = 0; sg < nsa; ++sg) {
                             const long long r = tc.m0 + (long long)sg * g.a_cb;
+                            if (g.kind == SUR_OP_TUP) {
+                                // Children r / C of the coarse pixels; 4.. (M padding) lie outside: zeros.
+                                const int ch = (int)(r >> g.lc), cc = (int)(r & ((1 << g.lc) - 1));
+                                tma_load_5d(sa + (uint32_t)(sg * g.a_cb * 128), &tmA, g.c0 + (ch & 1) * g.ld + cc, x,
+                                            ch >> 1, y, b, bar);
+                                continue;
+                            }
                             int tap = 4, c = (int)r;
                             if (g.kind == SUR_OP_TCONV3) {
                                 tap = (int)(r >> g.lc);
@@ -608,6 +627,12 @@ __global__ void __launch_bounds__(192, 1)
 #pragma unroll
                     for (int j = 0; j < NBOX; ++j) {
                         const int k = kb * 64 + j * CB;          // first K index of the box
+                        if (g.kind == SUR_OP_UPADJ) {
+                            const int ch = k >> g.lc, cc = k & ((1 << g.lc) - 1);
+                            tma_load_5d(sa + j * BOXB, &tmA, g.c0 + (ch & 1) * g.ld + cc, x0, ch >> 1, y0, b0,
+                                        smem_u32(&full[s]));
+                            continue;
+                        }
                         int tap = 4, cc = k;                     // PIX: centre tap, channels k..
                         if (g.kind == SUR_OP_CONV3) {
                             tap = k >> g.lc;
@@ -982,6 +1007,25 @@ cudaError_t dispatch_tma(int N, const CUtensorMap &ma, const CUtensorMap &mb, co
     return launch_tma<32, ASW>(ma, mb, g, mtiles, st);
 }
 
+// View of a halo-padded fine tensor [B][2H+2][2W+2][ld] as the children of coarse pixels:
+// (child column and channel, coarse x, child row, coarse y, image), starting at the first
+// interior pixel; child s, channel c is (s % 2 * ld + c, x, s / 2, y, image).  Boxes of cb
+// channels of one child for boxw x boxh x boxs coarse pixels.
+bool encode_children(CUtensorMap &m, const sur_operand &o, long long images, int cb, int boxw, int boxh, int boxs)
+{
+    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+    if (!enc) return false;
+    const cuuint64_t px = 2ull * o.ld, row = (2ull * o.W + 2) * px;      // bytes of a fine pixel and row
+    cuuint64_t dims[5] = {2ull * o.ld, (cuuint64_t)o.W, 2, (cuuint64_t)o.H, (cuuint64_t)images};
+    cuuint64_t strides[4] = {2 * px, row, 2 * row, (2ull * o.H + 2) * row};
+    cuuint32_t box[5] = {(cuuint32_t)cb, (cuuint32_t)boxw, 1, (cuuint32_t)boxh, (cuuint32_t)boxs};
+    cuuint32_t es[5] = {1, 1, 1, 1, 1};
+    char *first = const_cast<char *>(static_cast<const char *>(o.p)) + row + px;
+    return enc(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, first, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               cb == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Tensor maps of a TMA-eligible GEMM; false if the encoder rejects them.
 bool make_maps(const sur_gemm_args &a, int bn, CUtensorMap &ma, CUtensorMap &mb, TArgs &tg)
 {
@@ -1001,9 +1045,11 @@ bool make_maps(const sur_gemm_args &a, int bn, CUtensorMap &ma, CUtensorMap &mb,
     cuuint32_t es[4] = {1, 1, 1, 1};
     const CUtensorMapSwizzle sw = cb == 64 ? CU_TENSOR_MAP_SWIZZLE_128B
                                            : (cb == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE);
-    if (enc(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(a.a.p), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    if (a.a.kind == SUR_OP_UPADJ) {
+        if (!encode_children(ma, a.a, samples, cb, boxw, boxh, boxs)) return false;
+    } else if (enc(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(a.a.p), dims, strides, box, es,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return false;
     cuuint64_t bdims[2] = {(cuuint64_t)a.b.ld, (cuuint64_t)a.b.rows};
     cuuint64_t bstr[1] = {a.b.ld * e2};
@@ -1015,6 +1061,7 @@ bool make_maps(const sur_gemm_args &a, int bn, CUtensorMap &ma, CUtensorMap &mb,
         return false;
     tg.nkb = a.K / 64;
     tg.kind = a.a.kind;
+    tg.ld = a.a.ld;
     tg.lc = ilog2(C);
     tg.c0 = a.a.c0;
     tg.lh = ilog2(H);
@@ -1025,21 +1072,24 @@ bool make_maps(const sur_gemm_args &a, int bn, CUtensorMap &ma, CUtensorMap &mb,
     return true;
 }
 
-// Weight-gradient GEMMs: A = TCONV3 or TPIX, B = TPIX on the same pixel grid, dense FP32
-// output.  Rows of A at or beyond `rows` must read zero: TCONV3 rows of taps >= 9 load
-// boxes wholly outside the tensor (zeros), so M may exceed `rows` when rows >= 9 C (the
-// K padding of the weights); any other row range must lie inside `rows`.
+// Weight-gradient GEMMs: A = TCONV3, TUP or TPIX, B = TPIX on the same pixel grid, dense FP32
+// output.  Rows of A at or beyond `rows` must read zero: TCONV3 rows of taps >= 9 (TUP: of
+// children >= 4) load boxes wholly outside the tensor (zeros), so M may exceed `rows` when
+// rows >= 9 C (4 C; the K padding of the weights); any other row range must lie inside `rows`.
 bool tma_mn_eligible(const sur_gemm_args &a)
 {
     if (!g_tma_enabled || a.b.kind != SUR_OP_TPIX) return false;
-    if (a.a.kind != SUR_OP_TCONV3 && a.a.kind != SUR_OP_TPIX) return false;
+    if (a.a.kind != SUR_OP_TCONV3 && a.a.kind != SUR_OP_TPIX && a.a.kind != SUR_OP_TUP) return false;
     if (a.epi != SUR_EPI_F32_ATOMIC && a.epi != SUR_EPI_F32) return false;
     if (a.K % 64 || a.a.H != a.b.H || a.a.W != a.b.W || a.a.W < 8 || a.a.H < 1) return false;
     const long long hw = (long long)a.a.H * a.a.W;
     if (a.K % hw || a.N > a.b.rows) return false;
-    if (a.M > a.a.rows && !(a.a.kind == SUR_OP_TCONV3 && a.a.rows >= 9 * a.a.C)) return false;
+    if (a.M > a.a.rows && !((a.a.kind == SUR_OP_TCONV3 && a.a.rows >= 9 * a.a.C) ||
+                            (a.a.kind == SUR_OP_TUP && a.a.rows >= 4 * a.a.C)))
+        return false;
     if (hw % 64) return false;
     if (a.a.kind == SUR_OP_TCONV3 && !(a.a.C == 8 || a.a.C == 32 || a.a.C % 64 == 0)) return false;
+    if (a.a.kind == SUR_OP_TUP && !(a.a.C == 32 || a.a.C % 64 == 0)) return false;
     return true;
 }
 
@@ -1052,7 +1102,7 @@ bool make_maps_mn(const sur_gemm_args &a, int bn, CUtensorMap &ma, CUtensorMap &
     const int H = a.a.H, W = a.a.W;
     const long long images = a.K / ((long long)H * W);
     const int boxw = W < 64 ? W : 64, boxh = 64 / boxw;
-    const int acb = a.a.kind == SUR_OP_TCONV3 ? (a.a.C < 64 ? a.a.C : 64) : 64;
+    const int acb = a.a.kind != SUR_OP_TPIX ? (a.a.C < 64 ? a.a.C : 64) : 64;
     const int bcb = bn < 64 ? bn : 64;
     if (!(acb == 64 || acb == 32 || acb == 8) || !(bcb == 64 || bcb == 32)) return false;
     auto encode = [&](CUtensorMap &m, const sur_operand &o, int cb) {
@@ -1067,7 +1117,9 @@ bool make_maps_mn(const sur_gemm_args &a, int bn, CUtensorMap &ma, CUtensorMap &
                    CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
-    if (!encode(ma, a.a, acb) || !encode(mb, a.b, bcb)) return false;
+    if (!(a.a.kind == SUR_OP_TUP ? encode_children(ma, a.a, images, acb, boxw, boxh, 1) : encode(ma, a.a, acb)) ||
+        !encode(mb, a.b, bcb))
+        return false;
     // Descriptor fields: (lbo, sbo, k-step, layout) per channels of the MN atom.
     auto fields = [](int cb, int &lbo, int &sbo, int &kstep, int &sw) {
         if (cb == 64) { lbo = 8192; sbo = 1024; kstep = 2048; sw = 2; }
@@ -1082,7 +1134,8 @@ bool make_maps_mn(const sur_gemm_args &a, int bn, CUtensorMap &ma, CUtensorMap &
     const long long kb = a.K / 64;
     const long long kbps = (kb + a.splits - 1) / a.splits;
     tg.kind = a.a.kind;
-    tg.lc = a.a.kind == SUR_OP_TCONV3 ? ilog2(a.a.C) : 0;
+    tg.ld = a.a.ld;
+    tg.lc = a.a.kind != SUR_OP_TPIX ? ilog2(a.a.C) : 0;
     tg.lh = ilog2(H);
     tg.lw = ilog2(W);
     tg.c0 = a.a.c0;
@@ -1106,6 +1159,8 @@ bool tma_eligible(const sur_gemm_args &a)
         if (a.K > (9 * C + 63) / 64 * 64) return false;
     } else if (a.a.kind == SUR_OP_PIX) {
         if (C % 64 || a.K > C) return false;
+    } else if (a.a.kind == SUR_OP_UPADJ) {
+        if (!(C == 32 || C % 64 == 0) || a.K > 4 * C) return false;
     } else {
         return false;
     }
