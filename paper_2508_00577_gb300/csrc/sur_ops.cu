@@ -41,19 +41,27 @@ inline int log2i(int v)
 
 // Sum over the block of each thread's 8-channel partial sums into out[c] (atomic).  Every
 // thread of a block keeps one channel group, threadIdx.x % C8: the grid stride and the
-// block size (256) are multiples of C8 = C / 8 <= 32.
+// block size (256) are multiples of C8 = C / 8 <= 32, a power of two.  The sums are added by
+// consecutive threads to consecutive channels: with a thread adding its 8 channels in turn
+// (32-byte strides in a warp) the additions to one sector, 8 times as many, took most of the
+// time of the narrow levels (SiLU backward of 2^14 pixels x 256 channels: 63 us).
 __device__ __forceinline__ void block_colsum8(const float acc[8], int C8, float *out)
 {
     __shared__ float red[256][9];
+    const int t = threadIdx.x, C = C8 * 8, parts = 256 / C;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) red[threadIdx.x][j] = acc[j];
+    for (int j = 0; j < 8; ++j) red[t][j] = acc[j];
     __syncthreads();
-    if ((int)threadIdx.x < C8) {
-        for (int j = 0; j < 8; ++j) {
-            float s = 0.f;
-            for (int k = threadIdx.x; k < 256; k += C8) s += red[k][j];
-            atomicAdd(out + threadIdx.x * 8 + j, s);
-        }
+    // Thread = (channel t % C, part t / C of the threads that hold its group).
+    const int c = t % C;
+    float s = 0.f;
+    for (int k = (c >> 3) + C8 * (t / C); k < 256; k += C8 * parts) s += red[k][c & 7];
+    __syncthreads();
+    red[t][8] = s;
+    __syncthreads();
+    if (t < C) {
+        for (int q = 1; q < parts; ++q) s += red[t + q * C][8];
+        atomicAdd(out + t, s);
     }
 }
 
@@ -261,18 +269,27 @@ __global__ void __launch_bounds__(256) k_head(const bf16 *Y, long long M, int lh
         if (MODE != kHeadNext) {
             sd[t] = d;
             __syncwarp();
-#pragma unroll 8
-            for (int k = 0; k < 32; ++k) {
-                const int px = wi * 32 + k;
-                const float4 dk = sd[px];
-                bf16 *yp = reinterpret_cast<bf16 *>(sy + px * 5) + lane;
-                const float f = base + px < M ? __bfloat162float(*yp) : 0.f;
-                *yp = __float2bfloat16_rn(dk.x * wl[0] + dk.y * wl[1] + dk.z * wl[2] + dk.w * wl[3]);
-                gw[0] += dk.x * f;
-                gw[1] += dk.y * f;
-                gw[2] += dk.z * f;
-                gw[3] += dk.w * f;
-                if (lane < 4) gb += lane == 0 ? dk.x : (lane == 1 ? dk.y : (lane == 2 ? dk.z : dk.w));
+            // Eight pixels at a time: their reads go before the writes to the same array.
+#pragma unroll 1
+            for (int k8 = 0; k8 < 32; k8 += 8) {
+                float f[8];
+                float4 dk[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int px = wi * 32 + k8 + k;
+                    dk[k] = sd[px];
+                    f[k] = base + px < M ? __bfloat162float(reinterpret_cast<const bf16 *>(sy + px * 5)[lane]) : 0.f;
+                }
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    reinterpret_cast<bf16 *>(sy + (wi * 32 + k8 + k) * 5)[lane] =
+                        __float2bfloat16_rn(dk[k].x * wl[0] + dk[k].y * wl[1] + dk[k].z * wl[2] + dk[k].w * wl[3]);
+                    gw[0] += dk[k].x * f[k];
+                    gw[1] += dk[k].y * f[k];
+                    gw[2] += dk[k].z * f[k];
+                    gw[3] += dk[k].w * f[k];
+                    if (lane < 4) gb += lane == 0 ? dk[k].x : (lane == 1 ? dk[k].y : (lane == 2 ? dk[k].z : dk[k].w));
+                }
             }
             __syncthreads();
 #pragma unroll
