@@ -80,6 +80,30 @@ struct Epi {
     int *status;
 };
 
+// Four floats added to 16-byte aligned memory in one request.
+__device__ __forceinline__ void red_add4(float *p, float a, float b, float c, float d)
+{
+    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
+                 : "memory");
+}
+
+// 32 accumulator columns of the warp's 32 lanes, waited for (warp-collective).
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float v[32])
+{
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;");
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+}
+
 template <int BN>
 __device__ __forceinline__ void epilogue(const Epi &g, uint32_t tmem, long long m0, int n0, int warp, int lane,
                                          int cbeg = 0, int cend = BN)
@@ -105,27 +129,19 @@ __device__ __forceinline__ void epilogue(const Epi &g, uint32_t tmem, long long 
     };
 #pragma unroll 1
     for (int c0 = cbeg; c0 < cend; c0 += 32) {
-        uint32_t r[32];
-        const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + c0;
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-            "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-              "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-              "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]),
-              "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
-              "=r"(r[30]), "=r"(r[31])
-            : "r"(taddr));
-        asm volatile("tcgen05.wait::ld.sync.aligned;");
+        float v[32];
+        tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + c0, v);
         if (!rv) continue;
         const int col = n0 + c0;
-        float v[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
         if (g.epi == SUR_EPI_F32_ATOMIC) {
             float *o = static_cast<float *>(g.out) + row * g.ldo + g.co0 + col;
+            if ((reinterpret_cast<uintptr_t>(o) & 15) == 0) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) atomicAdd(o + j, v[j]);
+                for (int j = 0; j < 32; j += 4) red_add4(o + j, v[j], v[j + 1], v[j + 2], v[j + 3]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) atomicAdd(o + j, v[j]);
+            }
         } else if (g.epi == SUR_EPI_SHUF) {
             const int sidx = col / g.shuf_cout, c = col - sidx * g.shuf_cout;
             add_bias(v, g.bias + c);
@@ -894,6 +910,179 @@ __global__ void __launch_bounds__(32 * (CfgR<C, N>::EW + 2), CfgR<C, N>::CTAS)
     if (warp == 0) tmem_free(tmem, TCOLS);
 }
 
+// ---------------------------------------------------------------------------
+// Row-marching weight gradient of a 3x3 convolution (images at least 128 pixels wide)
+// ---------------------------------------------------------------------------
+// dW[tap C + c][n] = sum over pixels of X[pixel + tap][c] dZ[pixel][n], pixels along K, both
+// operands MN-major.  The MN-major TMA mainloop above loads a box of X per tap and 64 pixels,
+// and dZ again for each block of 128 rows: 0.8 + 0.2 KB a pixel at 32 x 32 channels, which
+// bound it (110 us at 2^20 pixels).  Here a CTA walks down a column of 128 pixels with rings of
+// X rows (halo-wide) and dZ rows in shared memory, and one instruction covers neighbouring
+// taps of a kernel row: the 128 rows of A are 128 / CB atoms of CB channels, each started one
+// pixel after the one before (the stride between MN atoms is a pixel).  Atoms past dx = +1
+// read pixels beyond the halo (or whatever the stage holds there); their rows of the
+// accumulator are never read.  The whole gradient stays in tensor memory, 3 kernel rows x NM
+// instructions x N columns, and is added to the output once per CTA.
+template <int CB, int N> struct CfgW {
+    static constexpr int RB = CB * 2, ATOMS = 128 / CB, NM = CB == 64 ? 2 : 1;
+    static constexpr int PX = 128 + (NM - 1) * 2 + ATOMS - 1;                 // pixels an instruction may touch
+    static constexpr int XROW = (PX * RB + 1023) / 1024 * 1024, ZRB = N * 2, ZROW = 128 * ZRB;
+    static constexpr int COLS = 3 * NM * N, TCOLS = COLS <= 128 ? 128 : (COLS <= 256 ? 256 : 512);
+    static constexpr int CTAS = TCOLS == 512 ? 1 : 2;
+    static constexpr int NX = CTAS == 1 ? 8 : (CB == 64 ? 4 : 5), NZ = CTAS == 2 && N == 64 ? 3 : 4;
+    static constexpr int SMEM = NX * XROW + NZ * ZROW + 1024;
+    static_assert(CTAS * (SMEM + 2048) <= 232448 && CTAS * TCOLS <= 512, "resident CTAs");
+};
+
+struct WArgs {
+    int c0, b_c0;         // first channel of A and of B
+    int C;                // channels of A: blockIdx.y takes CB of them
+    int lh, lw;           // image size
+    int tiles;            // image rows x columns of 128 pixels, all images
+    float *out;           // [9 C][ldo]
+    int ldo, co0;
+    int *status;
+};
+
+template <int CB, int N>
+__global__ void __launch_bounds__(192, CfgW<CB, N>::CTAS)
+    k_wgrad_rows(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmZ, const WArgs g)
+{
+    using Cf = CfgW<CB, N>;
+    constexpr int NX = Cf::NX, NZ = Cf::NZ;
+    extern __shared__ unsigned char dsm_raw[];
+    __shared__ __align__(8) uint64_t fullx[NX], emptyx[NX], fullz[NZ], emptyz[NZ], done_bar;
+    __shared__ uint32_t tmem_sh;
+    __shared__ int abort_flag;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    volatile int *abort_v = &abort_flag;
+    const int t0 = (int)((long long)g.tiles * blockIdx.x / gridDim.x);
+    const int t1 = (int)((long long)g.tiles * (blockIdx.x + 1) / gridDim.x);
+    const int H = 1 << g.lh, cbase = (int)blockIdx.y * CB;
+
+    if (warp == 0) tmem_alloc(&tmem_sh, Cf::TCOLS);
+    if (t == 0) {
+        for (int s = 0; s < NX; ++s) {
+            mbar_init(smem_u32(&fullx[s]), 1);
+            mbar_init(smem_u32(&emptyx[s]), 1);
+        }
+        for (int s = 0; s < NZ; ++s) {
+            mbar_init(smem_u32(&fullz[s]), 1);
+            mbar_init(smem_u32(&emptyz[s]), 1);
+        }
+        mbar_init(smem_u32(&done_bar), 1);
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tmem = tmem_sh;
+    const uint32_t xbase = (smem_u32(dsm_raw) + 1023u) & ~1023u, zbase = xbase + (uint32_t)(NX * Cf::XROW);
+
+    if (warp == 4) {
+        if (lane == 0) {
+            // ---------------- TMA producer ----------------
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmX)) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmZ)) : "memory");
+            int rx = 0, rz = 0;                                   // rows loaded so far
+            bool ok = true;
+            for (int i = t0; i < t1 && ok; ++i) {
+                const int y = i & (H - 1), col = i >> g.lh;
+                const int b = col >> (g.lw - 7), x0 = (col & ((1 << (g.lw - 7)) - 1)) << 7;
+                for (int yy = (i == t0 || y == 0) ? y : y + 2; yy <= y + 2 && ok; ++yy, ++rx) {
+                    const int s = rx % NX;
+                    if (rx >= NX && !mbar_wait(smem_u32(&emptyx[s]), (uint32_t)((rx / NX - 1) & 1), abort_v)) {
+                        *abort_v = 1;
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&fullx[s])),
+                                 "r"((uint32_t)(130 * Cf::RB)));
+                    tma_load_4d(xbase + (uint32_t)(s * Cf::XROW), &tmX, g.c0 + cbase, x0, yy, b, smem_u32(&fullx[s]));
+                }
+                if (!ok) break;
+                const int s = rz % NZ;
+                if (rz >= NZ && !mbar_wait(smem_u32(&emptyz[s]), (uint32_t)((rz / NZ - 1) & 1), abort_v)) {
+                    *abort_v = 1;
+                    break;
+                }
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&fullz[s])),
+                             "r"((uint32_t)Cf::ZROW));
+                tma_load_4d(zbase + (uint32_t)(s * Cf::ZROW), &tmZ, g.b_c0, x0 + 1, y + 1, b, smem_u32(&fullz[s]));
+                ++rz;
+            }
+            // No copy may be in flight when the CTA ends (after a wait gave up).
+            for (int k = rx > NX ? rx - NX : 0; k < rx; ++k) mbar_wait(smem_u32(&fullx[k % NX]), (uint32_t)((k / NX) & 1));
+            for (int k = rz > NZ ? rz - NZ : 0; k < rz; ++k) mbar_wait(smem_u32(&fullz[k % NZ]), (uint32_t)((k / NZ) & 1));
+        }
+    } else if (warp == 5) {
+        if (lane == 0) {
+            // ---------------- MMA issuer ----------------
+            const uint32_t idesc = make_idesc(N, true, true);
+            // A: swizzled atoms CB >= 32 take LBO = stride between MN atoms (one pixel) and
+            // SBO = stride between 8-pixel groups; the unswizzled 8-channel atoms the reverse.
+            constexpr uint32_t a_lbo = CB == 8 ? 8 * Cf::RB : Cf::RB, a_sbo = CB == 8 ? Cf::RB : 8 * Cf::RB;
+            constexpr uint32_t a_sw = CB == 64 ? 2 : (CB == 32 ? 4 : 0), b_sbo = 8 * Cf::ZRB, b_sw = N == 64 ? 2 : 4;
+            bool ok = true;
+            int top = 0, have = 0, lt = 0;
+            for (int i = t0; i < t1 && ok; ++i, ++lt) {
+                const int y = i & (H - 1);
+                for (; have < top + 3 && ok; ++have)
+                    if (!mbar_wait(smem_u32(&fullx[have % NX]), (uint32_t)((have / NX) & 1), abort_v)) ok = false;
+                const int sz = lt % NZ;
+                if (ok && !mbar_wait(smem_u32(&fullz[sz]), (uint32_t)((lt / NZ) & 1), abort_v)) ok = false;
+                if (!ok) {
+                    *abort_v = 1;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t rz = zbase + (uint32_t)(sz * Cf::ZROW);
+#pragma unroll 1
+                for (int dy = 0; dy < 3; ++dy) {
+                    const uint32_t ra = xbase + (uint32_t)((top + dy) % NX * Cf::XROW);
+#pragma unroll
+                    for (int m = 0; m < Cf::NM; ++m)
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {             // 16 pixels each
+                            const uint64_t da = smem_desc(ra + (uint32_t)((16 * k + 2 * m) * Cf::RB), a_lbo, a_sbo, a_sw);
+                            const uint64_t db = smem_desc(rz + (uint32_t)(16 * k * Cf::ZRB), b_sbo, b_sbo, b_sw);
+                            mma_bf16(tmem + (uint32_t)((dy * Cf::NM + m) * N), da, db, idesc, lt > 0 || k > 0 ? 1u : 0u);
+                        }
+                }
+                const int next = i + 1 < t1 && y != H - 1 ? 1 : 3;
+                for (int k = 0; k < next; ++k) mma_commit(smem_u32(&emptyx[(top + k) % NX]));
+                top += next;
+                mma_commit(smem_u32(&emptyz[sz]));
+            }
+            mma_commit(smem_u32(&done_bar));   // arrives once every MMA above completed
+        }
+    } else {
+        // ---------------- epilogue, once: thread = accumulator row = (atom, channel) ----------------
+        const bool fin = mbar_wait(smem_u32(&done_bar), 0);
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        if (!fin) *abort_v = 1;
+        __syncwarp();
+        if (__all_sync(0xffffffffu, fin && !*abort_v && t1 > t0)) {
+            const int row = warp * 32 + lane, atom = row / CB, c = row % CB;
+#pragma unroll 1
+            for (int q = 0; q < 3 * Cf::NM * (N / 32); ++q) {
+                const int n0 = q % (N / 32) * 32, dm = q / (N / 32), dy = dm / Cf::NM, dx = dm % Cf::NM * 2 + atom;
+                float v[32];
+                tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(dm * N + n0), v);
+                if (dx > 2) continue;
+                float *o = g.out + (long long)((dy * 3 + dx) * g.C + cbase + c) * g.ldo + g.co0 + n0;
+#pragma unroll
+                for (int j = 0; j < 32; j += 4) red_add4(o + j, v[j], v[j + 1], v[j + 2], v[j + 3]);
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    if (t == 0 && *abort_v) atomicExch(g.status, 1);
+    if (warp == 0) tmem_free(tmem, Cf::TCOLS);
+}
+
 }  // namespace
 
 }  // namespace evsur
@@ -1223,6 +1412,66 @@ int launch_rows(const sur_gemm_args &a, const Epi &e, cudaStream_t st)
     return cudaGetLastError() == cudaSuccess ? SUR_OK : SUR_ECUDA;
 }
 
+// Row-marching weight gradient: eligible shapes (of those tma_mn_eligible accepts) are whole
+// convolutions (rows of A are all 9 C, M at most padded) over images at least 128 pixels wide,
+// 32 or 64 output columns, 8, 32 or a multiple of 64 channels, and an output whose rows are
+// 16-byte aligned; the split count does not matter to it.
+bool wgrad_eligible(const sur_gemm_args &a)
+{
+    if (a.a.kind != SUR_OP_TCONV3 || a.epi != SUR_EPI_F32_ATOMIC || a.a.W < 128) return false;
+    if (a.M < 9 * a.a.C || a.a.rows < 9 * a.a.C || a.ldo % 4 || a.co0 % 4) return false;
+    return a.N == 32 || a.N == 64;
+}
+
+template <int CB, int N>
+int launch_wgrad(const sur_gemm_args &a, int *status, cudaStream_t st)
+{
+    using Cf = CfgW<CB, N>;
+    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+    if (!enc) return -1;
+    const int H = a.a.H, W = a.a.W;
+    const long long images = a.K / ((long long)H * W);
+    CUtensorMap mx, mz;
+    auto encode = [&](CUtensorMap &m, const sur_operand &o, int cb, int px) {
+        const size_t e2 = 2;
+        cuuint64_t dims[4] = {(cuuint64_t)o.ld, (cuuint64_t)(W + 2), (cuuint64_t)(H + 2), (cuuint64_t)images};
+        cuuint64_t strides[3] = {o.ld * e2, (cuuint64_t)(W + 2) * o.ld * e2, (cuuint64_t)(H + 2) * (W + 2) * o.ld * e2};
+        cuuint32_t box[4] = {(cuuint32_t)cb, (cuuint32_t)px, 1, 1}, es[4] = {1, 1, 1, 1};
+        const CUtensorMapSwizzle sw = cb == 64 ? CU_TENSOR_MAP_SWIZZLE_128B
+                                               : (cb == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE);
+        return enc(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(o.p), dims, strides, box, es,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    if (!encode(mx, a.a, CB, 130) || !encode(mz, a.b, N, 128)) return -1;
+    static int attr_dev = -1, sms = 0;
+    if (set_smem(k_wgrad_rows<CB, N>, Cf::SMEM, attr_dev) != cudaSuccess) return SUR_ECUDA;
+    if (!sms) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return SUR_ECUDA;
+    }
+    WArgs g;
+    g.c0 = a.a.c0;
+    g.b_c0 = a.b.c0;
+    g.C = a.a.C;
+    g.lh = ilog2(H);
+    g.lw = ilog2(W);
+    g.tiles = a.K / 128;
+    g.out = static_cast<float *>(a.out);
+    g.ldo = a.ldo;
+    g.co0 = a.co0;
+    g.status = status;
+    // As many CTAs as fit at once over the channel blocks, at least 8 rows each.
+    const int parts = a.a.C / CB;
+    int ctas = Cf::CTAS * sms / parts;
+    if (g.tiles / 8 < ctas) ctas = g.tiles / 8;
+    if (ctas < 1) ctas = 1;
+    k_wgrad_rows<CB, N><<<dim3(ctas, parts), 192, Cf::SMEM, st>>>(mx, mz, g);
+    return cudaGetLastError() == cudaSuccess ? SUR_OK : SUR_ECUDA;
+}
+
 }  // namespace
 
 void set_tma(bool on) { g_tma_enabled = on; }
@@ -1280,6 +1529,15 @@ int gemm(const sur_gemm_args &a, int *status, cudaStream_t st)
     if (mtiles > 0x7FFFFFFF) return SUR_EINVAL;
     const int bn = a.N % 128 == 0 ? 128 : (a.N % 64 == 0 ? 64 : 32);
     cudaError_t err;
+    if (tma_mn_eligible(a) && wgrad_eligible(a)) {
+        const int rc = a.N == 32 ? (a.a.C == 8 ? launch_wgrad<8, 32>(a, status, st)
+                                               : (a.a.C == 32 ? launch_wgrad<32, 32>(a, status, st)
+                                                              : launch_wgrad<64, 32>(a, status, st)))
+                                 : (a.a.C == 8 ? launch_wgrad<8, 64>(a, status, st)
+                                               : (a.a.C == 32 ? launch_wgrad<32, 64>(a, status, st)
+                                                              : launch_wgrad<64, 64>(a, status, st)));
+        if (rc >= 0) return rc;                // -1: a tensor map was refused
+    }
     if (tma_mn_eligible(a)) {
         CUtensorMap ma, mb;
         TArgs tg;
