@@ -18,7 +18,7 @@ bool fused2d_supported(int prec, int Q, const KParams &p)
 }
 
 // Default launch shape: the candidate with the least estimated time.  A CTA that marches p
-// row pairs runs p + 5 iterations per tile (the pipeline of four stages fills first), and the
+// row pairs runs p + 4 iterations per tile (the pipeline of four stages fills first), and the
 // time of one iteration depends on the strip width and on how many CTAs share an SM.  The
 // measured times of an iteration (us, thermal FP32; the ratios hold for the isothermal kernel
 // and 16-bit storage):
@@ -36,7 +36,7 @@ void fused2d_default_tile(const KParams &p, int *W, int *H)
     static const int widths[3] = {128, 96, 64}, per_sm[3] = {2, 2, 4};
     static const float iter_us[3][4] = {{1.50f, 2.35f, 0.f, 0.f}, {1.20f, 2.25f, 0.f, 0.f}, {1.28f, 1.60f, 2.20f, 2.90f}};
     static const int heights[] = {2, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 256};
-    constexpr int kFill = 5;
+    constexpr int kFill = 4;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)

@@ -277,7 +277,16 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &A, int bx, int y0, i
     // Pair indices: pair q holds rows 2q, 2q+1 (absolute, unwrapped).
     const int q0 = y0 / 2;
     const int qD_end = (y0 + Heff + 1) / 2;              // one past the last collided pair
-    const int qbeg = q0 - (MOM ? 2 : 3), qend = qD_end + (MOM ? 1 : 2);
+    // Rows, not pairs, bound what is needed: D of row y0 needs fields (C) of row y0 - 1, hence
+    // stresses (B) of row y0 - 2 and densities (A) of row y0 - 3, which lie in pairs q0 - 1,
+    // q0 - 1 and q0 - 2.  The other row of such a pair may come out undefined (from ring cells
+    // not written yet); nothing reads it.  Likewise A ends at pair qD_end + 1 (one iteration
+    // before the last) and B at pair qD_end.  Against filling by whole pairs (one iteration and
+    // two pulled f pairs more per tile), us per window of 50 steps: 331 x 203 x 2 837 -> 736,
+    // 256^2 x 16 2556 -> 2504, 9 x 1024^2 (20 steps) 6871 -> 6853; the values are the same.
+    // With 16-bit storage A and B run on in the last iteration: the conditions cost that
+    // kernel, which is bound by issue, 7 % on 9 x 1024^2.
+    const int qbeg = q0 - (MOM ? 1 : 2), qend = qD_end + (MOM ? 1 : 2);
     int rA = wrap_any(2 * qbeg, ny);                      // wrapped first row of the next A pair
     int rC = wrap_any(2 * (q0 - (MOM ? 0 : 1)), ny);      // ... of the next C pair
     int rD = wrap_any(2 * q0, ny);                        // ... of the next D (MOM: output) pair
@@ -299,7 +308,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &A, int bx, int y0, i
         const int sm1 = s0 == 0 ? 2 : s0 - 1;             // slot of q-1 (and of q-4)
         const int sm2 = s0 == 2 ? 0 : s0 + 1;             // slot of q-2 (q-3 shares s0)
         // ---------------- A: rho, j of pair q ----------------
-        if (inA) {
+        if (inA && (DEV || q < qend)) {
             fld(RHO, s0)[slot] = sum9(pf);
             fld(JX, s0)[slot] = ((pf[2] + pf[5]) + pf[8]) - ((pf[0] + pf[3]) + pf[6]);
             fld(JY, s0)[slot] = ((pf[6] + pf[7]) + pf[8]) - ((pf[0] + pf[1]) + pf[2]);
@@ -327,7 +336,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &A, int bx, int y0, i
                 }
             }
             rA = next_row(next_row(rA, ny), ny);
-            if (q < qend) {
+            if (q + (DEV ? 0 : 1) < qend) {
                 unsigned ro[4];
                 rows4(rA, ro);
                 pull(A.f, ro, pf, false);
@@ -336,7 +345,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &A, int bx, int y0, i
         __syncthreads();
 
         // ---------------- B: Korteweg stress of pair q-1 ----------------
-        if (inB && q - 1 >= q0 - (MOM ? 1 : 2)) {
+        if (inB && q - 1 >= q0 - 1 && (MOM || DEV || q < qend)) {
             const v2 *r2 = fld(RHO, sm2), *r1 = fld(RHO, sm1), *r0 = fld(RHO, s0);
             const v2 aW = r2[slot - 1], aC = r2[slot], aE = r2[slot + 1];     // pair q-2
             const v2 bW = r1[slot - 1], bC = r1[slot], bE = r1[slot + 1];     // pair q-1 (centre rows)
