@@ -5,6 +5,7 @@
 #pragma once
 
 #include "fused2d_tile.cuh"
+#include "pdl.cuh"
 
 namespace evlbm {
 namespace fused2d_impl {
@@ -15,6 +16,8 @@ template <int kW, bool THERMAL, bool WALLS, typename ST>
 __global__ void __launch_bounds__(threads_of<kW>(), Shape<kW>::MINB) k_fused2d(FusedArgs A)
 {
     extern __shared__ v2 smem[];
+    pdl_wait();
+    pdl_trigger();
     const int y0 = blockIdx.y * A.H;                       // H is even
     fused_tile<kW, THERMAL, false, WALLS, ST>(A, blockIdx.x, y0, min(A.H, A.ny - y0), blockIdx.z, smem);
 }
@@ -29,6 +32,8 @@ template <int kW, bool THERMAL, bool WALLS, typename ST>
 __global__ void __launch_bounds__(threads_of<kW>(), Shape<kW>::MINB) k_fused2d_bal(FusedArgs A)
 {
     extern __shared__ v2 smem[];
+    pdl_wait();
+    pdl_trigger();
     const int S = (A.nx + kW - 1) / kW, P = (A.ny + 1) / 2;
     const int parts = gridDim.x / S, strip = blockIdx.x % S, part = blockIdx.x / S;
     const long long T = (long long)A.nz * P;                 // row pairs of one strip, all layers
@@ -53,11 +58,12 @@ __global__ void __launch_bounds__(threads_of<kW>(), (kW == 64 ? 6 : 4) - (WALLS 
     k_moments2d(FusedArgs A)
 {
     extern __shared__ v2 smem[];
+    pdl_wait();
     const int y0 = blockIdx.y * A.H;                       // H is even
     fused_tile<kW, THERMAL, false, WALLS, ST, true>(A, blockIdx.x, y0, min(A.H, A.ny - y0), A.z0 + (int)blockIdx.z, smem);
 }
 
-// Chunks of 32 rows at most (16 row pairs after 4 that fill the pipeline), shorter while the
+// Chunks of 32 rows at most (16 row pairs after 2 that fill the pipeline), shorter while the
 // grid would leave SMs without a CTA; narrow strips on narrow lattices.
 template <bool THERMAL, bool WALLS, typename ST>
 cudaError_t launch_moments(FusedArgs A, int nz, cudaStream_t st)
@@ -71,9 +77,9 @@ cudaError_t launch_moments(FusedArgs A, int nz, cudaStream_t st)
         const dim3 grid(S, (A.ny + A.H - 1) / A.H, nz - z < 65535 ? nz - z : 65535);
         FusedArgs B = A;
         B.z0 = z;
-        if (W == 64) k_moments2d<64, THERMAL, WALLS, ST><<<grid, threads_of<64>(), moments_smem_of<64>(), st>>>(B);
-        else k_moments2d<128, THERMAL, WALLS, ST><<<grid, threads_of<128>(), moments_smem_of<128>(), st>>>(B);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e =
+            W == 64 ? launch_pdl(k_moments2d<64, THERMAL, WALLS, ST>, grid, threads_of<64>(), moments_smem_of<64>(), st, B)
+                    : launch_pdl(k_moments2d<128, THERMAL, WALLS, ST>, grid, threads_of<128>(), moments_smem_of<128>(), st, B);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -83,15 +89,16 @@ template <int W, bool THERMAL, bool WALLS, typename ST>
 cudaError_t launch_w(const FusedArgs &A, int nz, bool balanced, cudaStream_t st)
 {
     static bool attr = false;
-    static int resident = 0;
+    static int resident = 0, sms = 0;
     constexpr size_t smem = smem_of<W>();
+    constexpr int most = (int)(smem > kHandoffMax ? smem : kHandoffMax);
     if (!attr) {
         cudaError_t e = cudaFuncSetAttribute(k_fused2d<W, THERMAL, WALLS, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+                                             most);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_fused2d_bal<W, THERMAL, WALLS, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem);
-        int per_sm = 0, dev = 0, sms = 0;
+                                     most);
+        int per_sm = 0, dev = 0;
         if (e == cudaSuccess)
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fused2d_bal<W, THERMAL, WALLS, ST>,
                                                               threads_of<W>(), smem);
@@ -105,12 +112,12 @@ cudaError_t launch_w(const FusedArgs &A, int nz, bool balanced, cudaStream_t st)
     if (balanced) {
         const int S = (A.nx + W - 1) / W;
         const long long parts = min((long long)max(resident / S, 1), (long long)nz * ((A.ny + 1) / 2));
-        k_fused2d_bal<W, THERMAL, WALLS, ST><<<(unsigned)(S * parts), threads_of<W>(), smem, st>>>(A);
-    } else {
-        const dim3 grid((A.nx + W - 1) / W, (A.ny + A.H - 1) / A.H, nz);
-        k_fused2d<W, THERMAL, WALLS, ST><<<grid, threads_of<W>(), smem, st>>>(A);
+        return launch_pdl(k_fused2d_bal<W, THERMAL, WALLS, ST>, dim3((unsigned)(S * parts)), threads_of<W>(),
+                          handoff_smem(smem, S * parts, sms), st, A);
     }
-    return cudaGetLastError();
+    const dim3 grid((A.nx + W - 1) / W, (A.ny + A.H - 1) / A.H, nz);
+    return launch_pdl(k_fused2d<W, THERMAL, WALLS, ST>, grid, threads_of<W>(),
+                      handoff_smem(smem, (long long)grid.x * grid.y * grid.z, sms), st, A);
 }
 
 template <bool THERMAL, bool WALLS, typename ST>

@@ -34,6 +34,7 @@
 #include "bounds.cuh"
 #include "dev16.cuh"
 #include "dispatch.h"
+#include "pdl.cuh"
 #include "tmem.cuh"
 
 namespace evlbm {
@@ -339,9 +340,11 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
 
     // TMEM stash of the tile's pulled f (allocated by warp 0, freed after the last plane).
     __shared__ uint32_t tm_base_sh;
+    pdl_wait();
     if (t < 32) tmem::alloc(&tm_base_sh, TM_COLS);
     tmem::fence_sync();
     const uint32_t tmt = tm_addr(tm_base_sh, t);
+    pdl_trigger();                                        // after the allocation: no later CTA may take its columns
 
     const int qbeg = z0 - 3, qend = zend + 2;
     for (int q = qbeg; q <= qend; ++q) {
@@ -821,6 +824,7 @@ __global__ void __launch_bounds__(MGeo::NT, 3) k_moments3d(const Args<S> A, cons
     constexpr bool DEV = Store<S>::dev;
     constexpr int TX = MGeo::TX, TY = MGeo::TY, NT = MGeo::NT, WA = MGeo::WA, WB = MGeo::WB, SA = MGeo::SA, SB = MGeo::SB;
     __shared__ float RHO[3 * SA], PI[6 * SB];
+    pdl_wait();
     const int t = threadIdx.x, nx = A.nx, ny = A.ny, nz = A.nz;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     const int z0 = (int)blockIdx.z * A.HZ, zend = min(z0 + A.HZ, nz);
@@ -990,8 +994,7 @@ cudaError_t launch(const Args<S> &A, cudaStream_t st)
         attr_dev = dev;
     }
     const dim3 grid((A.nx + G::TX - 1) / G::TX, (A.ny + G::TY - 1) / G::TY, A.nfull + A.ntail);
-    k_fused3d<THERMAL, S><<<grid, G::NT, G::SMEM_BYTES, st>>>(A);
-    return cudaGetLastError();
+    return launch_pdl(k_fused3d<THERMAL, S>, grid, G::NT, G::SMEM_BYTES, st, A);
 }
 
 // z-chunks of at most H planes: chunks of H while more than 2 H planes remain, then the rest
@@ -1110,9 +1113,8 @@ cudaError_t moments_t(const KParams &p, const void *f, const void *g, const void
     while (A.HZ > 2 && (long long)gx * gy * ((p.nz + A.HZ - 1) / A.HZ) < 456) A.HZ >>= 1;
     while ((p.nz + A.HZ - 1) / A.HZ > 65535) A.HZ <<= 1;
     const dim3 grid(gx, gy, (p.nz + A.HZ - 1) / A.HZ);
-    if (p.thermal) k_moments3d<true, S><<<grid, MGeo::NT, 0, st>>>(A, M);
-    else k_moments3d<false, S><<<grid, MGeo::NT, 0, st>>>(A, M);
-    return cudaGetLastError();
+    return p.thermal ? launch_pdl(k_moments3d<true, S>, grid, MGeo::NT, 0, st, A, M)
+                     : launch_pdl(k_moments3d<false, S>, grid, MGeo::NT, 0, st, A, M);
 }
 
 template <typename S>

@@ -13,6 +13,7 @@
 
 #include "common.cuh"
 #include "dev16.cuh"
+#include "pdl.cuh"
 
 namespace evlbm {
 
@@ -186,6 +187,8 @@ template <typename real> struct RefFields {
 template <typename real, typename S, int Q>
 __global__ void k_init(KParams p, const real *rho_in, const real *u_in, const real *RT_in, S *f, S *g, float *Rout)
 {
+    pdl_wait();
+    pdl_trigger();
     Node nd;
     if (!node_of(p, nd)) return;
     constexpr int D = Lat<Q>::D;
@@ -251,6 +254,8 @@ __device__ __forceinline__ void pull_node(const KParams &p, const Node &nd, cons
 template <typename real, typename S, int Q>
 __global__ void k_moments(KParams p, const S *f, const S *g, const float *Rin, RefFields<real> w)
 {
+    pdl_wait();
+    pdl_trigger();
     Node nd;
     if (!node_of(p, nd)) return;
     constexpr int D = Lat<Q>::D;
@@ -291,6 +296,8 @@ __global__ void k_moments(KParams p, const S *f, const S *g, const float *Rin, R
 template <typename real, int Q>
 __global__ void k_stress(KParams p, RefFields<real> w)
 {
+    pdl_wait();
+    pdl_trigger();
     Node nd;
     if (!node_of(p, nd)) return;
     constexpr int D = Lat<Q>::D;
@@ -325,6 +332,8 @@ __global__ void k_stress(KParams p, RefFields<real> w)
 template <typename real, int Q>
 __global__ void k_macro(KParams p, RefFields<real> w)
 {
+    pdl_wait();
+    pdl_trigger();
     Node nd;
     if (!node_of(p, nd)) return;
     constexpr int D = Lat<Q>::D;
@@ -381,6 +390,8 @@ template <typename real, typename S, int Q>
 __global__ void k_collide(KParams p, RefFields<real> w, const S *f_src, const S *g_src, S *f_dst, S *g_dst,
                           const float *Rin, float *Rout)
 {
+    pdl_wait();
+    pdl_trigger();
     Node nd;
     if (!node_of(p, nd)) return;
     if (wall_col(p, nd.x)) return;                       // wall nodes: k_walls

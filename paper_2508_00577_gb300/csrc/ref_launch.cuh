@@ -48,11 +48,9 @@ cudaError_t ref_init_t(const KParams &p, const void *rho, const void *u, const v
                        void *Rout, cudaStream_t st)
 {
     const int B = node_block(p.N);
-    k_init<real, S, Q><<<node_grid(p.N, B), B, 0, st>>>(p, static_cast<const real *>(rho),
-                                                        static_cast<const real *>(u),
-                                                        static_cast<const real *>(RT), static_cast<S *>(f),
-                                                        static_cast<S *>(g), static_cast<float *>(Rout));
-    return cudaGetLastError();
+    return launch_pdl(k_init<real, S, Q>, node_grid(p.N, B), B, 0, st, p, static_cast<const real *>(rho),
+                      static_cast<const real *>(u), static_cast<const real *>(RT), static_cast<S *>(f),
+                      static_cast<S *>(g), static_cast<float *>(Rout));
 }
 
 template <typename real, typename S, int Q>
@@ -62,11 +60,11 @@ cudaError_t ref_macro_t(const KParams &p, void *scratch, const void *RT_iso, con
     const int B = node_block(p.N);
     const dim3 G = node_grid(p.N, B);
     RefFields<real> w = ref_fields<real>(scratch, p.N, RT_iso);
-    k_moments<real, S, Q><<<G, B, 0, st>>>(p, static_cast<const S *>(f), static_cast<const S *>(g),
-                                           static_cast<const float *>(Rin), w);
-    k_stress<real, Q><<<G, B, 0, st>>>(p, w);
-    k_macro<real, Q><<<G, B, 0, st>>>(p, w);
-    return cudaGetLastError();
+    cudaError_t e = launch_pdl(k_moments<real, S, Q>, G, B, 0, st, p, static_cast<const S *>(f),
+                               static_cast<const S *>(g), static_cast<const float *>(Rin), w);
+    if (e == cudaSuccess) e = launch_pdl(k_stress<real, Q>, G, B, 0, st, p, w);
+    if (e == cudaSuccess) e = launch_pdl(k_macro<real, Q>, G, B, 0, st, p, w);
+    return e;
 }
 
 template <typename real, typename S, int Q>
@@ -77,10 +75,10 @@ cudaError_t ref_step_t(const KParams &p, void *scratch, const void *RT_iso, cons
     if (e != cudaSuccess) return e;
     const int B = node_block(p.N);
     RefFields<real> w = ref_fields<real>(scratch, p.N, RT_iso);
-    k_collide<real, S, Q><<<node_grid(p.N, B), B, 0, st>>>(p, w, static_cast<const S *>(f),
-                                                           static_cast<const S *>(g), static_cast<S *>(fo),
-                                                           static_cast<S *>(go), static_cast<const float *>(Rin),
-                                                           static_cast<float *>(Rout));
+    e = launch_pdl(k_collide<real, S, Q>, node_grid(p.N, B), B, 0, st, p, w, static_cast<const S *>(f),
+                   static_cast<const S *>(g), static_cast<S *>(fo), static_cast<S *>(go),
+                   static_cast<const float *>(Rin), static_cast<float *>(Rout));
+    if (e != cudaSuccess) return e;
     if constexpr (!Store<S>::dev) {
         if (p.walls) {
             const long long nw = 2LL * p.ny * p.nz;
