@@ -747,20 +747,33 @@ __global__ void __launch_bounds__(192, 1)
 // row of the pattern.  Each input row then comes from L2 once per CTA (plus two per column
 // walked), and the weights (all 9 C x N of them) stay in shared memory.  The products are
 // accumulated in the same K order as there.
+//
+// Eight channels (the first layer, 16 bytes a pixel, unswizzled): an instruction's K = 16 spans
+// two taps, and the operand's stride along K is the distance between them: a pixel, from the
+// end of a row of taps to the start of the next, and from the last tap to a block of zeros (a
+// pixel times a zero weight would spread infinities).  That stride is unsigned, so the row in
+// slot 0 of the ring is loaded a second time behind the last slot.  The threads lay out the
+// nine taps' weights and the zeros.  On the TMA mainloop a K block took 8 boxes, whose requests bound it: 32 x 256^2 pixels to 32
+// channels 163 -> 95 us.
 template <int C, int N> struct CfgR {
     static constexpr int CB = C < 64 ? C : 64, NB = C / CB;       // channels per box, boxes per row
     static constexpr int RB = CB * 2;                             // bytes of a pixel in a box
     static constexpr int BOX = (130 * RB + 1023) / 1024 * 1024, ROW = NB * BOX;
-    static constexpr int KB = (9 * C + 63) / 64, WBYTES = KB * N * 128;
-    static constexpr int CTAS = N == 32 && C == 32 ? 3 : (N == 64 && C == 64 ? 1 : 2);
-    static constexpr int NR = C == 32 ? (N == 32 ? 5 : 6) : (N == 32 ? 4 : 8);
-    static constexpr int SMEM = WBYTES + NR * ROW + 1024;
+    static constexpr int KB = (9 * C + 63) / 64;
+    static constexpr int WBYTES = C == 8 ? 10 * N * 16 : KB * N * 128;
+    static constexpr int CTAS = C == 8 ? 4 : (N == 32 && C == 32 ? 3 : (N == 64 && C == 64 ? 1 : 2));
+    static constexpr int NR = C <= 32 ? (N == 32 ? 5 : 6) : (N == 32 ? 4 : 8);
+    static constexpr int ZEROS = C == 8 ? 2048 : 0;               // the 128 pixels paired with the last tap
+    static constexpr int SLOTS = C == 8 ? NR + 1 : NR;            // C = 8: slot NR repeats slot 0
+    static constexpr int SMEM = (WBYTES + 1023) / 1024 * 1024 + SLOTS * ROW + ZEROS + 1024;
     static constexpr int EW = N == 32 ? 4 : 8;                    // epilogue warps
     static_assert(CTAS * (SMEM + 2048) <= 232448, "shared memory per SM");
 };
 
 struct RArgs {
     int c0, b_c0;         // first channel of A, first K column of B
+    const bf16 *w;        // B and its row stride (C = 8)
+    int wld;
     int lh, lw;           // image size
     int tiles;            // output rows x columns of 128 pixels, all images
     Epi e;
@@ -798,21 +811,40 @@ __global__ void __launch_bounds__(32 * (CfgR<C, N>::EW + 2), CfgR<C, N>::CTAS)
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
+    const uint32_t wbase = (smem_u32(dsm_raw) + 1023u) & ~1023u, rbase = (wbase + Cf::WBYTES + 1023u) & ~1023u;
+    if constexpr (C == 8) {
+        // Chunk (n, tap) of 8 K, zeros at tap 9: core matrix (tap, n / 8) at (tap N / 8 + n / 8)
+        // 128 B.  Behind the ring the zero pixels.
+        unsigned char *wp = dsm_raw + (wbase - smem_u32(dsm_raw));
+        for (int i = t; i < 10 * N + Cf::ZEROS / 16; i += 32 * (EW + 2)) {
+            uint4 v = make_uint4(0, 0, 0, 0);
+            uint32_t off = rbase - wbase + (uint32_t)(Cf::SLOTS * Cf::ROW + (i - 10 * N) * 16);
+            if (i < 10 * N) {
+                const int tap = i / N, n = i % N;
+                if (tap < 9) v = __ldg(reinterpret_cast<const uint4 *>(g.w + (long long)n * g.wld + g.b_c0 + tap * 8));
+                off = (uint32_t)((tap * (N / 8) + n / 8) * 128 + n % 8 * 16);
+            }
+            *reinterpret_cast<uint4 *>(wp + off) = v;
+        }
+        // Written through the generic proxy, read through the async proxy.
+        asm volatile("fence.proxy.async.shared::cta;");
+    }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_sh;
-    const uint32_t wbase = (smem_u32(dsm_raw) + 1023u) & ~1023u, rbase = wbase + Cf::WBYTES;
 
     if (warp == EW) {
         if (lane == 0) {
             // ---------------- TMA producer: the weights, then the input rows ----------------
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&wbar)),
-                         "r"((uint32_t)Cf::WBYTES));
-            for (int kb = 0; kb < Cf::KB; ++kb)
-                tma_load_2d(wbase + (uint32_t)(kb * N * 128), &tmB, g.b_c0 + kb * 64, 0, smem_u32(&wbar));
+            if constexpr (C != 8) {
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&wbar)),
+                             "r"((uint32_t)Cf::WBYTES));
+                for (int kb = 0; kb < Cf::KB; ++kb)
+                    tma_load_2d(wbase + (uint32_t)(kb * N * 128), &tmB, g.b_c0 + kb * 64, 0, smem_u32(&wbar));
+            }
             int r = 0;                                            // rows loaded so far
             bool ok = true;
             for (int i = t0; i < t1 && ok; ++i) {
@@ -827,7 +859,9 @@ __global__ void __launch_bounds__(32 * (CfgR<C, N>::EW + 2), CfgR<C, N>::CTAS)
                         break;
                     }
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&full[s])),
-                                 "r"((uint32_t)(Cf::NB * 130 * Cf::RB)));
+                                 "r"((uint32_t)(Cf::NB * 130 * Cf::RB) << (C == 8 && s == 0 ? 1 : 0)));
+                    if (C == 8 && s == 0)
+                        tma_load_4d(rbase + (uint32_t)(NR * Cf::ROW), &tmA, g.c0, x0, yy, b, smem_u32(&full[0]));
 #pragma unroll
                     for (int j = 0; j < Cf::NB; ++j)
                         tma_load_4d(rbase + (uint32_t)(s * Cf::ROW + j * Cf::BOX), &tmA, g.c0 + j * Cf::CB, x0, yy, b,
@@ -836,14 +870,14 @@ __global__ void __launch_bounds__(32 * (CfgR<C, N>::EW + 2), CfgR<C, N>::CTAS)
             }
             // No copy may be in flight when the CTA ends (after a wait gave up, rows that no
             // MMA waited for).
-            mbar_wait(smem_u32(&wbar), 0);
+            if (C != 8) mbar_wait(smem_u32(&wbar), 0);
             for (int k = r > NR ? r - NR : 0; k < r; ++k) mbar_wait(smem_u32(&full[k % NR]), (uint32_t)((k / NR) & 1));
         }
     } else if (warp == EW + 1) {
         if (lane == 0) {
             // ---------------- MMA issuer ----------------
             const uint32_t idesc = make_idesc(N, false, false);
-            bool ok = t1 <= t0 || mbar_wait(smem_u32(&wbar), 0, abort_v);
+            bool ok = C == 8 || t1 <= t0 || mbar_wait(smem_u32(&wbar), 0, abort_v);
             if (!ok) *abort_v = 1;
             int top = 0, have = 0, lt = 0;                        // ring index of row y - 1, rows waited for
             for (int i = t0; i < t1 && ok; ++i, ++lt) {
@@ -863,6 +897,22 @@ __global__ void __launch_bounds__(32 * (CfgR<C, N>::EW + 2), CfgR<C, N>::CTAS)
 #pragma unroll 1
                 for (int dy = 0; dy < 3; ++dy) {
                     const uint32_t ra = rbase + (uint32_t)((top + dy) % NR * Cf::ROW);
+                    if constexpr (C == 8) {
+                        // Taps (0, 1), (2, 3), (4, 5), (6, 7), (8, zeros).
+                        auto taps = [&](int k, uint32_t a, uint32_t stride) {
+                            mma_bf16(acc_t, smem_desc(a, stride, 128), smem_desc(wbase + (uint32_t)(k * N * 16), N * 16, 128),
+                                     idesc, k > 0 ? 1u : 0u);
+                        };
+                        if (dy == 0) {
+                            taps(0, ra, 16);
+                            taps(2, ra + 32, Cf::ROW - 32);       // the next row: the next slot
+                        } else if (dy == 1) {
+                            taps(4, ra + 16, 16);
+                        } else {
+                            taps(6, ra, 16);
+                            taps(8, ra + 32, rbase + (uint32_t)(Cf::SLOTS * Cf::ROW) - (ra + 32));
+                        }
+                    } else
 #pragma unroll
                     for (int dx = 0; dx < 3; ++dx)
 #pragma unroll
@@ -1362,7 +1412,7 @@ bool tma_eligible(const sur_gemm_args &a)
 bool rows_eligible(const sur_gemm_args &a)
 {
     if (a.a.kind != SUR_OP_CONV3 || a.a.W < 128 || a.K != (9 * a.a.C + 63) / 64 * 64 || a.M != a.a.rows) return false;
-    return (a.a.C == 32 || a.a.C == 64) && (a.N == 32 || a.N == 64);
+    return ((a.a.C == 32 || a.a.C == 64) && (a.N == 32 || a.N == 64)) || (a.a.C == 8 && a.N == 32);
 }
 
 template <int C, int N>
@@ -1380,7 +1430,8 @@ int launch_rows(const sur_gemm_args &a, const Epi &e, cudaStream_t st)
                              (cuuint64_t)(H + 2) * (W + 2) * a.a.ld * e2};
     cuuint32_t box[4] = {(cuuint32_t)Cf::CB, 130, 1, 1}, es[4] = {1, 1, 1, 1};
     if (enc(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(a.a.p), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, Cf::CB == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE,
+            C == 8 ? CU_TENSOR_MAP_SWIZZLE_NONE : (Cf::CB == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B),
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return -1;
     cuuint64_t bdims[2] = {(cuuint64_t)a.b.ld, (cuuint64_t)a.b.rows}, bstr[1] = {a.b.ld * e2};
@@ -1401,6 +1452,8 @@ int launch_rows(const sur_gemm_args &a, const Epi &e, cudaStream_t st)
     RArgs g;
     g.c0 = a.a.c0;
     g.b_c0 = a.b.c0;
+    g.w = static_cast<const bf16 *>(a.b.p);
+    g.wld = a.b.ld;
     g.lh = ilog2(H);
     g.lw = ilog2(W);
     g.tiles = a.M / 128;
@@ -1550,8 +1603,9 @@ int gemm(const sur_gemm_args &a, int *status, cudaStream_t st)
         }
     }
     if (tma_eligible(a) && rows_eligible(a)) {
-        const int rc = a.a.C == 32 ? (a.N == 32 ? launch_rows<32, 32>(a, e, st) : launch_rows<32, 64>(a, e, st))
-                                   : (a.N == 32 ? launch_rows<64, 32>(a, e, st) : launch_rows<64, 64>(a, e, st));
+        const int rc = a.a.C == 8    ? launch_rows<8, 32>(a, e, st)
+                       : a.a.C == 32 ? (a.N == 32 ? launch_rows<32, 32>(a, e, st) : launch_rows<32, 64>(a, e, st))
+                                     : (a.N == 32 ? launch_rows<64, 32>(a, e, st) : launch_rows<64, 64>(a, e, st));
         if (rc >= 0) return rc;                // -1: a tensor map was refused
     }
     if (tma_eligible(a)) {
