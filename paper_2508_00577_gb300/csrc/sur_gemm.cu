@@ -20,6 +20,7 @@
 #include <cudaTypedefs.h>
 #include <stdint.h>
 
+#include "pdl.cuh"
 #include "surrogate.cuh"
 
 namespace evsur {
@@ -374,6 +375,8 @@ __global__ void __launch_bounds__(160, 1) k_gemm_cpasync(const KArgs g)
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
+    evlbm::pdl_wait();
+    evlbm::pdl_trigger();                          // tensor memory is allocated: no later CTA may take it
     const uint32_t tmem = tmem_sh;
     const uint32_t sbase = smem_u32(dsm);
 
@@ -568,6 +571,8 @@ __global__ void __launch_bounds__(192, 1)
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
+    evlbm::pdl_wait();
+    evlbm::pdl_trigger();                          // tensor memory is allocated: no later CTA may take it
     const uint32_t tmem = tmem_sh;
     const uint32_t sbase = (smem_u32(dsm_raw) + 1023u) & ~1023u;   // swizzle atoms need 1024-byte alignment
 
@@ -813,6 +818,7 @@ __global__ void __launch_bounds__(32 * (CfgR<C, N>::EW + 2), CfgR<C, N>::CTAS)
     }
     const uint32_t wbase = (smem_u32(dsm_raw) + 1023u) & ~1023u, rbase = (wbase + Cf::WBYTES + 1023u) & ~1023u;
     if constexpr (C == 8) {
+        evlbm::pdl_wait();                         // the weights
         // Chunk (n, tap) of 8 K, zeros at tap 9: core matrix (tap, n / 8) at (tap N / 8 + n / 8)
         // 128 B.  Behind the ring the zero pixels.
         unsigned char *wp = dsm_raw + (wbase - smem_u32(dsm_raw));
@@ -832,6 +838,8 @@ __global__ void __launch_bounds__(32 * (CfgR<C, N>::EW + 2), CfgR<C, N>::CTAS)
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
+    evlbm::pdl_wait();
+    evlbm::pdl_trigger();                          // tensor memory is allocated: no later CTA may take it
     const uint32_t tmem = tmem_sh;
 
     if (warp == EW) {
@@ -1027,6 +1035,8 @@ __global__ void __launch_bounds__(192, CfgW<CB, N>::CTAS)
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
+    evlbm::pdl_wait();
+    evlbm::pdl_trigger();                          // tensor memory is allocated: no later CTA may take it
     const uint32_t tmem = tmem_sh;
     const uint32_t xbase = (smem_u32(dsm_raw) + 1023u) & ~1023u, zbase = xbase + (uint32_t)(NX * Cf::XROW);
 
@@ -1212,8 +1222,7 @@ cudaError_t launch_cpasync(const KArgs &g, long long mtiles, int splits, cudaStr
     cudaError_t e = set_smem(k_gemm_cpasync<BN>, CfgA<BN>::SMEM, attr_dev);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)mtiles, (unsigned)(g.e.N / BN), (unsigned)splits);
-    k_gemm_cpasync<BN><<<grid, 160, CfgA<BN>::SMEM, st>>>(g);
-    return cudaGetLastError();
+    return evlbm::launch_pdl(k_gemm_cpasync<BN>, grid, 160, CfgA<BN>::SMEM, st, g);
 }
 
 template <int BN, int ASW, bool MN = false>
@@ -1233,8 +1242,7 @@ cudaError_t launch_tma(const CUtensorMap &ma, const CUtensorMap &mb, const TArgs
     gg.ntiles = g.e.N / BN;
     const long long tiles = (long long)gg.mtiles * gg.ntiles * (MN ? gg.splits : 1);
     const long long ctas = tiles < 2LL * sms ? tiles : 2LL * sms;   // two resident CTAs per SM
-    k_gemm_tma<BN, ASW, MN><<<(unsigned)ctas, 192, CfgT<BN>::SMEM, st>>>(ma, mb, gg);
-    return cudaGetLastError();
+    return evlbm::launch_pdl(k_gemm_tma<BN, ASW, MN>, (unsigned)ctas, 192, CfgT<BN>::SMEM, st, ma, mb, gg);
 }
 
 template <int ASW>
@@ -1461,8 +1469,8 @@ int launch_rows(const sur_gemm_args &a, const Epi &e, cudaStream_t st)
     // At least 8 rows a CTA, so that the two rows it loads beyond its own stay a small part.
     int ctas = Cf::CTAS * sms;
     if (g.tiles / 8 < ctas) ctas = g.tiles / 8 > 0 ? g.tiles / 8 : 1;
-    k_conv_rows<C, N><<<ctas, 32 * (Cf::EW + 2), Cf::SMEM, st>>>(ma, mb, g);
-    return cudaGetLastError() == cudaSuccess ? SUR_OK : SUR_ECUDA;
+    err = evlbm::launch_pdl(k_conv_rows<C, N>, ctas, 32 * (Cf::EW + 2), Cf::SMEM, st, ma, mb, g);
+    return err == cudaSuccess ? SUR_OK : SUR_ECUDA;
 }
 
 // Row-marching weight gradient: eligible shapes (of those tma_mn_eligible accepts) are whole
@@ -1521,8 +1529,8 @@ int launch_wgrad(const sur_gemm_args &a, int *status, cudaStream_t st)
     int ctas = Cf::CTAS * sms / parts;
     if (g.tiles / 8 < ctas) ctas = g.tiles / 8;
     if (ctas < 1) ctas = 1;
-    k_wgrad_rows<CB, N><<<dim3(ctas, parts), 192, Cf::SMEM, st>>>(mx, mz, g);
-    return cudaGetLastError() == cudaSuccess ? SUR_OK : SUR_ECUDA;
+    const cudaError_t err = evlbm::launch_pdl(k_wgrad_rows<CB, N>, dim3(ctas, parts), 192, Cf::SMEM, st, mx, mz, g);
+    return err == cudaSuccess ? SUR_OK : SUR_ECUDA;
 }
 
 }  // namespace

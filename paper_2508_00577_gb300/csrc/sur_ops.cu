@@ -4,12 +4,17 @@
 // gradients or the state update, the loss terms and first-layer input gradient of
 // unrolled training, Adam, the BF16 operand copies of the weights, and the per-domain
 // fallback indicators.  The kernels over activations are bound by HBM: 16-byte accesses,
-// consecutive threads on consecutive bytes, pixel indices by shifts.
+// consecutive threads on consecutive bytes, pixel indices by shifts.  The kernels of a pass are
+// dependent launches (pdl.cuh): a training step has 80 of them, 2612 -> 2503 us at 16 x 256^2,
+// and a window of 32 x 256^2 1319 -> 1303 us.
 #include <stdint.h>
 
+#include "pdl.cuh"
 #include "surrogate.cuh"
 
 namespace evsur {
+
+using evlbm::launch_pdl;
 
 namespace {
 
@@ -79,6 +84,8 @@ template <bool POOL>
 __global__ void __launch_bounds__(256, POOL ? 4 : 5) k_silu_bwd(const bf16 *dY, int ldd, const bf16 *dP, const bf16 *Z, long long M,
                                                   int lh, int lw, int c8s, bf16 *dZ, float *dbias)
 {
+    evlbm::pdl_wait();
+    evlbm::pdl_trigger();
     const int C8 = 1 << c8s, C = C8 << 3;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     GRID_STRIDE(e, M << c8s)
@@ -123,6 +130,8 @@ __global__ void __launch_bounds__(256, POOL ? 4 : 5) k_silu_bwd(const bf16 *dY, 
 __global__ void __launch_bounds__(256) k_colsum(const bf16 *X, int ldx, long long M, int lh, int lw, int c8s,
                                                 float *out)
 {
+    evlbm::pdl_wait();
+    evlbm::pdl_trigger();
     const int C8 = 1 << c8s;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
@@ -143,6 +152,8 @@ __global__ void __launch_bounds__(256) k_colsum(const bf16 *X, int ldx, long lon
 // 2-byte accesses, took 46 us at 2^18 coarse pixels x 32 channels).
 __global__ void __launch_bounds__(256) k_pool2(const bf16 *X, int ldx, long long Mc, int lh, int lw, int c8s, bf16 *Y)
 {
+    evlbm::pdl_wait();
+    evlbm::pdl_trigger();
     const int Wf2 = 2 * (1 << lw) + 2, C8 = 1 << c8s, C = C8 << 3;
     GRID_STRIDE(e, Mc << c8s)
     {
@@ -172,6 +183,8 @@ __global__ void __launch_bounds__(256) k_pool2(const bf16 *X, int ldx, long long
 // channels 4..7 zero.
 __global__ void k_pack_in(const float *x, long long M, int lh, int lw, const float *norm, bf16 *X)
 {
+    evlbm::pdl_wait();
+    evlbm::pdl_trigger();
     GRID_STRIDE(m, M)
     {
         float v[8];
@@ -205,6 +218,8 @@ __global__ void __launch_bounds__(256) k_head(const bf16 *Y, long long M, int lh
                                               const float *dO, float *loss, float *xn, bf16 *dY, float *dWh,
                                               float *dbh)
 {
+    evlbm::pdl_wait();
+    evlbm::pdl_trigger();
     __shared__ uint4 sy[256 * 5];
     __shared__ float w[4 * 32];
     __shared__ float4 sd[MODE == kHeadNext ? 1 : 256];
@@ -333,6 +348,8 @@ __global__ void __launch_bounds__(256) k_head(const bf16 *Y, long long M, int lh
 __global__ void k_unroll_term(const float *xp, const float *yt, long long M, const float *norm, float inv, float *G,
                               float *dO, float *loss)
 {
+    evlbm::pdl_wait();
+    evlbm::pdl_trigger();
     __shared__ float red[256];
     float acc = 0.f;
     GRID_STRIDE(m, M)
@@ -365,6 +382,8 @@ __global__ void k_unroll_term(const float *xp, const float *yt, long long M, con
 __global__ void k_conv0_dx(const bf16 *dZ, const bf16 *Wb, int Kp, long long M, int lh, int lw, const float *norm,
                            float *G)
 {
+    evlbm::pdl_wait();
+    evlbm::pdl_trigger();
     __shared__ float w[9][32][4];
     for (int e = threadIdx.x; e < 9 * 32 * 4; e += blockDim.x) {
         const int tap = e / 128, co = (e / 4) % 32, c = e % 4;
@@ -401,6 +420,8 @@ __global__ void k_conv0_dx(const bf16 *dZ, const bf16 *Wb, int Kp, long long M, 
 __global__ void k_adam(float *w, const float *gr, float *m, float *v, long long n, float lr, float b1, float b2,
                        float eps, float c1, float c2)
 {
+    evlbm::pdl_wait();
+    evlbm::pdl_trigger();
     GRID_STRIDE(i, n)
     {
         const float g = gr[i];
@@ -427,6 +448,8 @@ struct WeightTab {
 };
 __global__ void __launch_bounds__(256) k_weights(const __grid_constant__ WeightTab tab)
 {
+    evlbm::pdl_wait();
+    evlbm::pdl_trigger();
     int j = 0;
     while (j + 1 < 2 * tab.n && (int)blockIdx.x >= tab.first[j + 1]) ++j;
     const WeightCopy &w = tab.L[j >> 1];
@@ -532,78 +555,68 @@ cudaError_t silu_bwd(const bf16 *dY, int ldd, const bf16 *dP, const bf16 *Z, lon
     const int s = log2i(C >> 3);
     if (C != 8 << s || C > 256) return cudaErrorInvalidValue;
     const int g = grid_res(M << s, dP ? 4 : 5);
-    if (dP) k_silu_bwd<true><<<g, 256, 0, st>>>(dY, ldd, dP, Z, M, lh, lw, s, dZ, dbias);
-    else k_silu_bwd<false><<<g, 256, 0, st>>>(dY, ldd, dP, Z, M, lh, lw, s, dZ, dbias);
-    return cudaGetLastError();
+    if (dP) return launch_pdl(k_silu_bwd<true>, g, 256, 0, st, dY, ldd, dP, Z, M, lh, lw, s, dZ, dbias);
+    return launch_pdl(k_silu_bwd<false>, g, 256, 0, st, dY, ldd, dP, Z, M, lh, lw, s, dZ, dbias);
 }
 
 cudaError_t colsum(const bf16 *X, int ldx, long long M, int lh, int lw, int C, float *out, cudaStream_t st)
 {
     const int s = log2i(C >> 3);
     if (C != 8 << s || C > 256 || ldx % 8 || (reinterpret_cast<uintptr_t>(X) & 15)) return cudaErrorInvalidValue;
-    k_colsum<<<grid_res(M << s, 6), 256, 0, st>>>(X, ldx, M, lh, lw, s, out);
-    return cudaGetLastError();
+    return launch_pdl(k_colsum, grid_res(M << s, 6), 256, 0, st, X, ldx, M, lh, lw, s, out);
 }
 
 cudaError_t pool2(const bf16 *X, int ldx, long long Mc, int lh, int lw, int C, bf16 *Y, cudaStream_t st)
 {
     const int s = log2i(C >> 3);
     if (C != 8 << s || ldx % 8 || (reinterpret_cast<uintptr_t>(X) & 15)) return cudaErrorInvalidValue;
-    k_pool2<<<grid_1d(Mc << s), 256, 0, st>>>(X, ldx, Mc, lh, lw, s, Y);
-    return cudaGetLastError();
+    return launch_pdl(k_pool2, grid_1d(Mc << s), 256, 0, st, X, ldx, Mc, lh, lw, s, Y);
 }
 
 cudaError_t pack_in(const float *x, long long M, int lh, int lw, const float *norm, bf16 *X, cudaStream_t st)
 {
-    k_pack_in<<<grid_1d(M), 256, 0, st>>>(x, M, lh, lw, norm, X);
-    return cudaGetLastError();
+    return launch_pdl(k_pack_in, grid_1d(M), 256, 0, st, x, M, lh, lw, norm, X);
 }
 
 cudaError_t head_next(const bf16 *Y, long long M, int lh, int lw, const float *Wh, const float *bh, const float *norm,
                       const float *x, float *xn, cudaStream_t st)
 {
-    k_head<kHeadNext><<<grid_res(M, 5), 256, 0, st>>>(Y, M, lh, lw, Wh, bh, norm, x, nullptr, nullptr, nullptr, xn,
-                                                   nullptr, nullptr, nullptr);
-    return cudaGetLastError();
+    return launch_pdl(k_head<kHeadNext>, grid_res(M, 5), 256, 0, st, Y, M, lh, lw, Wh, bh, norm, x, nullptr, nullptr,
+                      nullptr, xn, nullptr, nullptr, nullptr);
 }
 
 cudaError_t head_loss_bwd(const bf16 *Y, long long M, int lh, int lw, const float *Wh, const float *bh,
                           const float *norm, const float *x, const float *yt, float *loss, bf16 *dY, float *dWh,
                           float *dbh, cudaStream_t st)
 {
-    k_head<kHeadLoss><<<grid_res(M, 3), 256, 0, st>>>(Y, M, lh, lw, Wh, bh, norm, x, yt, nullptr, loss, nullptr, dY, dWh,
-                                                   dbh);
-    return cudaGetLastError();
+    return launch_pdl(k_head<kHeadLoss>, grid_res(M, 3), 256, 0, st, Y, M, lh, lw, Wh, bh, norm, x, yt, nullptr, loss,
+                      nullptr, dY, dWh, dbh);
 }
 
 cudaError_t head_bwd(const bf16 *Y, long long M, int lh, int lw, const float *Wh, const float *dO, bf16 *dY,
                      float *dWh, float *dbh, cudaStream_t st)
 {
-    k_head<kHeadBwd><<<grid_res(M, 6), 256, 0, st>>>(Y, M, lh, lw, Wh, nullptr, nullptr, nullptr, nullptr, dO, nullptr,
-                                                  nullptr, dY, dWh, dbh);
-    return cudaGetLastError();
+    return launch_pdl(k_head<kHeadBwd>, grid_res(M, 6), 256, 0, st, Y, M, lh, lw, Wh, nullptr, nullptr, nullptr, nullptr,
+                      dO, nullptr, nullptr, dY, dWh, dbh);
 }
 
 cudaError_t unroll_term(const float *xp, const float *yt, long long M, const float *norm, float inv, float *G, float *dO,
                         float *loss, cudaStream_t st)
 {
-    k_unroll_term<<<grid_1d(M), 256, 0, st>>>(xp, yt, M, norm, inv, G, dO, loss);
-    return cudaGetLastError();
+    return launch_pdl(k_unroll_term, grid_1d(M), 256, 0, st, xp, yt, M, norm, inv, G, dO, loss);
 }
 
 cudaError_t conv0_dx(const bf16 *dZ, const bf16 *Wb, int Kp, long long M, int lh, int lw, const float *norm, float *G,
                      cudaStream_t st)
 {
     if (Kp < 72 || (reinterpret_cast<uintptr_t>(dZ) & 15)) return cudaErrorInvalidValue;
-    k_conv0_dx<<<grid_1d(M), 256, 0, st>>>(dZ, Wb, Kp, M, lh, lw, norm, G);
-    return cudaGetLastError();
+    return launch_pdl(k_conv0_dx, grid_1d(M), 256, 0, st, dZ, Wb, Kp, M, lh, lw, norm, G);
 }
 
 cudaError_t adam(float *w, const float *g, float *m, float *v, long long n, float lr, float b1, float b2, float eps,
                  float c1, float c2, cudaStream_t st)
 {
-    k_adam<<<grid_1d(n), 256, 0, st>>>(w, g, m, v, n, lr, b1, b2, eps, c1, c2);
-    return cudaGetLastError();
+    return launch_pdl(k_adam, grid_1d(n), 256, 0, st, w, g, m, v, n, lr, b1, b2, eps, c1, c2);
 }
 
 cudaError_t copy_weights(const WeightCopy *layers, int n, cudaStream_t st)
@@ -621,8 +634,7 @@ cudaError_t copy_weights(const WeightCopy *layers, int n, cudaStream_t st)
         blocks += (adj + kWeightChunk - 1) / kWeightChunk;
     }
     tab.first[2 * n] = blocks;
-    k_weights<<<blocks, 256, 0, st>>>(tab);
-    return cudaGetLastError();
+    return launch_pdl(k_weights, blocks, 256, 0, st, tab);
 }
 
 cudaError_t indicators(const float *F, int batch, long long Mb, float rho_mid, double *out, int *invalid,
