@@ -105,18 +105,39 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float v[32])
     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
 }
 
-template <int BN>
+// 16 columns, as above.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16])
+{
+    uint32_t r[16];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;");
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+}
+
+struct NoOp {
+    __device__ void operator()() const {}
+};
+
+// Columns cbeg .. cend - 1 of the 32 rows of lane quarter `warp`.  drained() runs once the
+// warp's accumulator columns are in registers: the next tile's instructions may overwrite them
+// while the values here are still worked on.
+// CS columns (32, or 16 with fewer registers) are worked on at a time.
+template <int BN, int CS = 32, class D = NoOp>
 __device__ __forceinline__ void epilogue(const Epi &g, uint32_t tmem, long long m0, int n0, int warp, int lane,
-                                         int cbeg = 0, int cend = BN)
+                                         int cbeg = 0, int cend = BN, D drained = D())
 {
     const long long row = m0 + warp * 32 + lane;
     const bool rv = row < g.M;
     const long long orow = rv && g.pix ? pad_pix(row, g.lh, g.lw) : row;
-    // 32 consecutive bias values, as 16-byte loads where the array allows it.
-    auto add_bias = [&](float v[32], const float *b) {
+    // CS consecutive bias values, as 16-byte loads where the array allows it.
+    auto add_bias = [&](float v[CS], const float *b) {
         if ((reinterpret_cast<uintptr_t>(b) & 15) == 0) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
+            for (int j = 0; j < CS / 4; ++j) {
                 const float4 q = __ldg(reinterpret_cast<const float4 *>(b) + j);
                 v[4 * j] += q.x;
                 v[4 * j + 1] += q.y;
@@ -125,23 +146,25 @@ __device__ __forceinline__ void epilogue(const Epi &g, uint32_t tmem, long long 
             }
         } else {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] += __ldg(b + j);
+            for (int j = 0; j < CS; ++j) v[j] += __ldg(b + j);
         }
     };
 #pragma unroll 1
-    for (int c0 = cbeg; c0 < cend; c0 += 32) {
-        float v[32];
-        tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + c0, v);
+    for (int c0 = cbeg; c0 < cend; c0 += CS) {
+        float v[CS];
+        if constexpr (CS == 32) tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + c0, v);
+        else tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + c0, v);
+        if (c0 + CS >= cend) drained();
         if (!rv) continue;
         const int col = n0 + c0;
         if (g.epi == SUR_EPI_F32_ATOMIC) {
             float *o = static_cast<float *>(g.out) + row * g.ldo + g.co0 + col;
             if ((reinterpret_cast<uintptr_t>(o) & 15) == 0) {
 #pragma unroll
-                for (int j = 0; j < 32; j += 4) red_add4(o + j, v[j], v[j + 1], v[j + 2], v[j + 3]);
+                for (int j = 0; j < CS; j += 4) red_add4(o + j, v[j], v[j + 1], v[j + 2], v[j + 3]);
             } else {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) atomicAdd(o + j, v[j]);
+                for (int j = 0; j < CS; ++j) atomicAdd(o + j, v[j]);
             }
         } else if (g.epi == SUR_EPI_SHUF) {
             const int sidx = col / g.shuf_cout, c = col - sidx * g.shuf_cout;
@@ -152,28 +175,35 @@ __device__ __forceinline__ void epilogue(const Epi &g, uint32_t tmem, long long 
             const int y = (int)((row >> g.lw) & (Hc - 1)), x = (int)(row & (Wc - 1));
             const long long qf = ((b * 2 * Hc + 2 * y + (sidx >> 1)) << (g.lw + 1)) | (2 * x + (sidx & 1));
             for_halo(qf, g.lh + 1, g.lw + 1,
-                     [&](long long t) { store32_bf16(g.y + t * g.ldy + g.cy0 + c, v); });
+                     [&](long long t) { store_bf16<CS>(g.y + t * g.ldy + g.cy0 + c, v); });
         } else {
             if (g.bias) add_bias(v, g.bias + col);
             if (g.epi == SUR_EPI_F32) {
                 float4 *o = reinterpret_cast<float4 *>(static_cast<float *>(g.out) + orow * g.ldo + g.co0 + col);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) o[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                for (int j = 0; j < CS / 4; ++j) o[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             } else {
-                if (g.out) store32_bf16(static_cast<bf16 *>(g.out) + orow * g.ldo + g.co0 + col, v);
+                if (g.out) store_bf16<CS>(static_cast<bf16 *>(g.out) + orow * g.ldo + g.co0 + col, v);
                 if (g.epi == SUR_EPI_CONV) {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] = silu(v[j]);
+                    for (int j = 0; j < CS; ++j) v[j] = silu(v[j]);
                     if (g.pix) {
                         for_halo(row, g.lh, g.lw,
-                                 [&](long long t) { store32_bf16(g.y + t * g.ldy + g.cy0 + col, v); });
+                                 [&](long long t) { store_bf16<CS>(g.y + t * g.ldy + g.cy0 + col, v); });
                     } else {
-                        store32_bf16(g.y + row * g.ldy + g.cy0 + col, v);
+                        store_bf16<CS>(g.y + row * g.ldy + g.cy0 + col, v);
                     }
                 }
             }
         }
     }
+}
+
+// This thread's arrival on the barrier of a drained accumulator.
+__device__ __forceinline__ void arrive_drained(uint64_t *bar)
+{
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 template <int BN> struct Tmem {
@@ -456,6 +486,8 @@ struct TArgs {
     Epi e;
 };
 
+template <int BN, bool MN> constexpr int kEpiWarps = !MN && BN >= 64 ? 8 : 4;
+
 template <int BN> struct CfgT {
     // Two CTAs per SM: 97-101 KB of stages each.
     static constexpr int NS = BN == 128 ? 3 : (BN == 64 ? 4 : 5);
@@ -498,10 +530,14 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
 // swizzle).  Each CTA walks tiles blockIdx.x, blockIdx.x + gridDim.x, ... with
 // two TMEM accumulators, so the epilogue of one tile overlaps the mainloop of
 // the next.
-//   warp 4 (one thread): TMA producer        full[s]   <- expect_tx + TMA bytes
-//   warp 5 (one thread): MMA issuer          empty[s]  <- tcgen05.commit
-//   warps 0-3: epilogue                      tfull[b]  <- tcgen05.commit (accumulator b ready)
-//                                            tempty[b] <- 128 epilogue arrivals (b drained)
+//   warp EW (one thread): TMA producer       full[s]   <- expect_tx + TMA bytes
+//   warp EW + 1 (one thread): MMA issuer     empty[s]  <- tcgen05.commit
+//   warps 0 .. EW - 1: epilogue              tfull[b]  <- tcgen05.commit (accumulator b ready)
+//                                            tempty[b] <- 32 EW epilogue arrivals (b drained)
+// Tiles of 64 and 128 columns have EW = 8 epilogue warps, each half the columns (the weight
+// gradients, which only add their sums once, 4), and a warp releases its accumulator as soon as
+// it holds the values: with 4, which released it after the stores, 64 -> 128 channels at
+// 32 x 64^2 took 39.7 us, now 34.3; 128 -> 128, bound by the operands' L2 reads, the same.
 // Tile of the persistent loop: output block (m0, n0) and its K range.  MN-major mode
 // orders tiles (split, m, n), n fastest, so that tiles over the same pixels run together.
 struct TileCoord {
@@ -537,7 +573,7 @@ __device__ __forceinline__ TileCoord tile_coord(const TArgs &g, int tile)
 // swizzled MN-major layouts take LBO = stride between MN atoms and SBO = stride between
 // 8-row K groups; the unswizzled one LBO = K-group stride and SBO = MN stride.
 template <int BN, int ASW, bool MN>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(32 * (kEpiWarps<BN, MN> + 2), kEpiWarps<BN, MN> == 8 ? 2 : 1)
     k_gemm_tma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TArgs g)
 {
     using Cf = CfgT<BN>;
@@ -546,6 +582,7 @@ __global__ void __launch_bounds__(192, 1)
     constexpr int NBOX = 64 / CB;             // A boxes per K block
     constexpr int BOXB = BM * ASW;            // bytes per A box
     constexpr int TCOLS = 2 * BN < 32 ? 32 : 2 * BN;
+    constexpr int EW = kEpiWarps<BN, MN>, CW = BN * 4 / EW;   // epilogue warps, columns of each
     extern __shared__ unsigned char dsm_raw[];
     __shared__ __align__(8) uint64_t full[NS], empty[NS], tfull[2], tempty[2], done_bar;
     __shared__ uint32_t tmem_sh;
@@ -562,7 +599,7 @@ __global__ void __launch_bounds__(192, 1)
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&tfull[b]), 1);
-            mbar_init(smem_u32(&tempty[b]), 128);
+            mbar_init(smem_u32(&tempty[b]), 32 * EW);
         }
         mbar_init(smem_u32(&done_bar), 1);
         abort_flag = 0;
@@ -576,7 +613,7 @@ __global__ void __launch_bounds__(192, 1)
     const uint32_t tmem = tmem_sh;
     const uint32_t sbase = (smem_u32(dsm_raw) + 1023u) & ~1023u;   // swizzle atoms need 1024-byte alignment
 
-    if (warp == 4) {
+    if (warp == EW) {
         if (lane == 0) {
             // ---------------- TMA producer ----------------
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
@@ -668,7 +705,7 @@ __global__ void __launch_bounds__(192, 1)
                 }
             }
         }
-    } else if (warp == 5) {
+    } else if (warp == EW + 1) {
         if (lane == 0) {
             // ---------------- MMA issuer ----------------
             const uint32_t idesc = make_idesc(BN, MN, MN);
@@ -715,7 +752,7 @@ __global__ void __launch_bounds__(192, 1)
             mma_commit(smem_u32(&done_bar));   // arrives once every MMA above completed
         }
     } else {
-        // ---------------- epilogue (warps 0-3) ----------------
+        // ---------------- epilogue (lane quarter warp % 4, column half warp / 4) ----------------
         int lt = 0;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++lt) {
             const int buf = lt & 1;
@@ -726,9 +763,8 @@ __global__ void __launch_bounds__(192, 1)
                 break;
             }
             const TileCoord tc = tile_coord<MN>(g, tile);
-            epilogue<BN>(g.e, tmem + (uint32_t)(buf * BN), tc.m0, tc.n0 * BN, warp, lane);
-            asm volatile("tcgen05.fence::before_thread_sync;");
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[buf])));
+            epilogue<BN>(g.e, tmem + (uint32_t)(buf * BN), tc.m0, tc.n0 * BN, warp & 3, lane, (warp >> 2) * CW,
+                         (warp >> 2) * CW + CW, [&] { arrive_drained(&tempty[buf]); });
         }
         // Tensor memory must be idle before it is freed.
         if (!mbar_wait(smem_u32(&done_bar), 0)) *abort_v = 1;
@@ -766,12 +802,17 @@ template <int C, int N> struct CfgR {
     static constexpr int BOX = (130 * RB + 1023) / 1024 * 1024, ROW = NB * BOX;
     static constexpr int KB = (9 * C + 63) / 64;
     static constexpr int WBYTES = C == 8 ? 10 * N * 16 : KB * N * 128;
-    static constexpr int CTAS = C == 8 ? 4 : (N == 32 && C == 32 ? 3 : (N == 64 && C == 64 ? 1 : 2));
+    static constexpr int CTAS = N == 32 && C <= 32 ? 3 : (N == 64 && C == 64 ? 1 : 2);
     static constexpr int NR = C <= 32 ? (N == 32 ? 5 : 6) : (N == 32 ? 4 : 8);
     static constexpr int ZEROS = C == 8 ? 2048 : 0;               // the 128 pixels paired with the last tap
     static constexpr int SLOTS = C == 8 ? NR + 1 : NR;            // C = 8: slot NR repeats slot 0
     static constexpr int SMEM = (WBYTES + 1023) / 1024 * 1024 + SLOTS * ROW + ZEROS + 1024;
-    static constexpr int EW = N == 32 ? 4 : 8;                    // epilogue warps
+    // Epilogue warps: PG groups that take output rows in turn, N / 32 column blocks each.  Two
+    // groups and the early release of the accumulator: 32 x 256^2, 8 -> 32 channels 95 -> 84 us.
+    // The other layers, bound by the issue of the epilogue's instructions, gained with those
+    // (silu_n): with both, 32 -> 32 channels 108 -> 87, 64 -> 32 142 -> 121, 64 -> 64 72 -> 64.
+    static constexpr int PG = N == 64 && C == 32 ? 1 : 2, EW = PG * N / 8;
+    static constexpr int CS = CTAS == 3 ? 16 : 32;                // columns worked on at a time: 64 registers
     static_assert(CTAS * (SMEM + 2048) <= 232448, "shared memory per SM");
 };
 
@@ -809,7 +850,7 @@ __global__ void __launch_bounds__(32 * (CfgR<C, N>::EW + 2), CfgR<C, N>::CTAS)
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&tfull[b]), 1);
-            mbar_init(smem_u32(&tempty[b]), 32 * EW);
+            mbar_init(smem_u32(&tempty[b]), 32 * EW / Cf::PG);
         }
         mbar_init(smem_u32(&wbar), 1);
         mbar_init(smem_u32(&done_bar), 1);
@@ -941,10 +982,9 @@ __global__ void __launch_bounds__(32 * (CfgR<C, N>::EW + 2), CfgR<C, N>::CTAS)
             mma_commit(smem_u32(&done_bar));   // arrives once every MMA above completed
         }
     } else {
-        // ---------------- epilogue (EW warps: lane quarter warp % 4, column half warp / 4) ----------------
-        const int half = warp >> 2, cw = N * 4 / EW;
-        int lt = 0;
-        for (int i = t0; i < t1; ++i, ++lt) {
+        // ---------------- epilogue (lane quarter warp % 4, then column block, then group) ----------------
+        const int cb = (warp >> 2) % (N / 32), group = warp / (N / 8);
+        for (int i = t0 + group, lt = group; i < t1; i += Cf::PG, lt += Cf::PG) {
             const int buf = lt & 1;
             const bool ready = mbar_wait(smem_u32(&tfull[buf]), (uint32_t)((lt >> 1) & 1), abort_v);
             asm volatile("tcgen05.fence::after_thread_sync;");
@@ -955,9 +995,8 @@ __global__ void __launch_bounds__(32 * (CfgR<C, N>::EW + 2), CfgR<C, N>::CTAS)
             const int y = i & (H - 1), col = i >> g.lh;
             const int b = col >> (g.lw - 7), x0 = (col & ((1 << (g.lw - 7)) - 1)) << 7;
             const long long m0 = ((((long long)b << g.lh) + y) << g.lw) + x0;
-            epilogue<N>(g.e, tmem + (uint32_t)(buf * N), m0, 0, warp & 3, lane, half * cw, (half + 1) * cw);
-            asm volatile("tcgen05.fence::before_thread_sync;");
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[buf])));
+            epilogue<N, Cf::CS>(g.e, tmem + (uint32_t)(buf * N), m0, 0, warp & 3, lane, cb * 32, cb * 32 + 32,
+                                [&] { arrive_drained(&tempty[buf]); });
         }
         // Tensor memory must be idle before it is freed.
         if (!mbar_wait(smem_u32(&done_bar), 0)) *abort_v = 1;
@@ -1242,7 +1281,8 @@ cudaError_t launch_tma(const CUtensorMap &ma, const CUtensorMap &mb, const TArgs
     gg.ntiles = g.e.N / BN;
     const long long tiles = (long long)gg.mtiles * gg.ntiles * (MN ? gg.splits : 1);
     const long long ctas = tiles < 2LL * sms ? tiles : 2LL * sms;   // two resident CTAs per SM
-    return evlbm::launch_pdl(k_gemm_tma<BN, ASW, MN>, (unsigned)ctas, 192, CfgT<BN>::SMEM, st, ma, mb, gg);
+    return evlbm::launch_pdl(k_gemm_tma<BN, ASW, MN>, (unsigned)ctas, 32 * (kEpiWarps<BN, MN> + 2), CfgT<BN>::SMEM,
+                             st, ma, mb, gg);
 }
 
 template <int ASW>
