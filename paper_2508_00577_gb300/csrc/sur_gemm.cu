@@ -185,8 +185,7 @@ __device__ __forceinline__ void epilogue(const Epi &g, uint32_t tmem, long long 
             } else {
                 if (g.out) store_bf16<CS>(static_cast<bf16 *>(g.out) + orow * g.ldo + g.co0 + col, v);
                 if (g.epi == SUR_EPI_CONV) {
-#pragma unroll
-                    for (int j = 0; j < CS; ++j) v[j] = silu(v[j]);
+                    silu_n<CS>(v);
                     if (g.pix) {
                         for_halo(row, g.lh, g.lw,
                                  [&](long long t) { store_bf16<CS>(g.y + t * g.ldy + g.cy0 + col, v); });

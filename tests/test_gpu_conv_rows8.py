@@ -45,3 +45,29 @@ def test_infinity_stays_in_its_neighbourhood():
     want = np.zeros((H, W), bool)
     want[2:5, 99:102] = True
     np.testing.assert_array_equal(bad, want)
+
+
+def test_silu_over_the_whole_range():
+    """Zero input, so that z is the bias: ordinary values, values beyond the packed form's range
+    beside them, and the ends of the range, against FP64 (one BF16 rounding of z and one of
+    silu; where e^-z overflows silu is -0, at -inf NaN)."""
+    Bn, H, W = 1, 2, 128
+    M = Bn * H * W
+    X = torch.zeros((Bn, H + 2, W + 2, 8), dtype=torch.bfloat16, device=dev)
+    Wb = torch.zeros((32, 128), dtype=torch.bfloat16, device=dev)
+    for big in ([], [79.5, 80.5, -80.5, 1e30], [-87.5, -88.5, -90.0, -1e30], [float("inf"), float("-inf"), float("nan")]):
+        z = np.array((big + list(np.linspace(-30.0, 30.0, 32)))[:32], dtype=np.float32)
+        z[31], z[30] = 0.0, 17.5
+        bias = torch.tensor(z, device=dev)
+        Y = torch.full((Bn, H + 2, W + 2, 32), 3.0, dtype=torch.bfloat16, device=dev)
+        gemm(op(X, S.SUR_OP_CONV3, 8, 0, 8, M, H, W), op(Wb, S.SUR_OP_DENSE, 128, rows=32), M, 32, 128,
+             epi=S.SUR_EPI_CONV, bias=bias, y=Y, ldy=32)
+        got = interior(Y.float().cpu().numpy())
+        with np.errstate(over="ignore", invalid="ignore"):
+            want = z.astype(np.float64) / (1.0 + np.exp(-z.astype(np.float64)))
+        want[z < -88.8] = 0.0
+        want[np.isneginf(z)] = np.nan
+        np.testing.assert_array_equal(np.isnan(got), np.broadcast_to(np.isnan(want), got.shape))
+        np.testing.assert_array_equal(np.isinf(got), np.broadcast_to(np.isinf(want), got.shape))
+        ok = np.isfinite(want)
+        assert np.all(np.abs(got[..., ok] - want[ok]) <= 2 ** -8 * np.abs(want[ok]) + 1e-35)
