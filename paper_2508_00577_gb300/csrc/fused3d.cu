@@ -283,6 +283,8 @@ __device__ __forceinline__ void psi3_poly(float A0, float A1, float A2, float ou
 // 512 (16-bit storage).  The thermal kernel with 16-bit storage spills ~30 B per thread at
 // that budget; 8 warps per SM with 245 registers and no spill was measured slower (2.11
 // against 2.49 GLUPS at 256^3, an earlier form).
+// Every sum of products below is written with its fused multiply-adds, so that all forms of the
+// kernel round alike.
 template <bool THERMAL, typename S>
 __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3d(const Args<S> A)
 {
@@ -407,20 +409,20 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
                     if (i == 13) continue;
                     const float v = r[1 + czi(i)][c0 + cyi(i) * WA + cxi(i)];
                     const float w = wi(i);
-                    if (cxi(i)) gx += (cxi(i) * w) * v;
-                    if (cyi(i)) gy += (cyi(i) * w) * v;
-                    if (czi(i)) gz += (czi(i) * w) * v;
-                    lap += w * (v - rc);
+                    if (cxi(i)) gx = fmaf(cxi(i) * w, v, gx);
+                    if (cyi(i)) gy = fmaf(cyi(i) * w, v, gy);
+                    if (czi(i)) gz = fmaf(czi(i) * w, v, gz);
+                    lap = fmaf(w, v - rc, lap);
                 }
                 gx *= 3.f; gy *= 3.f; gz *= 3.f; lap *= 6.f;
-                const float s = -a * rc * rc - kappa * rc * lap - 0.5f * kappa * (gx * gx + gy * gy + gz * gz);
+                const float s = -fmaf(a * rc, rc, fmaf(kappa * rc, lap, 0.5f * kappa * fmaf(gx, gx, fmaf(gy, gy, gz * gz))));
                 float *pr = PI + sb(cx, cy);
-                pr[0] = s + kappa * gx * gx;
+                pr[0] = fmaf(kappa * gx, gx, s);
                 pr[SB] = kappa * gx * gy;
                 pr[2 * SB] = kappa * gx * gz;
-                pr[3 * SB] = s + kappa * gy * gy;
+                pr[3 * SB] = fmaf(kappa * gy, gy, s);
                 pr[4 * SB] = kappa * gy * gz;
-                pr[5 * SB] = s + kappa * gz * gz;
+                pr[5 * SB] = fmaf(kappa * gz, gz, s);
             }
         }
         __syncthreads();
@@ -493,34 +495,34 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
                         const float *pp = PI + b0 + oy * WB + ox;
                         if (ox) {
                             const float cw = ox * w;
-                            T[0] += cw * pp[0];
-                            T[1] += cw * pp[SB];
-                            T[2] += cw * pp[2 * SB];
+                            T[0] = fmaf(cw, pp[0], T[0]);
+                            T[1] = fmaf(cw, pp[SB], T[1]);
+                            T[2] = fmaf(cw, pp[2 * SB], T[2]);
                         }
                         if (oy) {
                             const float cw = oy * w;
-                            T[0] += cw * pp[SB];
-                            T[1] += cw * pp[3 * SB];
-                            T[2] += cw * pp[4 * SB];
+                            T[0] = fmaf(cw, pp[SB], T[0]);
+                            T[1] = fmaf(cw, pp[3 * SB], T[1]);
+                            T[2] = fmaf(cw, pp[4 * SB], T[2]);
                         }
-                        Sz[0] += w * pp[2 * SB];
-                        Sz[1] += w * pp[4 * SB];
-                        Sz[2] += w * pp[5 * SB];
+                        Sz[0] = fmaf(w, pp[2 * SB], Sz[0]);
+                        Sz[1] = fmaf(w, pp[4 * SB], Sz[1]);
+                        Sz[2] = fmaf(w, pp[5 * SB], Sz[2]);
                     }
                 float *fq = PF + s0 * 3 * SC + pc, *fq1 = PF + sm1 * 3 * SC + pc, *fq2 = PF + sm2 * 3 * SC + pc;
                 float F[3];
 #pragma unroll
                 for (int m = 0; m < 3; ++m) {
                     fq[m * SC] = (1.f / 6.f) * (T[m] - Sz[m]);           // plane q,   cz = -1 (first term)
-                    fq1[m * SC] += (2.f / 3.f) * T[m];                  // plane q-1, cz = 0
-                    F[m] = -3.f * (fq2[m * SC] + (1.f / 6.f) * (T[m] + Sz[m]));   // plane q-2, complete
+                    fq1[m * SC] = fmaf(2.f / 3.f, T[m], fq1[m * SC]);                  // plane q-1, cz = 0
+                    F[m] = -3.f * fmaf(1.f / 6.f, T[m] + Sz[m], fq2[m * SC]);   // plane q-2, complete
                 }
                 if (!runC) continue;
                 const float Fx = F[0], Fy = F[1], Fz = F[2];
                 const float rho = RHO[sm2 * SA + sa(cx, cy)];
                 const float *jr = J + sm2 * 3 * SC + sc(cx, cy);
                 const float ir = rcpa(rho);
-                const float ux = (jr[0] + 0.5f * Fx) * ir, uy = (jr[SC] + 0.5f * Fy) * ir, uz = (jr[2 * SC] + 0.5f * Fz) * ir;
+                const float ux = fmaf(0.5f, Fx, jr[0]) * ir, uy = fmaf(0.5f, Fy, jr[SC]) * ir, uz = fmaf(0.5f, Fz, jr[2 * SC]) * ir;
                 float RT;
                 if (THERMAL) {
                     if (!(GST && k == 0)) {
@@ -533,8 +535,8 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
                             Gam += h;
                         }
                     }
-                    const float E = (Gam + 0.5f * (ux * Fx + uy * Fy + uz * Fz)) * ir;
-                    RT = (2.f / 3.f) * (E - 0.5f * (ux * ux + uy * uy + uz * uz));
+                    const float E = fmaf(0.5f, fmaf(ux, Fx, fmaf(uy, Fy, uz * Fz)), Gam) * ir;
+                    RT = (2.f / 3.f) * fmaf(-0.5f, fmaf(ux, ux, fmaf(uy, uy, uz * uz)), E);
                 } else {
                     const unsigned n = (unsigned)zc * (unsigned)nx * (unsigned)ny +
                                        (unsigned)wrapi(y0 + cy, ny) * (unsigned)nx + (unsigned)wrapi(x0 + cx, nx);
@@ -543,25 +545,25 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
                 // EOS in the Enskog gauge: P0 = P_E = rho RT Z, gamma0 = 1 + rho Z'/Z [+ 2/3 Z].
                 float Z, dlnZ;
                 if (A.eos == 0) {
-                    Z = rcpa(1.f - b * rho);
-                    dlnZ = b * rho * Z;
+                    Z = rcpa(fmaf(-b, rho, 1.f));
+                    dlnZ = __fmul_rn(b * rho, Z);
                 } else {
-                    const float eta = 0.25f * b * rho;
-                    const float num = 1.f + eta + eta * eta - eta * eta * eta;
+                    const float eta = __fmul_rn(0.25f * b, rho);
+                    const float num = fmaf(eta, fmaf(eta, 1.f - eta, 1.f), 1.f);
                     const float iom = rcpa(1.f - eta);
                     Z = num * iom * iom * iom;
-                    dlnZ = eta * (4.f + 4.f * eta - 2.f * eta * eta) * iom * rcpa(num);
+                    dlnZ = __fmul_rn(eta * fmaf(eta, fmaf(-2.f, eta, 4.f), 4.f) * iom, rcpa(num));
                 }
-                const float g0 = THERMAL ? 1.f + dlnZ + (2.f / 3.f) * Z : 1.f + dlnZ;
-                const float th = RT * Z;
-                const float th3m1 = 3.f * th - 1.f;
+                const float g0 = THERMAL ? fmaf(2.f / 3.f, Z, 1.f + dlnZ) : 1.f + dlnZ;
+                const float th = __fmul_rn(RT, Z);
+                const float th3m1 = fmaf(3.f, th, -1.f);
                 float *cf = CF + sm2 * 7 * SC + sc(cx, cy);
                 cf[0] = ux;
                 cf[SC] = uy;
                 cf[2 * SC] = uz;
-                cf[3 * SC] = rho * ux * (ux * ux + th3m1);
-                cf[4 * SC] = rho * uy * (uy * uy + th3m1);
-                cf[5 * SC] = rho * uz * (uz * uz + th3m1);
+                cf[3 * SC] = rho * ux * fmaf(ux, ux, th3m1);
+                cf[4 * SC] = rho * uy * fmaf(uy, uy, th3m1);
+                cf[5 * SC] = rho * uz * fmaf(uz, uz, th3m1);
                 cf[6 * SC] = th - RT;
                 if (k == 0) {
                     // The slot still holds plane q-3, collided by this thread in stage D of
@@ -591,20 +593,20 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
             const int c0 = sc(dcx, dcy);
             const int xp = c0 + 1, xm = c0 - 1, yp = c0 + WC, ym = c0 - WC;
             const float ux = F0[c0], uy = F0[SC + c0], uz = F0[2 * SC + c0];
-            const float P0 = rho * th;
+            const float P0 = __fmul_rn(rho, th);
             const float divu = 0.5f * ((F0[xp] - F0[xm]) + (F0[SC + yp] - F0[SC + ym]) + (Fp[2 * SC + c0] - Fm[2 * SC + c0]));
-            const float Phi1 = P0 * (5.f / 3.f - g0) * divu;
+            const float Phi1 = __fmul_rn(P0 * (5.f / 3.f - g0), divu);
             // Phi_aa = Phi' - d_a[rho u_a (u_a^2 + 3 theta0 - 1)] (sign cancelling the c^3 = c bias).
-            const float Phx = Phi1 - 0.5f * (F0[3 * SC + xp] - F0[3 * SC + xm]);
-            const float Phy = Phi1 - 0.5f * (F0[4 * SC + yp] - F0[4 * SC + ym]);
-            const float Phz = Phi1 - 0.5f * (Fp[5 * SC + c0] - Fm[5 * SC + c0]);
+            const float Phx = fmaf(-0.5f, F0[3 * SC + xp] - F0[3 * SC + xm], Phi1);
+            const float Phy = fmaf(-0.5f, F0[4 * SC + yp] - F0[4 * SC + ym], Phi1);
+            const float Phz = fmaf(-0.5f, Fp[5 * SC + c0] - Fm[5 * SC + c0], Phi1);
             const float lP0h = 0.5f * lambda * P0, lPhi = lambda * Phi1;
-            const float qx = lP0h * (F0[6 * SC + xp] - F0[6 * SC + xm]) + ux * lPhi;
-            const float qy = lP0h * (F0[6 * SC + yp] - F0[6 * SC + ym]) + uy * lPhi;
-            const float qz = lP0h * (Fp[6 * SC + c0] - Fm[6 * SC + c0]) + uz * lPhi;
+            const float qx = fmaf(lP0h, F0[6 * SC + xp] - F0[6 * SC + xm], ux * lPhi);
+            const float qy = fmaf(lP0h, F0[6 * SC + yp] - F0[6 * SC + ym], uy * lPhi);
+            const float qz = fmaf(lP0h, Fp[6 * SC + c0] - Fm[6 * SC + c0], uz * lPhi);
 
             const float lir = lambda * rcpa(rho);
-            const float usx = ux + Fx * lir, usy = uy + Fy * lir, usz = uz + Fz * lir;
+            const float usx = fmaf(Fx, lir, ux), usy = fmaf(Fy, lir, uy), usz = fmaf(Fz, lir, uz);
             // Separable equilibria: h_i = X[c_ix] * YZ[c_iy][c_iz] (+ X'[c_ix] * YZ'[..]),
             // the per-axis Psi factors combined once per node (Eqs. feq, f_star, geq, gstar).
             // f^eq and g^eq are evaluated with the rounding-exact functions of the 16-bit
@@ -616,9 +618,9 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
                 ey[k] = refP(k - 1, uy, th);
                 ez[k] = refP(k - 1, uz, th);
             }
-            psi3(usx, th + usx * usx + Phx * lir, sx);
-            psi3(usy, th + usy * usy + Phy * lir, sy);
-            psi3(usz, th + usz * usz + Phz * lir, sz);
+            psi3(usx, fmaf(Phx, lir, fmaf(usx, usx, th)), sx);
+            psi3(usy, fmaf(Phy, lir, fmaf(usy, usy, th)), sy);
+            psi3(usz, fmaf(Phz, lir, fmaf(usz, usz, th)), sz);
             float rex[3], rsx[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
@@ -651,26 +653,26 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
             float Ag[3], As[3], rpx[3], Sy[3], Sz[3], Ty[3], Tz[3], py[3], pz[3];
             float hq[3] = {0.f, 0.f, 0.f};
             if (THERMAL) {
-                const float es = e - 0.5f * (Fx * Fx + Fy * Fy + Fz * Fz) * (lir * lir);
+                const float es = fmaf(-0.5f, __fmul_rn(fmaf(Fx, Fx, fmaf(Fy, Fy, Fz * Fz)), lir * lir), e);
                 auto psiS = [&](float v, float o3[3]) {
-                    const float vv = v * v;
-                    psi3_poly(0.5f * vv, v * (th + 0.5f * vv), th * th + vv * (2.5f * th + 0.5f * vv), o3);
+                    const float vv = __fmul_rn(v, v);
+                    psi3_poly(0.5f * vv, __fmul_rn(v, fmaf(0.5f, vv, th)), fmaf(th, th, vv * fmaf(2.5f, th, 0.5f * vv)), o3);
                 };
                 float T[3], px[3];
-                psi3(usx, th + usx * usx, px);
+                psi3(usx, fmaf(usx, usx, th), px);
                 psiS(usx, T);
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     Ag[k] = ref_A(rho, e, ex[k], refS(k - 1, ux, th));
                     rpx[k] = rho * px[k];
-                    As[k] = rho * (es * px[k] + T[k]);
+                    As[k] = rho * fmaf(es, px[k], T[k]);
                     Sy[k] = refS(k - 1, uy, th);
                     Sz[k] = refS(k - 1, uz, th);
                 }
                 psiS(usy, Ty);
                 psiS(usz, Tz);
-                psi3(usy, th + usy * usy, py);
-                psi3(usz, th + usz * usz, pz);
+                psi3(usy, fmaf(usy, usy, th), py);
+                psi3(usz, fmaf(usz, usz, th), pz);
                 hq[0] = 0.5f * qx;
                 hq[1] = 0.5f * qy;
                 hq[2] = 0.5f * qz;
@@ -699,7 +701,7 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
                     // f first (its output written before the g are loaded: fewer live registers)
                     auto emit_f = [&](int cx, float Ey, float Sly, float iwxy, unsigned i, float hf) {
                         const float feq = ref_f_of(rex[cx + 1], Ey);
-                        const float vf = kh * hf + keq * feq + kst * (rsx[cx + 1] * Sly);
+                        const float vf = fmaf(kh, hf, fmaf(keq, feq, kst * (rsx[cx + 1] * Sly)));
                         if (act) stc(A.fo, i * N + out, 27ull * N, (vf - feq) * (inv_f * (iwxy * iwz)));
                     };
                     if (kz < 2) {
@@ -740,7 +742,7 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
                     for (int j = 0; j < 3; ++j) {
                         C[j] = ref_D(ey[j], Sy[j], ezk, Szk);
                         P[j] = py[j] * pzk;
-                        Dd[j] = Ty[j] * pzk + py[j] * Tzk;
+                        Dd[j] = fmaf(Ty[j], pzk, py[j] * Tzk);
                     }
 #pragma unroll
                     for (int j = 0; j < 9; ++j) {
@@ -748,11 +750,11 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
                         const unsigned i = (unsigned)j + 9u * (unsigned)kz;
                         const float iw = (cx ? 6.f : 1.5f) * (cy ? 6.f : 1.5f) * iwz;
                         const float geq = ref_g_of(Ag[cx + 1], rex[cx + 1], E[cy + 1], C[cy + 1]);
-                        float gst = As[cx + 1] * P[cy + 1] + rpx[cx + 1] * Dd[cy + 1];
+                        float gst = fmaf(As[cx + 1], P[cy + 1], rpx[cx + 1] * Dd[cy + 1]);
                         if (cx != 0 && cy == 0) gst += cz == 0 ? cx * hq[0] : 0.f;
                         if (cx == 0 && cy != 0) gst += cz == 0 ? cy * hq[1] : 0.f;
                         if (cx == 0 && cy == 0) gst += float(cz) * hq[2];
-                        const float vg = kh * hg9[j] + keq * geq + kst * gst;
+                        const float vg = fmaf(kh, hg9[j], fmaf(keq, geq, kst * gst));
                         if (act) stc(A.go, i * N + out, 27ull * N, (vg - geq) * (inv_g * iw));
                     }
                 } else {
@@ -763,7 +765,7 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
                         const unsigned i = (unsigned)j + 9u * (unsigned)kz;
                         const float h = hf9[j];
                         const float feq = ref_f_of(rex[cx + 1], E[cy + 1]);
-                        float v = kh * h + keq * feq + kst * (rsx[cx + 1] * Sl[cy + 1]);
+                        float v = fmaf(kh, h, fmaf(keq, feq, kst * (rsx[cx + 1] * Sl[cy + 1])));
                         if constexpr (DEV)
                             v = (v - feq) * (inv_f * ((cx ? 6.f : 1.5f) * (cy ? 6.f : 1.5f) * iwz));
                         // The output is not read again this step: a streaming store keeps L2 for
@@ -777,7 +779,7 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
                         for (int j = 0; j < 3; ++j) {
                             C[j] = ref_D(ey[j], Sy[j], ezk, Szk);
                             P[j] = py[j] * pzk;
-                            Dd[j] = Ty[j] * pzk + py[j] * Tzk;
+                            Dd[j] = fmaf(Ty[j], pzk, py[j] * Tzk);
                         }
 #pragma unroll
                         for (int j = 0; j < 9; ++j) {
@@ -786,12 +788,12 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
                             const unsigned i = (unsigned)j + 9u * (unsigned)kz;
                             const float h = PRE ? gD[i] : ldc(A.g, i * N + sn, 27ull * N);   // FP32 storage here
                             const float geq = ref_g_of(Ag[cx + 1], rex[cx + 1], E[cy + 1], C[cy + 1]);
-                            float gst = As[cx + 1] * P[cy + 1] + rpx[cx + 1] * Dd[cy + 1];
+                            float gst = fmaf(As[cx + 1], P[cy + 1], rpx[cx + 1] * Dd[cy + 1]);
                             // g' on the |c| = 1 populations
                             if (cx != 0 && cy == 0) gst += cz == 0 ? cx * hq[0] : 0.f;
                             if (cx == 0 && cy != 0) gst += cz == 0 ? cy * hq[1] : 0.f;
                             if (cx == 0 && cy == 0) gst += float(cz) * hq[2];
-                            if (act) stc(A.go, i * N + out, 27ull * N, kh * h + keq * geq + kst * gst);
+                            if (act) stc(A.go, i * N + out, 27ull * N, fmaf(kh, h, fmaf(keq, geq, kst * gst)));
                         }
                     }
                 }
