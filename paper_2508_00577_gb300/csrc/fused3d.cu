@@ -283,12 +283,18 @@ __device__ __forceinline__ void psi3_poly(float A0, float A1, float A2, float ou
 // 512 (16-bit storage).  The thermal kernel with 16-bit storage spills ~30 B per thread at
 // that budget; 8 warps per SM with 245 registers and no spill was measured slower (2.11
 // against 2.49 GLUPS at 256^3, an earlier form).
-// Every sum of products below is written with its fused multiply-adds, so that all forms of the
-// kernel round alike.
-template <bool THERMAL, typename S>
-__global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3d(const Args<S> A)
+//
+// ONE (FP32 storage): one CTA per SM with up to 255 registers, for grids of at most one CTA per
+// SM.  There every plane is a chain of load latencies with nothing else to run, so the loads go
+// out together: stage A's three column passes are unrolled, and stage C's g are loaded before
+// stage A's barrier.  75 x 50 x 61, 20 steps: 1990 -> 1614 us.  Every sum of products below is
+// written with its fused multiply-adds, so that both forms of the kernel round alike and a
+// lattice's values do not depend on which of them its launch shape takes.
+template <bool THERMAL, typename S, bool ONE>
+__global__ void __launch_bounds__(TileOf<S>::G::NT, ONE ? 1 : TileOf<S>::G::MINB) k_fused3d(const Args<S> A)
 {
     constexpr bool DEV = Store<S>::dev;
+    static_assert(!(ONE && DEV), "16-bit storage has one CTA per SM as it is");
     constexpr bool GST = DEV && THERMAL;                  // the g-stash layout of the TMEM columns
     using G = typename TileOf<S>::G;
     constexpr int TX = G::TX, TY = G::TY, NT = G::NT, WA = G::WA, WB = G::WB, WC = G::WC;
@@ -357,7 +363,7 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
         if (q <= zend + 2) {
             unsigned zo[3];
             plane_offsets(q, nx, ny, nz, zo);
-#pragma unroll 1
+#pragma unroll(ONE ? PA : 1)
             for (int k = 0; k < PA; ++k) {
                 int cx, cy;
                 if (!colA(k, cx, cy)) continue;
@@ -388,10 +394,24 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
                 }
             }
         }
-        __syncthreads();
-
         const bool haveP = q - 1 >= z0 - 2 && q - 1 <= zend + 1;   // stage B writes Pi(q-1)
         const bool runC = q - 2 >= z0 - 1 && q - 2 <= zend;        // stage C's plane is needed
+        float gC[ONE && THERMAL ? 54 : 1];                         // ONE: stage C's g, tile and ring column
+        if constexpr (ONE && THERMAL) {
+            if (haveP && runC) {
+                unsigned zo[3];
+                plane_offsets(q - 2, nx, ny, nz, zo);
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    int cx, cy;
+                    if (!colC(k, cx, cy)) continue;
+                    const Cell c = cell_of(x0 + cx, y0 + cy, nx, ny);
+#pragma unroll
+                    for (int i = 0; i < 27; ++i) gC[27 * k + i] = ldc(A.g, src_of(i, c, zo, N), 27ull * N);
+                }
+            }
+        }
+        __syncthreads();
 
         // ---------------- B: Korteweg stress of plane q-1 ----------------
         if (haveP) {
@@ -525,7 +545,10 @@ __global__ void __launch_bounds__(TileOf<S>::G::NT, TileOf<S>::G::MINB) k_fused3
                 const float ux = fmaf(0.5f, Fx, jr[0]) * ir, uy = fmaf(0.5f, Fy, jr[SC]) * ir, uz = fmaf(0.5f, Fz, jr[2 * SC]) * ir;
                 float RT;
                 if (THERMAL) {
-                    if (!(GST && k == 0)) {
+                    if constexpr (ONE) {
+#pragma unroll
+                        for (int i = 0; i < 27; ++i) Gam += gC[27 * k + i];
+                    } else if (!(GST && k == 0)) {
                         const Cell c = cell_of(x0 + cx, y0 + cy, nx, ny);
 #pragma unroll
                         for (int i = 0; i < 27; ++i) {
@@ -982,8 +1005,8 @@ __global__ void __launch_bounds__(MGeo::NT, 3) k_moments3d(const Args<S> A, cons
     }
 }
 
-template <bool THERMAL, typename S>
-cudaError_t launch(const Args<S> &A, cudaStream_t st)
+template <bool THERMAL, typename S, bool ONE>
+cudaError_t launch_k(const Args<S> &A, dim3 grid, cudaStream_t st)
 {
     using G = typename TileOf<S>::G;
     static int attr_dev = -1;
@@ -991,12 +1014,31 @@ cudaError_t launch(const Args<S> &A, cudaStream_t st)
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (attr_dev != dev) {
-        e = cudaFuncSetAttribute(k_fused3d<THERMAL, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM_BYTES);
+        e = cudaFuncSetAttribute(k_fused3d<THERMAL, S, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM_BYTES);
         if (e != cudaSuccess) return e;
         attr_dev = dev;
     }
+    return launch_pdl(k_fused3d<THERMAL, S, ONE>, grid, G::NT, G::SMEM_BYTES, st, A);
+}
+
+int sm_count()
+{
+    static int sms = 0;
+    int dev = 0;
+    if (!sms && (cudaGetDevice(&dev) != cudaSuccess ||
+                 cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1))
+        sms = 152;
+    return sms;
+}
+
+template <bool THERMAL, typename S>
+cudaError_t launch(const Args<S> &A, cudaStream_t st)
+{
+    using G = typename TileOf<S>::G;
     const dim3 grid((A.nx + G::TX - 1) / G::TX, (A.ny + G::TY - 1) / G::TY, A.nfull + A.ntail);
-    return launch_pdl(k_fused3d<THERMAL, S>, grid, G::NT, G::SMEM_BYTES, st, A);
+    if constexpr (!Store<S>::dev)
+        if ((long long)grid.x * grid.y * grid.z <= sm_count()) return launch_k<THERMAL, S, true>(A, grid, st);
+    return launch_k<THERMAL, S, false>(A, grid, st);
 }
 
 // z-chunks of at most H planes: chunks of H while more than 2 H planes remain, then the rest
@@ -1030,18 +1072,15 @@ struct Chunks {
 
 // Default z-chunk: the height with the least estimated time.  A CTA that marches h planes
 // runs h + 5 iterations (pipeline fill); while all CTAs are resident the longest one decides,
-// and an SM that holds one CTA of the FP32 kernel instead of two runs an iteration in 0.62 of
-// the time (5.6 against 9 us); with more CTAs than slots the slots share the iterations and
+// and an SM that holds one CTA of the FP32 kernel (its ONE form) instead of two runs an
+// iteration in 0.48 of the time (4.3 against 9 us); with more CTAs than slots the slots share the iterations and
 // the shortest chunk's length is partly lost at the end.  Against the former rule (64
 // planes), us per step: 75 x 50 x 61 FP32 258 -> 90, BF16 672 -> 183; 32^3 132 -> 34;
 // 64 x 64 x 160 527 -> 144 (10 planes), 128^3 579 -> 419 and 1398 -> 811; 256^3 takes 128.
 template <class G> int default_chunk(const KParams &p)
 {
     constexpr int kFill = 5;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-        sms = 152;
+    const int sms = sm_count();
     const double slots = (double)sms * G::MINB;
     const long long tiles = (long long)((p.nx + G::TX - 1) / G::TX) * ((p.ny + G::TY - 1) / G::TY);
     double best = 1e300;
@@ -1059,7 +1098,7 @@ template <class G> int default_chunk(const KParams &p)
         }
         const double ctas = (double)(tiles * n);
         double t;
-        if (ctas <= slots) t = (longest + kFill) * (G::MINB == 2 && ctas <= sms ? 0.62 : 1.0);
+        if (ctas <= slots) t = (longest + kFill) * (G::MINB == 2 && ctas <= sms ? 0.48 : 1.0);
         else t = (p.nz + (double)kFill * n) * tiles / slots + 0.5 * (shortest + kFill);
         if (t < best) {
             best = t;
