@@ -13,8 +13,9 @@
 //     cp.async.bulk.tensor boxes of 128 pixels of the shifted window, swizzled
 //     128/64 B (none for 8 channels); B (the weights) is one swizzled box.  The
 //     children of the coarse pixels (UPADJ, TUP) are boxes of a five-dimensional
-//     view of the fine tensor.  One thread issues the copies, one the MMAs, four
-//     warps run the epilogue.
+//     view of the fine tensor.  One thread issues the copies, one the MMAs, four or
+//     eight warps run the epilogue.  On images at least 128 pixels wide the narrow layers
+//     march down the rows instead (k_conv_rows, k_wgrad_rows).
 //   * cp.async: every other operand form; four producer warps, one MMA warp.
 #include <cuda.h>
 #include <cudaTypedefs.h>
