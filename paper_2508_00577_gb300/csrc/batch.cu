@@ -576,7 +576,11 @@ int lbm_batch_get_tile(const lbm_batch *b, int *tile_w, int *tile_h)
 int lbm_batch_autotune(lbm_batch *b, int probe_steps, int *tile_w, int *tile_h)
 {
     if (!b || probe_steps < 1) return LBM_EINVAL;
-    const int heights[] = {32, 64, 128, 256, 512};     // 512: every domain of <= 512 rows in one chunk
+    // 512: every domain of <= 512 rows in one chunk.  8 and 16 are for ensembles whose items of
+    // 32 rows are fewer than the CTAs the GPU holds (us per step: 24 domains of up to 160^2,
+    // 275456 nodes, 30.4 at 96 x 32 -> 16.5 at 64 x 8; 12 of up to 288^2, 386816 nodes, 32.4 -> 19.9 at 96 x 16) and
+    // are left out where they would make more than two items per CTA.
+    const int heights[] = {8, 16, 32, 64, 128, 256, 512};
     // Each shape is timed on one persistent launch of 2 * probe_steps steps, as in a run,
     // where the last items of a step overlap the first items of the next.  The launch
     // starts from a copy of the current state; an even step count ends in the current
@@ -610,10 +614,12 @@ int lbm_batch_autotune(lbm_batch *b, int probe_steps, int *tile_w, int *tile_h)
     const bool have_copy = saved && copy_state(false) == cudaSuccess;
     if (saved && !have_copy) rc = LBM_ECUDA;
     for (int wi = 0; wi < evlbm::kFusedWidthCount && rc == LBM_OK; ++wi) {
-        for (int hi = 0; hi < 5 && rc == LBM_OK; ++hi) {
+        for (int hi = 0; hi < 7 && rc == LBM_OK; ++hi) {
             b->tile_w = evlbm::kFusedWidths[wi];
             b->tile_h = heights[hi];
             if ((rc = retile(b))) break;
+            const int resident = b->P.thermal ? evlbm::grid_for<true>(b->tile_w) : evlbm::grid_for<false>(b->tile_w);
+            if (b->tile_h < 32 && b->items_per_step > 2 * resident) continue;
             float ms = 0.f;
             if (saved) {
                 if (copy_state(true) != cudaSuccess || cudaEventRecord(e0, b->stream) != cudaSuccess ||
