@@ -578,8 +578,8 @@ int lbm_batch_autotune(lbm_batch *b, int probe_steps, int *tile_w, int *tile_h)
     if (!b || probe_steps < 1) return LBM_EINVAL;
     // 512: every domain of <= 512 rows in one chunk.  8 and 16 are for ensembles whose items of
     // 32 rows are fewer than the CTAs the GPU holds (us per step: 24 domains of up to 160^2,
-    // 275456 nodes, 30.4 at 96 x 32 -> 16.5 at 64 x 8; 12 of up to 288^2, 386816 nodes, 32.4 -> 19.9 at 96 x 16) and
-    // are left out where they would make more than two items per CTA.
+    // 275456 nodes, 30.4 at 96 x 32 -> 16.5 at 64 x 8; 12 of up to 288^2, 386816 nodes, 32.4 ->
+    // 19.9 at 96 x 16) and are left out where they would make more than two items per CTA.
     const int heights[] = {8, 16, 32, 64, 128, 256, 512};
     // Each shape is timed on one persistent launch of 2 * probe_steps steps, as in a run,
     // where the last items of a step overlap the first items of the next.  The launch
