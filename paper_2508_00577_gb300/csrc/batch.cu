@@ -124,6 +124,7 @@ __global__ void __launch_bounds__(threads_of<kW>(), Shape<kW>::MINB) k_batch(Bat
         A.nx = D.nx;
         A.ny = D.ny;
         A.nz = 1;
+        A.z0 = 0;
         A.H = D.H;
         A.N = (unsigned)D.nx * (unsigned)D.ny;
         A.eos = B.eos;

@@ -94,8 +94,7 @@ cudaError_t fused2d_moments(int prec, const KParams &p, const void *f, const voi
 {
     if (!fused2d_supported(prec, 9, p)) return cudaErrorNotSupported;
     if (prec != 1) return fused2d_moments16(prec, p, f, g, RT_iso, Rin, o, st);
-    FusedArgs A = make_args(p, f, g, nullptr, nullptr, RT_iso, Rin, nullptr);
-    moment_args(A, o);
+    const MomentArgs A = moment_args(p, f, g, RT_iso, Rin, o);
     if (p.walls)
         return p.thermal ? launch_moments<true, true, float>(A, p.nz, st) : launch_moments<false, true, float>(A, p.nz, st);
     return p.thermal ? launch_moments<true, false, float>(A, p.nz, st) : launch_moments<false, false, float>(A, p.nz, st);

@@ -35,8 +35,7 @@ cudaError_t fused2d_step16(int prec, const KParams &p, const void *f, const void
 cudaError_t fused2d_moments16(int prec, const KParams &p, const void *f, const void *g, const void *RT_iso,
                               const void *Rin, const MomentOut &o, cudaStream_t st)
 {
-    FusedArgs A = make_args(p, f, g, nullptr, nullptr, RT_iso, Rin, nullptr);
-    moment_args(A, o);
+    const MomentArgs A = moment_args(p, f, g, RT_iso, Rin, o);
     if (prec == 2)
         return p.thermal ? launch_moments<true, false, __half>(A, p.nz, st) : launch_moments<false, false, __half>(A, p.nz, st);
     return p.thermal ? launch_moments<true, false, __nv_bfloat16>(A, p.nz, st)

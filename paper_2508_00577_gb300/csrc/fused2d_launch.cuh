@@ -55,18 +55,18 @@ __global__ void __launch_bounds__(threads_of<kW>(), Shape<kW>::MINB) k_fused2d_b
 // thermal 1024^2 layers (moments 141, stress 88, macro 153, export 173).
 template <int kW, bool THERMAL, bool WALLS, typename ST>
 __global__ void __launch_bounds__(threads_of<kW>(), (kW == 64 ? 6 : 4) - (WALLS || Store<ST>::dev ? (kW == 64 ? 2 : 1) : 0))
-    k_moments2d(FusedArgs A)
+    k_moments2d(MomentArgs A)
 {
     extern __shared__ v2 smem[];
     pdl_wait();
     const int y0 = blockIdx.y * A.H;                       // H is even
-    fused_tile<kW, THERMAL, false, WALLS, ST, true>(A, blockIdx.x, y0, min(A.H, A.ny - y0), A.z0 + (int)blockIdx.z, smem);
+    fused_tile<kW, THERMAL, false, WALLS, ST>(A, blockIdx.x, y0, min(A.H, A.ny - y0), A.z0 + (int)blockIdx.z, smem);
 }
 
-// Chunks of 32 rows at most (16 row pairs after 2 that fill the pipeline), shorter while the
+// Chunks of 32 rows at most (16 row pairs after 3 that fill the pipeline), shorter while the
 // grid would leave SMs without a CTA; narrow strips on narrow lattices.
 template <bool THERMAL, bool WALLS, typename ST>
-cudaError_t launch_moments(FusedArgs A, int nz, cudaStream_t st)
+cudaError_t launch_moments(MomentArgs A, int nz, cudaStream_t st)
 {
     const int W = A.nx > 64 ? 128 : 64, S = (A.nx + W - 1) / W;
     A.H = 32;
@@ -75,7 +75,7 @@ cudaError_t launch_moments(FusedArgs A, int nz, cudaStream_t st)
     // A z extent of the grid is limited to 65535: larger stacks of layers go in parts.
     for (int z = 0; z < nz; z += 65535) {
         const dim3 grid(S, (A.ny + A.H - 1) / A.H, nz - z < 65535 ? nz - z : 65535);
-        FusedArgs B = A;
+        MomentArgs B = A;
         B.z0 = z;
         const cudaError_t e =
             W == 64 ? launch_pdl(k_moments2d<64, THERMAL, WALLS, ST>, grid, threads_of<64>(), moments_smem_of<64>(), st, B)
@@ -159,17 +159,17 @@ inline FusedArgs make_args(const KParams &p, const void *f, const void *g, void 
     A.wall_uy[0] = float(p.wall_u[0][1]);
     A.wall_uy[1] = float(p.wall_u[1][1]);
     A.wall_RT = float(p.wall_RT);
-    A.m_rho = A.m_u = A.m_T = A.m_F = nullptr;
-    A.Rh = A.Ri = 1.f;
-    A.Rl = 0.f;
     A.z0 = 0;
     return A;
 }
 
-// Arguments of the moments kernel: outputs (any may be NULL) and the gas constant T is divided
-// by (1: R T itself).
-inline void moment_args(FusedArgs &A, const MomentOut &o)
+// Arguments of the moments kernel: a state, outputs (any may be NULL) and the gas constant T is
+// divided by (1: R T itself).
+inline MomentArgs moment_args(const KParams &p, const void *f, const void *g, const void *RT_iso, const void *Rin,
+                              const MomentOut &o)
 {
+    MomentArgs A;
+    static_cast<FusedArgs &>(A) = make_args(p, f, g, nullptr, nullptr, RT_iso, Rin, nullptr);
     A.m_rho = o.rho;
     A.m_u = o.u;
     A.m_T = o.T;
@@ -177,6 +177,7 @@ inline void moment_args(FusedArgs &A, const MomentOut &o)
     A.Rh = float(o.R);
     A.Rl = float(o.R - double(A.Rh));
     A.Ri = float(1.0 / o.R);
+    return A;
 }
 
 // Launch shape of a step: strip width W and chunk height (A.H); balanced persistent grid.
