@@ -19,7 +19,7 @@ __global__ void __launch_bounds__(threads_of<kW>(), Shape<kW>::MINB) k_fused2d(F
     pdl_wait();
     pdl_trigger();
     const int y0 = blockIdx.y * A.H;                       // H is even
-    fused_tile<kW, THERMAL, false, WALLS, ST>(A, blockIdx.x, y0, min(A.H, A.ny - y0), blockIdx.z, smem);
+    fused_tile<kW, THERMAL, false, WALLS, ST>(A, blockIdx.x, y0, min(A.H, A.ny - y0), A.z0 + (int)blockIdx.z, smem);
 }
 
 // Balanced persistent variant: a grid of S x parts CTAs (S strips, parts = the
@@ -49,6 +49,19 @@ __global__ void __launch_bounds__(threads_of<kW>(), Shape<kW>::MINB) k_fused2d_b
     }
 }
 
+// A grid of chunks by layers takes at most kGridYZ of either: taller chunks where there would
+// be more of them, and larger stacks in parts.
+constexpr int kGridYZ = 65535;
+template <class ARGS, class F> cudaError_t in_layers(ARGS A, int nz, F launch_part)
+{
+    while ((A.ny + A.H - 1) / A.H > kGridYZ) A.H *= 2;
+    for (; A.z0 < nz; A.z0 += kGridYZ) {
+        const cudaError_t e = launch_part(A, min(nz - A.z0, kGridYZ));
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 // Macroscopic fields of the current state: stages A to C of the step in one pass, reading the
 // populations once and writing the fields (72 + 16 bytes per node with FP32 storage).  The
 // four stage kernels it replaces passed through ~20 scratch fields per node: 555 us on nine
@@ -71,18 +84,12 @@ cudaError_t launch_moments(MomentArgs A, int nz, cudaStream_t st)
     const int W = A.nx > 64 ? 128 : 64, S = (A.nx + W - 1) / W;
     A.H = 32;
     while (A.H > 4 && (long long)S * ((A.ny + A.H - 1) / A.H) * nz < 456) A.H >>= 1;
-    while ((A.ny + A.H - 1) / A.H > 65535) A.H <<= 1;
-    // A z extent of the grid is limited to 65535: larger stacks of layers go in parts.
-    for (int z = 0; z < nz; z += 65535) {
-        const dim3 grid(S, (A.ny + A.H - 1) / A.H, nz - z < 65535 ? nz - z : 65535);
-        MomentArgs B = A;
-        B.z0 = z;
-        const cudaError_t e =
-            W == 64 ? launch_pdl(k_moments2d<64, THERMAL, WALLS, ST>, grid, threads_of<64>(), moments_smem_of<64>(), st, B)
-                    : launch_pdl(k_moments2d<128, THERMAL, WALLS, ST>, grid, threads_of<128>(), moments_smem_of<128>(), st, B);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    return in_layers(A, nz, [&](const MomentArgs &B, int layers) {
+        const dim3 grid(S, (B.ny + B.H - 1) / B.H, layers);
+        return W == 64 ? launch_pdl(k_moments2d<64, THERMAL, WALLS, ST>, grid, threads_of<64>(), moments_smem_of<64>(), st, B)
+                       : launch_pdl(k_moments2d<128, THERMAL, WALLS, ST>, grid, threads_of<128>(), moments_smem_of<128>(), st,
+                                    B);
+    });
 }
 
 template <int W, bool THERMAL, bool WALLS, typename ST>
@@ -115,9 +122,11 @@ cudaError_t launch_w(const FusedArgs &A, int nz, bool balanced, cudaStream_t st)
         return launch_pdl(k_fused2d_bal<W, THERMAL, WALLS, ST>, dim3((unsigned)(S * parts)), threads_of<W>(),
                           handoff_smem(smem, S * parts, sms), st, A);
     }
-    const dim3 grid((A.nx + W - 1) / W, (A.ny + A.H - 1) / A.H, nz);
-    return launch_pdl(k_fused2d<W, THERMAL, WALLS, ST>, grid, threads_of<W>(),
-                      handoff_smem(smem, (long long)grid.x * grid.y * grid.z, sms), st, A);
+    return in_layers(A, nz, [&](const FusedArgs &B, int layers) {
+        const dim3 grid((B.nx + W - 1) / W, (B.ny + B.H - 1) / B.H, layers);
+        return launch_pdl(k_fused2d<W, THERMAL, WALLS, ST>, grid, threads_of<W>(),
+                          handoff_smem(smem, (long long)grid.x * grid.y * grid.z, sms), st, B);
+    });
 }
 
 template <bool THERMAL, bool WALLS, typename ST>
