@@ -851,8 +851,8 @@ __global__ void __launch_bounds__(MGeo::NT, 3) k_moments3d(const Args<S> A, cons
     __shared__ float RHO[3 * SA], PI[6 * SB];
     pdl_wait();
     const int t = threadIdx.x, nx = A.nx, ny = A.ny, nz = A.nz;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-    const int z0 = (int)blockIdx.z * A.HZ, zend = min(z0 + A.HZ, nz);
+    const int gx = (nx + TX - 1) / TX, x0 = (int)(blockIdx.x % gx) * TX, y0 = (int)(blockIdx.x / gx) * TY;
+    const int z0 = (int)blockIdx.y * A.HZ, zend = min(z0 + A.HZ, nz);
     const unsigned N = A.N;
     const float a = A.a, kappa = A.kappa;
     auto sa = [](int cx, int cy) { return (cy + 2) * WA + (cx + 2); };
@@ -1148,12 +1148,13 @@ cudaError_t moments_t(const KParams &p, const void *f, const void *g, const void
     M.Rl = float(o.R - double(M.Rh));
     M.Ri = float(1.0 / o.R);
     // Chunks of 32 planes (after 4 that fill the pipeline), shorter while the grid would leave
-    // slots of the GPU (152 SMs x 3) empty.
-    const int gx = (p.nx + MGeo::TX - 1) / MGeo::TX, gy = (p.ny + MGeo::TY - 1) / MGeo::TY;
+    // slots of the GPU (152 SMs x 3) empty.  The tiles run along the grid's x, which alone is
+    // not limited to 65535.
+    const long long tiles = (long long)((p.nx + MGeo::TX - 1) / MGeo::TX) * ((p.ny + MGeo::TY - 1) / MGeo::TY);
     A.HZ = 32;
-    while (A.HZ > 2 && (long long)gx * gy * ((p.nz + A.HZ - 1) / A.HZ) < 456) A.HZ >>= 1;
+    while (A.HZ > 2 && tiles * ((p.nz + A.HZ - 1) / A.HZ) < 456) A.HZ >>= 1;
     while ((p.nz + A.HZ - 1) / A.HZ > 65535) A.HZ <<= 1;
-    const dim3 grid(gx, gy, (p.nz + A.HZ - 1) / A.HZ);
+    const dim3 grid((unsigned)tiles, (p.nz + A.HZ - 1) / A.HZ);
     return p.thermal ? launch_pdl(k_moments3d<true, S>, grid, MGeo::NT, 0, st, A, M)
                      : launch_pdl(k_moments3d<false, S>, grid, MGeo::NT, 0, st, A, M);
 }
@@ -1163,7 +1164,9 @@ cudaError_t step_t(const KParams &p, const void *f, const void *g, void *fo, voi
                    const void *Rin, void *Rout, cudaStream_t st)
 {
     Args<S> A = make_args3<S>(p, f, g, fo, go, RT_iso, Rin, Rout);
-    z_chunks(p.tile_h > 0 ? p.tile_h : default_chunk<typename TileOf<S>::G>(p), p.nz, A);
+    int H = p.tile_h > 0 ? p.tile_h : default_chunk<typename TileOf<S>::G>(p);
+    z_chunks(H, p.nz, A);
+    while (A.nfull + A.ntail > 65535) z_chunks(H *= 2, p.nz, A);      // the grid's z extent
     return p.thermal ? launch<true, S>(A, st) : launch<false, S>(A, st);
 }
 
