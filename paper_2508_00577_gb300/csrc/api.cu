@@ -183,6 +183,13 @@ __global__ void k_scale_field(const float *T, float R, long long N, float *RT)
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x)
         RT[n] = R * T[n];
 }
+// T = R T / R in place, for the R that the fused fields do not divide by (an FP64 division in
+// their kernel: 9 x 1024^2, 168 -> 185 us with it behind a branch).
+__global__ void k_divide_field(float *T, double R, long long N)
+{
+    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x)
+        T[n] = float(double(T[n]) / R);
+}
 // Initial fields, FP64 as the caller passed them (rho [N], u [D][N], T [N]), checked and
 // converted on the device: out = (rho, u, R T) in the scratch precision; *bad = the lowest
 // node with rho or T not finite and > 0 or u not finite (left at N when all are valid).
@@ -375,8 +382,14 @@ int lbm_moments_device(lbm_ctx *c, float *d_rho, float *d_u, float *d_T)
 {
     if (!c) return LBM_EINVAL;
     cudaError_t e = cudaSuccess;
-    if (fused_moments(c, {d_rho, d_u, d_T, nullptr, c->P.R}, &e))
+    const bool divides = c->P.R >= evlbm::kLeastR && c->P.R <= evlbm::kMostR;
+    if (fused_moments(c, {d_rho, d_u, d_T, nullptr, divides ? c->P.R : 1.0}, &e)) {
+        if (e == cudaSuccess && d_T && !divides) {
+            k_divide_field<<<(int)(c->N < 256 * 4096 ? (c->N + 255) / 256 : 4096), 256, 0, c->stream>>>(d_T, c->P.R, c->N);
+            e = cudaGetLastError();
+        }
         return e == cudaSuccess ? LBM_OK : cuda_fail(c, e, "lbm_moments_device");
+    }
     int rc = run_macro(c);
     if (rc) return rc;
     e = fp64(c) ? evlbm::ref_export_f64(c->Q, c->K, c->scratch, c->P.R, d_rho, d_u, d_T, c->stream)

@@ -41,11 +41,25 @@ struct FieldOffsets {
 };
 
 // Device outputs of the fused moments kernels (any may be NULL): rho [N], u [D][N], T [N] =
-// R T / R (R = 1: R T itself), F [D][N].
+// R T / R (R = 1: R T itself; 2^-100 <= R <= 2^100), F [D][N].
 struct MomentOut {
     float *rho, *u, *T, *F;
     double R;
 };
+constexpr double kLeastR = 0x1p-100, kMostR = 0x1p100;
+// The divisor of R T: R = h + l and i = 1 / R.
+struct GasConstant {
+    float h, l, i;
+    explicit GasConstant(double R = 1.0) : h(float(R)), l(float(R - double(h))), i(float(1.0 / R)) {}
+};
+// R T / R to within a rounding, exact for R = 1: the quotient by the reciprocal and its residual's
+// correction, which an infinite quotient does not have (inf - inf).
+__device__ __forceinline__ float over_R(float RT, const GasConstant &R)
+{
+    const float q = RT * R.i;
+    const float t = fmaf(fmaf(-q, R.l, fmaf(-q, R.h, RT)), R.i, q);
+    return isfinite(t) ? t : q;
+}
 // Macroscopic fields of the current state on lattices a fused step supports, as that step's
 // own stages compute them.
 cudaError_t fused2d_moments(int prec, const KParams &p, const void *f, const void *g, const void *RT_iso,

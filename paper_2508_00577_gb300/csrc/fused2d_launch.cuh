@@ -183,9 +183,7 @@ inline MomentArgs moment_args(const KParams &p, const void *f, const void *g, co
     A.m_u = o.u;
     A.m_T = o.T;
     A.m_F = o.F;
-    A.Rh = float(o.R);
-    A.Rl = float(o.R - double(A.Rh));
-    A.Ri = float(1.0 / o.R);
+    A.R = GasConstant(o.R);
     return A;
 }
 

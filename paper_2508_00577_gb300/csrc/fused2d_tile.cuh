@@ -106,20 +106,13 @@ struct FusedArgs {
 };
 
 // Arguments of the macroscopic fields: outputs rho [N], u [2][N], T [N], F [2][N] (any may be
-// NULL); T = R T / R with R = Rh + Rl and Ri = 1 / R.  A type of its own: with these members in
+// NULL); T = R T / R.  A type of its own: with these members in
 // FusedArgs the compiler spent fewer registers on the step (156 for 166 at 128 columns) and
 // 9 x 1024^2 thermal took 328.7 us a step, 321.2 without them (325.6 before there were any).
 struct MomentArgs : FusedArgs {
     float *m_rho, *m_u, *m_T, *m_F;
-    float Rh, Rl, Ri;
+    GasConstant R;
 };
-
-// RT / R to within a rounding (R = Rh + Rl, Ri ~ 1 / R); exact for R = 1.
-__device__ __forceinline__ float over_R(float RT, float Rh, float Rl, float Ri)
-{
-    const float q = RT * Ri;
-    return fmaf(fmaf(-q, Rl, fmaf(-q, Rh, RT)), Ri, q);
-}
 
 __device__ __forceinline__ int wrap_any(int v, int n)
 {
@@ -435,7 +428,7 @@ __device__ __forceinline__ void fused_tile(const ARGS &A, int bx, int y0, int ro
                 put(A.m_rho, rho);
                 put(A.m_u, ux);
                 put(A.m_u ? A.m_u + N : nullptr, uy);
-                put(A.m_T, V(over_R(RT.x, A.Rh, A.Rl, A.Ri), over_R(RT.y, A.Rh, A.Rl, A.Ri)));
+                put(A.m_T, V(over_R(RT.x, A.R), over_R(RT.y, A.R)));
                 put(A.m_F, Fx);
                 put(A.m_F ? A.m_F + N : nullptr, Fy);
             } else {

@@ -840,7 +840,7 @@ struct MGeo {
 };
 struct MArgs {
     float *rho, *u, *T, *F;                       // outputs, any may be NULL
-    float Rh, Rl, Ri;                             // R = Rh + Rl, Ri ~ 1 / R
+    GasConstant R;
 };
 
 template <bool THERMAL, typename S>
@@ -993,8 +993,7 @@ __global__ void __launch_bounds__(MGeo::NT, 3) k_moments3d(const Args<S> A, cons
             } else {
                 RT = ldc(A.RT_iso, n, N);
             }
-            const float qt = RT * M.Ri;                            // RT / R, exact for R = 1
-            M.T[n] = fmaf(fmaf(-qt, M.Rl, fmaf(-qt, M.Rh, RT)), M.Ri, qt);
+            M.T[n] = over_R(RT, M.R);
         }
         if (M.rho) M.rho[n] = rho;
 #pragma unroll
@@ -1144,9 +1143,7 @@ cudaError_t moments_t(const KParams &p, const void *f, const void *g, const void
     M.u = o.u;
     M.T = o.T;
     M.F = o.F;
-    M.Rh = float(o.R);
-    M.Rl = float(o.R - double(M.Rh));
-    M.Ri = float(1.0 / o.R);
+    M.R = GasConstant(o.R);
     // Chunks of 32 planes (after 4 that fill the pipeline), shorter while the grid would leave
     // slots of the GPU (152 SMs x 3) empty.  The tiles run along the grid's x, which alone is
     // not limited to 65535.
