@@ -112,6 +112,7 @@ bool dev16(const lbm_ctx *c) { return c->P.precision == LBM_FP16_DEV || c->P.pre
 bool fused_moments(lbm_ctx *c, const evlbm::MomentOut &o, cudaError_t *e)
 {
     if (fp64(c)) return false;
+    c->K.follows = 0;
     const void *f = c->f[c->cur], *g = c->g[c->cur], *R = c->R[c->cur];
     if (evlbm::fused2d_supported(c->P.precision, c->Q, c->K)) {
         *e = evlbm::fused2d_moments(c->P.precision, c->K, f, g, c->RT_iso, R, o, c->stream);
@@ -343,6 +344,7 @@ int lbm_step(lbm_ctx *c, int n_steps)
         if (e != cudaSuccess) return cuda_fail(c, e, "lbm_step");
         c->cur = nx;
         c->steps++;
+        c->K.follows = K.follows = 1;
     }
     return LBM_OK;
 }
@@ -369,6 +371,7 @@ int lbm_reset_device(lbm_ctx *c, const float *d_rho, const float *d_u, const flo
     const long long N = c->N;
     long long blocks = (N + 255) / 256;
     if (blocks > 4096) blocks = 4096;
+    c->K.follows = 0;
     k_scale_field<<<(int)blocks, 256, 0, c->stream>>>(d_T, float(c->P.R), N, static_cast<float *>(c->RT_iso));
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
@@ -409,6 +412,7 @@ int lbm_populations(lbm_ctx *c, double *f, double *g)
         CK(c, cudaStreamSynchronize(c->stream));
         return LBM_OK;
     }
+    c->K.follows = 0;
     double *tmp = nullptr;
     CK(c, cudaMalloc(&tmp, sizeof(double) * cnt));
     for (int which = 0; which < (c->P.thermal && g ? 2 : 1); ++which) {
@@ -430,6 +434,7 @@ int lbm_conserved(lbm_ctx *c, double out[5])
 {
     if (!c || !out) return c ? fail(c, LBM_EINVAL, "out is NULL") : LBM_EINVAL;
     int bad = 0;
+    c->K.follows = 0;
     cudaError_t e = evlbm::totals(c->P.precision, c->Q, c->K, c->f[c->cur], c->g[c->cur], c->R[c->cur], c->red, out,
                                   &bad, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "lbm_conserved");
@@ -504,6 +509,7 @@ int lbm_set_tile(lbm_ctx *c, int tile_w, int tile_h)
     }
     c->K.tile_w = (c->Q == 27 && tile_h >= 1) ? evlbm::fused3d_tile_w(c->P.precision) : tile_w;
     c->K.tile_h = tile_h;
+    c->K.follows = 0;
     return LBM_OK;
 }
 
@@ -605,6 +611,7 @@ int lbm_autotune(lbm_ctx *c, int probe_steps, int *tile_w, int *tile_h)
             // One untimed launch, then probe_steps timed ones; input stays c->f[c->cur].
             for (int s = 0; s <= probe_steps && e == cudaSuccess; ++s) {
                 if (s == 1) e = cudaEventRecord(e0, c->stream);
+                K.follows = s > 0;
                 if (e == cudaSuccess)
                     e = evlbm::fused2d_step(c->P.precision, K, c->f[c->cur], c->g[c->cur], c->f[nx], c->g[nx],
                                             c->RT_iso, c->R[c->cur], c->R[nx], c->stream);
@@ -628,6 +635,7 @@ int lbm_autotune(lbm_ctx *c, int probe_steps, int *tile_w, int *tile_h)
                 bw = evlbm::kFusedWidths[wi];
                 bh = heights[hi] < c->P.ny ? heights[hi] : c->P.ny;
             }
+    c->K.follows = 0;
     c->K.tile_w = bw;
     c->K.tile_h = bh;
     if (tile_w) *tile_w = bw;

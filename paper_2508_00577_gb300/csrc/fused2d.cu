@@ -83,10 +83,10 @@ cudaError_t fused2d_step(int prec, const KParams &p, const void *f, const void *
     bool balanced;
     launch_shape(p, A, W, balanced);
     if (p.walls)
-        return p.thermal ? launch<true, true, float>(W, A, p.nz, balanced, st)
-                         : launch<false, true, float>(W, A, p.nz, balanced, st);
-    return p.thermal ? launch<true, false, float>(W, A, p.nz, balanced, st)
-                     : launch<false, false, float>(W, A, p.nz, balanced, st);
+        return p.thermal ? launch<true, true, float>(W, A, p.nz, balanced, p.follows != 0, st)
+                         : launch<false, true, float>(W, A, p.nz, balanced, p.follows != 0, st);
+    return p.thermal ? launch<true, false, float>(W, A, p.nz, balanced, p.follows != 0, st)
+                     : launch<false, false, float>(W, A, p.nz, balanced, p.follows != 0, st);
 }
 
 cudaError_t fused2d_moments(int prec, const KParams &p, const void *f, const void *g, const void *RT_iso,

@@ -17,7 +17,8 @@ cudaError_t step16(const KParams &p, const void *f, const void *g, void *fo, voi
     int W;
     bool balanced;
     launch_shape(p, A, W, balanced);
-    return p.thermal ? launch<true, false, S>(W, A, p.nz, balanced, st) : launch<false, false, S>(W, A, p.nz, balanced, st);
+    return p.thermal ? launch<true, false, S>(W, A, p.nz, balanced, p.follows != 0, st)
+                     : launch<false, false, S>(W, A, p.nz, balanced, p.follows != 0, st);
 }
 
 }  // namespace

@@ -92,20 +92,27 @@ cudaError_t launch_moments(MomentArgs A, int nz, cudaStream_t st)
     });
 }
 
+// One step.  A step that follows a step of its context overlaps that one's end (pdl.cuh); the
+// first after other work does not.  Overlapping grids keep the places of the grid before: the
+// CTAs of a grid that leaves slots of the SMs free would else be placed around those of, say,
+// the kernel that set the populations, several on the SMs that have slots at that moment, and
+// all steps after it would keep to these SMs.  331 x 203 x 2 (136 CTAs), reset, 50 steps and
+// fields: 758 us with every step overlapping, 638 so, 737 with none.  (Claiming the rest of an
+// SM's shared memory, so that no second CTA fits beside the first, gave 647, but kept the grids
+// of other streams out too: eight such lattices at once 104 us a step, now 59.)
 template <int W, bool THERMAL, bool WALLS, typename ST>
-cudaError_t launch_w(const FusedArgs &A, int nz, bool balanced, cudaStream_t st)
+cudaError_t launch_w(const FusedArgs &A, int nz, bool balanced, bool follows, cudaStream_t st)
 {
     static bool attr = false;
-    static int resident = 0, sms = 0;
+    static int resident = 0;
     constexpr size_t smem = smem_of<W>();
-    constexpr int most = (int)(smem > kHandoffMax ? smem : kHandoffMax);
     if (!attr) {
         cudaError_t e = cudaFuncSetAttribute(k_fused2d<W, THERMAL, WALLS, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             most);
+                                             (int)smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_fused2d_bal<W, THERMAL, WALLS, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     most);
-        int per_sm = 0, dev = 0;
+                                     (int)smem);
+        int per_sm = 0, dev = 0, sms = 0;
         if (e == cudaSuccess)
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fused2d_bal<W, THERMAL, WALLS, ST>,
                                                               threads_of<W>(), smem);
@@ -119,24 +126,23 @@ cudaError_t launch_w(const FusedArgs &A, int nz, bool balanced, cudaStream_t st)
     if (balanced) {
         const int S = (A.nx + W - 1) / W;
         const long long parts = min((long long)max(resident / S, 1), (long long)nz * ((A.ny + 1) / 2));
-        return launch_pdl(k_fused2d_bal<W, THERMAL, WALLS, ST>, dim3((unsigned)(S * parts)), threads_of<W>(),
-                          handoff_smem(smem, S * parts, sms), st, A);
+        return launch_overlap(follows, k_fused2d_bal<W, THERMAL, WALLS, ST>, dim3((unsigned)(S * parts)),
+                              threads_of<W>(), smem, st, A);
     }
     return in_layers(A, nz, [&](const FusedArgs &B, int layers) {
         const dim3 grid((B.nx + W - 1) / W, (B.ny + B.H - 1) / B.H, layers);
-        return launch_pdl(k_fused2d<W, THERMAL, WALLS, ST>, grid, threads_of<W>(),
-                          handoff_smem(smem, (long long)grid.x * grid.y * grid.z, sms), st, B);
+        return launch_overlap(follows, k_fused2d<W, THERMAL, WALLS, ST>, grid, threads_of<W>(), smem, st, B);
     });
 }
 
 template <bool THERMAL, bool WALLS, typename ST>
-cudaError_t launch(int W, const FusedArgs &A, int nz, bool balanced, cudaStream_t st)
+cudaError_t launch(int W, const FusedArgs &A, int nz, bool balanced, bool follows, cudaStream_t st)
 {
     switch (W) {
-    case 64: return launch_w<64, THERMAL, WALLS, ST>(A, nz, balanced, st);
-    case 96: return launch_w<96, THERMAL, WALLS, ST>(A, nz, balanced, st);
-    case 192: return launch_w<192, THERMAL, WALLS, ST>(A, nz, balanced, st);
-    default: return launch_w<128, THERMAL, WALLS, ST>(A, nz, balanced, st);
+    case 64: return launch_w<64, THERMAL, WALLS, ST>(A, nz, balanced, follows, st);
+    case 96: return launch_w<96, THERMAL, WALLS, ST>(A, nz, balanced, follows, st);
+    case 192: return launch_w<192, THERMAL, WALLS, ST>(A, nz, balanced, follows, st);
+    default: return launch_w<128, THERMAL, WALLS, ST>(A, nz, balanced, follows, st);
     }
 }
 

@@ -17,29 +17,13 @@ namespace evlbm {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Dynamic shared memory of a kernel whose grid leaves slots of the SMs free: as much as keeps
-// one more CTA than the grid's share from fitting on an SM.  Otherwise the next grid's CTAs
-// would be placed while this one still runs, several on the SMs that happen to have free slots,
-// and stay there (136 CTAs of the 331 x 203 x 2 lattice on 152 SMs: 818 us per 50 steps, 660
-// with one CTA per SM handing over to the next, 736 without overlap).  The D3Q27 kernel loses
-// more by the smaller L1 than it gains (75 x 50 x 61: 1950 us, 2021 with this), and the FP64
-// stage kernels gain nothing (694, 690), so neither uses it.
-constexpr size_t kSmemPerSM = 233472, kSmemPerCta = 1024;
-inline size_t handoff_smem(size_t smem, long long ctas, int sms)
-{
-    const long long r = (ctas + sms - 1) / sms;
-    if (r > 3) return smem;
-    const size_t least = kSmemPerSM / (size_t)(r + 1) - kSmemPerCta + 128;
-    return smem > least ? smem : least / 128 * 128;
-}
-constexpr size_t kHandoffMax = kSmemPerSM / 2;
-
 template <class... P, class... Q>
-cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Q... args)
+cudaError_t launch_overlap(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                           Q... args)
 {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -50,6 +34,11 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
     if (e != cudaSuccess) cudaGetLastError();      // reported here: not left for a later call to find
     return e;
+}
+template <class... P, class... Q>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Q... args)
+{
+    return launch_overlap(true, kernel, grid, block, smem, st, args...);
 }
 
 }  // namespace evlbm
