@@ -96,6 +96,7 @@ void fill_kparams(lbm_ctx *c)
     k.eos = p.eos;
     k.thermal = p.thermal;
     k.force_form = p.force_form;
+    k.alone = 1;
     k.a = p.a;
     k.b = p.b;
     k.kappa = p.kappa;
@@ -509,6 +510,7 @@ int lbm_set_tile(lbm_ctx *c, int tile_w, int tile_h)
     }
     c->K.tile_w = (c->Q == 27 && tile_h >= 1) ? evlbm::fused3d_tile_w(c->P.precision) : tile_w;
     c->K.tile_h = tile_h;
+    c->K.alone = tile_h == 0;
     c->K.follows = 0;
     return LBM_OK;
 }
@@ -543,6 +545,7 @@ static int autotune3d(lbm_ctx *c, int probe_steps, int *tile_w, int *tile_h)
     float tmin[7];
     for (int hi = 0; hi < nh; ++hi) tmin[hi] = 1e30f;
     KParams K = c->K;
+    K.alone = 1;
     cudaError_t e = cudaSuccess;
     // Two rounds over the candidates, each keeping its faster time: a single probe of a
     // few launches is not repeatable to the few per cent that separate neighbouring chunks.
@@ -574,6 +577,7 @@ static int autotune3d(lbm_ctx *c, int probe_steps, int *tile_w, int *tile_h)
         }
     c->K.tile_w = evlbm::fused3d_tile_w(c->P.precision);
     c->K.tile_h = bh;
+    c->K.alone = 1;
     if (tile_w) *tile_w = evlbm::fused3d_tile_w(c->P.precision);
     if (tile_h) *tile_h = bh;
     return LBM_OK;

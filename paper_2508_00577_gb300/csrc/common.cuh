@@ -20,6 +20,7 @@ struct KParams {
     double c_eq;         // 2 beta
     double c_star;       // (dt/lambda)(1 - beta)
     int tile_w, tile_h;  // launch shape of the fused kernel (0 = default)
+    int alone;           // 1: the shape may take whole SMs (lbm_set_tile: the caller's shapes do not)
     int follows;         // 1: this step's launch follows a step of the same shape (launch_w)
     int walls;           // 1: the columns x = 0 and x = nx-1 are wall nodes (lbm_set_walls)
     double wall_u[2][3]; // velocity of the wall at x = 0 and at x = nx-1

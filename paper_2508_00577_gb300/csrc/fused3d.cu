@@ -285,7 +285,8 @@ __device__ __forceinline__ void psi3_poly(float A0, float A1, float A2, float ou
 // against 2.49 GLUPS at 256^3, an earlier form).
 //
 // ONE (FP32 storage): one CTA per SM with up to 255 registers, for grids of at most one CTA per
-// SM.  There every plane is a chain of load latencies with nothing else to run, so the loads go
+// SM whose shape the library picked (a shape the caller sets leaves room for other contexts: two
+// of 75 x 50 x 61 at once took 139 us a step with ONE, 129 without; one alone 77 and 96).  There every plane is a chain of load latencies with nothing else to run, so the loads go
 // out together: stage A's three column passes are unrolled, and stage C's g are loaded before
 // stage A's barrier.  75 x 50 x 61, 20 steps: 1990 -> 1614 us.  Every sum of products below is
 // written with its fused multiply-adds, so that both forms of the kernel round alike and a
@@ -1031,12 +1032,12 @@ int sm_count()
 }
 
 template <bool THERMAL, typename S>
-cudaError_t launch(const Args<S> &A, cudaStream_t st)
+cudaError_t launch(const Args<S> &A, bool alone, cudaStream_t st)
 {
     using G = typename TileOf<S>::G;
     const dim3 grid((A.nx + G::TX - 1) / G::TX, (A.ny + G::TY - 1) / G::TY, A.nfull + A.ntail);
     if constexpr (!Store<S>::dev)
-        if ((long long)grid.x * grid.y * grid.z <= sm_count()) return launch_k<THERMAL, S, true>(A, grid, st);
+        if (alone && (long long)grid.x * grid.y * grid.z <= sm_count()) return launch_k<THERMAL, S, true>(A, grid, st);
     return launch_k<THERMAL, S, false>(A, grid, st);
 }
 
@@ -1164,7 +1165,7 @@ cudaError_t step_t(const KParams &p, const void *f, const void *g, void *fo, voi
     int H = p.tile_h > 0 ? p.tile_h : default_chunk<typename TileOf<S>::G>(p);
     z_chunks(H, p.nz, A);
     while (A.nfull + A.ntail > 65535) z_chunks(H *= 2, p.nz, A);      // the grid's z extent
-    return p.thermal ? launch<true, S>(A, st) : launch<false, S>(A, st);
+    return p.thermal ? launch<true, S>(A, p.alone != 0, st) : launch<false, S>(A, p.alone != 0, st);
 }
 
 }  // namespace
