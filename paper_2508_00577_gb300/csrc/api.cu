@@ -28,6 +28,7 @@ struct lbm_ctx {
     void *scratch;         // stage-kernel fields, allocated on first use
     void *red;             // reduction work space
     long long steps;
+    int own_chunk;         // default z-chunk of the fused D3Q27 kernel (0: not asked for yet)
     char err[512];
 };
 
@@ -107,6 +108,12 @@ void fill_kparams(lbm_ctx *c)
 }
 
 bool dev16(const lbm_ctx *c) { return c->P.precision == LBM_FP16_DEV || c->P.precision == LBM_BF16_DEV; }
+
+int own_chunk(lbm_ctx *c)
+{
+    if (!c->own_chunk) c->own_chunk = evlbm::fused3d_default_chunk(c->P.precision, c->K);
+    return c->own_chunk;
+}
 
 // Macroscopic fields by the fused kernels where a fused step applies: one launch, the fields
 // straight to `o`.  False where it does not (FP64, literal force form, D3Q27 walls).
@@ -326,7 +333,7 @@ int lbm_step(lbm_ctx *c, int n_steps)
     // The launch shape is settled once per call (small lattices are bound by the launches).
     KParams K = c->K;
     if (fused && K.tile_w <= 0) evlbm::fused2d_default_tile(K, &K.tile_w, &K.tile_h);
-    if (fused3 && K.tile_h <= 0) K.tile_h = evlbm::fused3d_default_chunk(c->P.precision, K);
+    if (fused3 && K.tile_h <= 0) K.tile_h = own_chunk(c);
     for (int s = 0; s < n_steps; ++s) {
         const int nx = c->cur ^ 1;
         cudaError_t e;
@@ -535,7 +542,7 @@ static int autotune3d(lbm_ctx *c, int probe_steps, int *tile_w, int *tile_h)
     CK(c, cudaEventCreate(&e1));
     // The powers of two and the default of the lattice's size.
     int heights[7], nh = 0;
-    for (int h : {evlbm::fused3d_default_chunk(c->P.precision, c->K), 8, 16, 32, 64, 128, 256}) {
+    for (int h : {own_chunk(c), 8, 16, 32, 64, 128, 256}) {
         const int H = h < c->P.nz ? h : c->P.nz;
         bool seen = false;
         for (int k = 0; k < nh; ++k) seen = seen || heights[k] == H;

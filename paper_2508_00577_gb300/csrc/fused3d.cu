@@ -31,6 +31,9 @@
 // reference record (a 16- and an 8-byte load, L1/L2 hits after the first) and the
 // stored deviation; stage D writes the node's new record and the deviations of its
 // populations from the equilibria it computed for the collision.
+#include <algorithm>
+#include <map>
+
 #include "bounds.cuh"
 #include "dev16.cuh"
 #include "dispatch.h"
@@ -1070,36 +1073,54 @@ struct Chunks {
     int HZ, nfull, ntail, tail[kMaxTail + 1];
 };
 
-// Default z-chunk: the height with the least estimated time.  A CTA that marches h planes
-// runs h + 5 iterations (pipeline fill); while all CTAs are resident the longest one decides,
-// and an SM that holds one CTA of the FP32 kernel (its ONE form) instead of two runs an
-// iteration in 0.48 of the time (4.3 against 9 us); with more CTAs than slots the slots share the iterations and
-// the shortest chunk's length is partly lost at the end.  Against the former rule (64
-// planes), us per step: 75 x 50 x 61 FP32 258 -> 90, BF16 672 -> 183; 32^3 132 -> 34;
-// 64 x 64 x 160 527 -> 144 (10 planes), 128^3 579 -> 419 and 1398 -> 811; 256^3 takes 128.
+// Iterations until the last CTA ends, when `slots` slots take the CTAs in grid order (chunk by
+// chunk, `tiles` of each) as they become free.
+long long finish_of(const Chunks &c, long long tiles, long long slots, int fill)
+{
+    std::map<long long, long long> free_at{{0, slots}};               // time -> slots that are free from then on
+    for (int k = 0; k < c.nfull + c.ntail; ++k) {
+        const int d = fill + (k < c.nfull ? c.HZ : c.tail[k - c.nfull + 1] - c.tail[k - c.nfull]);
+        for (long long need = tiles; need > 0;) {
+            const auto first = free_at.begin();
+            const long long t = first->first, n = first->second < need ? first->second : need;
+            if ((first->second -= n) == 0) free_at.erase(first);
+            free_at[t + d] += n;
+            need -= n;
+        }
+    }
+    return free_at.rbegin()->first;
+}
+
+// Default z-chunk: the height with the least estimated time.  A CTA that marches h planes runs
+// h + 6 iterations, the first of which, without stages C and D, make the fill as long as 5.
+// While all CTAs are resident the longest one decides, and an SM that holds one CTA of the FP32
+// kernel (its ONE form) instead of two runs an iteration in 0.6 of the time; with more CTAs than
+// slots it is the end of the last one, for a third replaced by the iterations' share of a slot,
+// as CTAs speed up when others of their SM have ended.  Over 96 lattices of 12 to 320 planes and
+// rows (FP32 and 16-bit storage, both thermal and not) this takes 1.003 times the best height's
+// time, 1.12 at most; with half the shortest chunk added to the share in place of the end, 1.06
+// and 1.68, and up to 1.49 times that of 64 planes.  us a step with 64 planes and with this:
+// 75 x 50 x 61 FP32 258 -> 78, BF16 672 -> 177; 32^3 132 -> 24; 64 x 64 x 160 527 -> 131; 128^3
+// 579 -> 382 and 1398 -> 735; 170 x 96 x 161 600 -> 488; 256^3 takes 128.
 template <class G> int default_chunk(const KParams &p)
 {
-    constexpr int kFill = 5;
-    const int sms = sm_count();
-    const double slots = (double)sms * G::MINB;
+    constexpr int kFill = 5, kMostChunks = 4096;
+    const long long sms = sm_count(), slots = sms * G::MINB;
     const long long tiles = (long long)((p.nx + G::TX - 1) / G::TX) * ((p.ny + G::TY - 1) / G::TY);
     double best = 1e300;
-    int bh = 1;
+    int bh = 512;
     for (int h = 1; h <= 512; h += h < 16 ? 1 : (h < 64 ? 8 : 64)) {
         if (h > p.nz && h > 1) break;
         Chunks c;
         z_chunks(h, p.nz, c);
         const long long n = c.nfull + c.ntail;
-        int longest = c.nfull ? c.HZ : 0, shortest = c.HZ;
-        for (int k = 0; k < c.ntail; ++k) {
-            const int len = c.tail[k + 1] - c.tail[k];
-            longest = len > longest ? len : longest;
-            shortest = len < shortest ? len : shortest;
-        }
-        const double ctas = (double)(tiles * n);
-        double t;
-        if (ctas <= slots) t = (longest + kFill) * (G::MINB == 2 && ctas <= sms ? 0.48 : 1.0);
-        else t = (p.nz + (double)kFill * n) * tiles / slots + 0.5 * (shortest + kFill);
+        if (n > kMostChunks) continue;
+        int longest = c.nfull ? c.HZ : 0;
+        for (int k = 0; k < c.ntail; ++k) longest = std::max(longest, c.tail[k + 1] - c.tail[k]);
+        const double t = tiles * n <= slots
+                             ? (longest + kFill) * (G::MINB == 2 && tiles * n <= sms ? 0.6 : 1.0)
+                             : 0.7 * finish_of(c, tiles, slots, kFill) +
+                                   0.3 * (p.nz + (double)kFill * n) * tiles / slots;
         if (t < best) {
             best = t;
             bh = h;

@@ -64,8 +64,8 @@ print(json.dumps(out))
 
 
 def test_own_shape_stays_in_bounds():
-    lib = os.path.join(ROOT, "paper_2508_00577_gb300", "libevlbm_bc.so")
-    assert os.path.exists(lib), "the bounds-checked library is not built"
+    from paper_2508_00577_gb300 import _build
+    lib = _build.build(bounds_check=True)
     r = subprocess.run([sys.executable, "-c", f"ROOT = {ROOT!r}\n" + CHILD], capture_output=True, text=True,
                        env=dict(os.environ, EVLBM_LIBRARY=lib), timeout=600)
     assert r.returncode == 0, r.stderr[-2000:]
