@@ -1506,9 +1506,11 @@ int launch_rows(const sur_gemm_args &a, const Epi &e, cudaStream_t st)
     g.lw = ilog2(W);
     g.tiles = a.M / 128;
     g.e = e;
-    // At least 8 rows a CTA, so that the two rows it loads beyond its own stay a small part.
+    // Rows for every CTA that fits, down to one: the two rows a CTA loads beyond its own cost less
+    // than idle SMs (infer of 1 x 16 x 256, us: at least 8 rows a CTA 249, 4 197, 2 172, 1 162;
+    // 1 x 256^2 256, 212, 190, 189; 8 x 256^2 423, 410, 410, 410).
     int ctas = Cf::CTAS * sms;
-    if (g.tiles / 8 < ctas) ctas = g.tiles / 8 > 0 ? g.tiles / 8 : 1;
+    if (g.tiles < ctas) ctas = g.tiles;
     err = evlbm::launch_pdl(k_conv_rows<C, N>, ctas, 32 * (Cf::EW + 2), Cf::SMEM, st, ma, mb, g);
     return err == cudaSuccess ? SUR_OK : SUR_ECUDA;
 }
@@ -1564,10 +1566,14 @@ int launch_wgrad(const sur_gemm_args &a, int *status, cudaStream_t st)
     g.ldo = a.ldo;
     g.co0 = a.co0;
     g.status = status;
-    // As many CTAs as fit at once over the channel blocks, at least 8 rows each.
-    const int parts = a.a.C / CB;
+    // As many CTAs as fit at once over the channel blocks, with at least 8 rows each: every CTA
+    // adds its sums to the same 9 C x N values at the end.  Below that, one row each until every
+    // SM has one (training step of 1 x 16 x 256, us: at least 8 rows a CTA 706 and, with the
+    // convolutions' one row, 564 when there is one row for all that fit, 471 so; 1 x 256^2 822,
+    // 699, 666; 4 x 128^2 696, 655, 640; 16 x 256^2 2382 each).
+    const int parts = a.a.C / CB, least = g.tiles / 8 > sms ? g.tiles / 8 : (g.tiles < sms ? g.tiles : sms);
     int ctas = Cf::CTAS * sms / parts;
-    if (g.tiles / 8 < ctas) ctas = g.tiles / 8;
+    if (least < ctas) ctas = least;
     if (ctas < 1) ctas = 1;
     const cudaError_t err = evlbm::launch_pdl(k_wgrad_rows<CB, N>, dim3(ctas, parts), 192, Cf::SMEM, st, mx, mz, g);
     return err == cudaSuccess ? SUR_OK : SUR_ECUDA;
