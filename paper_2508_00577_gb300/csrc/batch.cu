@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(threads_of<kW>(), Shape<kW>::MINB) k_batch(Bat
         A.walls = 0;
         A.wall_uy[0] = A.wall_uy[1] = A.wall_RT = 0.f;
         const int y0 = (k / D.strips) * D.H;
-        fused_tile<kW, THERMAL, true>(A, k % D.strips, y0, min(D.H, D.ny - y0), 0, smem);
+        fused_tile<kW, THERMAL>(A, k % D.strips, y0, min(D.H, D.ny - y0), 0, smem);
         __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();

@@ -59,25 +59,25 @@ template <typename S> struct Store;
 
 template <> struct Store<double> {
     static constexpr bool dev = false;
-    __device__ static __forceinline__ double load(const double *p) { return __ldg(p); }
+    __device__ static __forceinline__ double load(const double *p) { return __ldca(p); }
     __device__ static __forceinline__ void store(double *p, double v) { *p = v; }
 };
 template <> struct Store<float> {
     static constexpr bool dev = false;
-    __device__ static __forceinline__ float load(const float *p) { return __ldg(p); }
+    __device__ static __forceinline__ float load(const float *p) { return __ldca(p); }
     __device__ static __forceinline__ void store(float *p, float v) { *p = v; }
 };
 template <> struct Store<__half> {
     static constexpr bool dev = true;
     // Value after a round trip through the storage format (registers only).
     __device__ static __forceinline__ float round(float v) { return __half2float(__float2half_rn(v)); }
-    __device__ static __forceinline__ float load(const __half *p) { return __half2float(__ldg(p)); }
+    __device__ static __forceinline__ float load(const __half *p) { return __half2float(__ldca(p)); }
     __device__ static __forceinline__ void store(__half *p, float v) { *p = __float2half_rn(v); }
 };
 template <> struct Store<__nv_bfloat16> {
     static constexpr bool dev = true;
     __device__ static __forceinline__ float round(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
-    __device__ static __forceinline__ float load(const __nv_bfloat16 *p) { return __bfloat162float(__ldg(p)); }
+    __device__ static __forceinline__ float load(const __nv_bfloat16 *p) { return __bfloat162float(__ldca(p)); }
     __device__ static __forceinline__ void store(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
 };
 

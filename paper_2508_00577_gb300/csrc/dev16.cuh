@@ -46,11 +46,11 @@ struct Ref16 {
 // the second; a record buffer of N nodes holds kRecBytes * N bytes.
 constexpr size_t kRecBytes = 4 * sizeof(float) + 2 * sizeof(float);
 
-// Record of node n of a lattice of N nodes (read-only path).
+// Record of node n of a lattice of N nodes.
 __device__ __forceinline__ Ref16 load_rec(const float *R, long long N, long long n)
 {
-    const float4 a = __ldg(reinterpret_cast<const float4 *>(R) + n);
-    const float2 b = __ldg(reinterpret_cast<const float2 *>(R + 4 * N) + n);
+    const float4 a = __ldca(reinterpret_cast<const float4 *>(R) + n);
+    const float2 b = __ldca(reinterpret_cast<const float2 *>(R + 4 * N) + n);
     return Ref16{a.x, {a.y, a.z, a.w}, b.x, b.y};
 }
 

@@ -19,7 +19,7 @@ __global__ void __launch_bounds__(threads_of<kW>(), Shape<kW>::MINB) k_fused2d(F
     pdl_wait();
     pdl_trigger();
     const int y0 = blockIdx.y * A.H;                       // H is even
-    fused_tile<kW, THERMAL, false, WALLS, ST>(A, blockIdx.x, y0, min(A.H, A.ny - y0), A.z0 + (int)blockIdx.z, smem);
+    fused_tile<kW, THERMAL, WALLS, ST>(A, blockIdx.x, y0, min(A.H, A.ny - y0), A.z0 + (int)blockIdx.z, smem);
 }
 
 // Balanced persistent variant: a grid of S x parts CTAs (S strips, parts = the
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(threads_of<kW>(), Shape<kW>::MINB) k_fused2d_b
         const int p0 = (int)(g - (long long)layer * P);
         const int p1 = (int)min((long long)P, p0 + (g1 - g));
         const int y0 = 2 * p0;
-        fused_tile<kW, THERMAL, false, WALLS, ST>(A, strip, y0, min(2 * p1, A.ny) - y0, layer, smem);
+        fused_tile<kW, THERMAL, WALLS, ST>(A, strip, y0, min(2 * p1, A.ny) - y0, layer, smem);
         __syncthreads();
         g += p1 - p0;
     }
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(threads_of<kW>(), (kW == 64 ? 6 : 4) - (WALLS 
     extern __shared__ v2 smem[];
     pdl_wait();
     const int y0 = blockIdx.y * A.H;                       // H is even
-    fused_tile<kW, THERMAL, false, WALLS, ST>(A, blockIdx.x, y0, min(A.H, A.ny - y0), A.z0 + (int)blockIdx.z, smem);
+    fused_tile<kW, THERMAL, WALLS, ST>(A, blockIdx.x, y0, min(A.H, A.ny - y0), A.z0 + (int)blockIdx.z, smem);
 }
 
 // Chunks of 32 rows at most (16 row pairs after 3 that fill the pipeline), shorter while the

@@ -122,38 +122,37 @@ __device__ __forceinline__ int wrap_any(int v, int n)
 __device__ __forceinline__ int prev_row(int r, int ny) { return r == 0 ? ny - 1 : r - 1; }
 __device__ __forceinline__ int next_row(int r, int ny) { return r == ny - 1 ? 0 : r + 1; }
 
-// CG: the populations were written earlier in the same launch (persistent ensemble kernel),
-// so the read-only path (ld.global.nc) is not allowed.  A plain L1-cached load (ld.global.ca)
-// is: the CTA reads them only after thread 0's gpu-scope acquire of the domain's completion
-// counter (which pairs with the producers' fence + atomic release) and a CTA barrier, and an
-// acquire at gpu scope makes every later load of the CTA observe the released writes.
-template <bool CG> __device__ __forceinline__ float ldpop(const float *p) { return CG ? __ldca(p) : __ldg(p); }
+// Loads of populations.  A CTA is resident before they are written, by the step before (a
+// dependent launch) or by another CTA of the persistent ensemble kernel, so the read-only path
+// (ld.global.nc), which asks for data that does not change while the kernel runs, is not allowed,
+// however long before the load the writes end.  A plain L1-cached load (ld.global.ca) is: it
+// follows pdl_wait or, in the ensemble, a CTA barrier behind thread 0's gpu-scope acquire of the
+// domain's completion counter (which pairs with the producers' fence + atomic release), and either
+// makes the CTA observe the writes.  Both kinds of load take the same time (9 x 1024^2 thermal,
+// 321.2 us a step).
+__device__ __forceinline__ float ldpop(const float *p) { return __ldca(p); }
 
 // Pulled populations of rows (r, r+1) of one column: h_i(y) = h~_i(x - c_ix, y - c_iy).
 // ro[k] = offset of wrapped row r - 1 + k (k = 0..3), cols[k] = wrapped column x - 1 + k.
-template <bool CG>
-__device__ __forceinline__ void pull18(const float *__restrict__ base, unsigned N, const unsigned ro[4],
-                                       const int cols[3], v2 h[9])
+__device__ __forceinline__ void pull18(const float *base, unsigned N, const unsigned ro[4], const int cols[3], v2 h[9])
 {
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         const int cx = i % 3 - 1, cy = i / 3 - 1;
         const float *p = base + i * N + cols[1 - cx];
         const float *p0 = p + ro[1 - cy], *p1 = p + ro[2 - cy];
-        h[i] = V(in_bounds(p0 - base, 9ull * N) ? ldpop<CG>(p0) : 0.f, in_bounds(p1 - base, 9ull * N) ? ldpop<CG>(p1) : 0.f);
+        h[i] = V(in_bounds(p0 - base, 9ull * N) ? ldpop(p0) : 0.f, in_bounds(p1 - base, 9ull * N) ? ldpop(p1) : 0.f);
     }
 }
 
 // A wall column's own populations of rows (r, r+1): wall nodes do not stream.
-template <bool CG>
-__device__ __forceinline__ void pull_own(const float *__restrict__ base, unsigned N, const unsigned ro[4], int col,
-                                         v2 h[9])
+__device__ __forceinline__ void pull_own(const float *base, unsigned N, const unsigned ro[4], int col, v2 h[9])
 {
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         const float *p = base + i * N + col;
         const float *p0 = p + ro[1], *p1 = p + ro[2];
-        h[i] = V(in_bounds(p0 - base, 9ull * N) ? ldpop<CG>(p0) : 0.f, in_bounds(p1 - base, 9ull * N) ? ldpop<CG>(p1) : 0.f);
+        h[i] = V(in_bounds(p0 - base, 9ull * N) ? ldpop(p0) : 0.f, in_bounds(p1 - base, 9ull * N) ? ldpop(p1) : 0.f);
     }
 }
 
@@ -172,7 +171,7 @@ __device__ __forceinline__ void pull18_dev(const float *base_, const float *R, u
     const unsigned short *base = reinterpret_cast<const unsigned short *>(base_);
     auto one = [&](int cx, int cy, unsigned i, unsigned n) {
         if (!(in_bounds(i * N + n, 9ull * N) && in_bounds(n, N))) return 0.f;
-        const float d = Bits16<S>::to_f(__ldg(base + i * N + n));
+        const float d = Bits16<S>::to_f(__ldca(base + i * N + n));
         const Ref16 r = load_rec(R, N, n);
         return G ? decode_g<9>(cx, cy, 0, r, d) : decode_f<9>(cx, cy, 0, r, d);
     };
@@ -189,20 +188,19 @@ __device__ __forceinline__ v2 sum9(const v2 h[9])
 }
 
 // One tile: rows y0 .. y0 + rows - 1 (y0 even, y0 + rows <= ny) of strip bx of layer
-// bz.  smem holds smem_of<kW>() bytes.  CG selects loads that may see populations
-// written by other CTAs of the same launch.  A CTA that runs several tiles must pass a
+// bz.  smem holds smem_of<kW>() bytes.  A CTA that runs several tiles must pass a
 // barrier between them (the rings are reused).  WALLS compiles in the wall columns
 // (FusedArgs::walls); without it the kernel has no trace of them.  MomentArgs stop it after
 // stage C, which writes the macroscopic fields: A then runs on 2 halo columns and 1 halo row
 // pair, B on 1 column, C on the strip itself, and smem holds moments_smem_of<kW>() bytes.
-template <int kW, bool THERMAL, bool CG, bool WALLS = false, typename ST = float, class ARGS = FusedArgs>
+template <int kW, bool THERMAL, bool WALLS = false, typename ST = float, class ARGS = FusedArgs>
 __device__ __forceinline__ void fused_tile(const ARGS &A, int bx, int y0, int rows, int bz, v2 *smem)
 {
     constexpr bool MOM = std::is_same<ARGS, MomentArgs>::value;
     // 16-bit deviation storage (ST = __half / __nv_bfloat16): pulls decode, stage D encodes
     // against the node's new reference record (dev16.cuh); no wall columns, no ensemble.
     constexpr bool DEV = Store<ST>::dev;
-    static_assert(!(DEV && (WALLS || CG)), "16-bit storage runs the single-lattice kernel without walls");
+    static_assert(!(DEV && WALLS), "16-bit storage runs without walls");
     constexpr int S = slots_of<kW>();
     enum { RHO, JX, JY, PXX, PXY, PYY, UX, UY, QX, QY, WQ };
     auto fld = [&](int field, int slot3) -> v2 * { return smem + (field * kDepth + slot3) * S; };
@@ -262,9 +260,9 @@ __device__ __forceinline__ void fused_tile(const ARGS &A, int bx, int y0, int ro
             if (gp) pull18_dev<ST, true>(base, A.Rin, N, ro, cols, h);
             else pull18_dev<ST, false>(base, A.Rin, N, ro, cols, h);
         } else if (wallc) {
-            pull_own<CG>(base, N, ro, cols[1], h);
+            pull_own(base, N, ro, cols[1], h);
         } else {
-            pull18<CG>(base, N, ro, cols, h);
+            pull18(base, N, ro, cols, h);
         }
     };
     auto rows4 = [&](int r, unsigned ro[4]) {      // rows r-1 .. r+2 of the layer
@@ -327,8 +325,8 @@ __device__ __forceinline__ void fused_tile(const ARGS &A, int bx, int y0, int ro
                         const int i = (s + 1) + 3 * (cy + 1);
                         const float *pp = A.f + i * N + cols[1 - s];
                         const float *p0 = pp + ro[1 - cy], *p1 = pp + ro[2 - cy];
-                        m = m + V(in_bounds(p0 - A.f, 9ull * N) ? ldpop<CG>(p0) : 0.f,
-                                  in_bounds(p1 - A.f, 9ull * N) ? ldpop<CG>(p1) : 0.f);
+                        m = m + V(in_bounds(p0 - A.f, 9ull * N) ? ldpop(p0) : 0.f,
+                                  in_bounds(p1 - A.f, 9ull * N) ? ldpop(p1) : 0.f);
                     }
                     fr[0] = m;
                 } else {
@@ -412,7 +410,7 @@ __device__ __forceinline__ void fused_tile(const ARGS &A, int bx, int y0, int ro
             } else {
                 const float *Tp = A.RT_iso + layer + cols[1];
                 const float *T0 = Tp + (unsigned)rC * nx, *T1 = Tp + (unsigned)next_row(rC, ny) * nx;
-                RT = V(in_bounds(T0 - A.RT_iso, N) ? ldpop<CG>(T0) : 0.f, in_bounds(T1 - A.RT_iso, N) ? ldpop<CG>(T1) : 0.f);
+                RT = V(in_bounds(T0 - A.RT_iso, N) ? ldpop(T0) : 0.f, in_bounds(T1 - A.RT_iso, N) ? ldpop(T1) : 0.f);
                 rC = next_row(next_row(rC, ny), ny);
             }
             if constexpr (MOM) {

@@ -202,12 +202,12 @@ __device__ __forceinline__ void tm_ld9f(uint32_t tb, int s, int kz, float v[9])
 // 16-bit storage loads and stores the raw deviation.
 __device__ __forceinline__ float ldc(const float *base, unsigned off, unsigned long long n)
 {
-    return in_bounds(off, n) ? __ldg(base + off) : 0.f;
+    return in_bounds(off, n) ? base[off] : 0.f;
 }
 template <typename S>
 __device__ __forceinline__ float ldc(const S *base, unsigned off, unsigned long long n)
 {
-    return in_bounds(off, n) ? Bits16<S>::to_f(__ldg(reinterpret_cast<const unsigned short *>(base) + off)) : 0.f;
+    return in_bounds(off, n) ? Bits16<S>::to_f(__ldca(reinterpret_cast<const unsigned short *>(base) + off)) : 0.f;
 }
 __device__ __forceinline__ void stc(float *base, unsigned off, unsigned long long n, float v)
 {

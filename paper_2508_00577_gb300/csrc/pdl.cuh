@@ -3,8 +3,9 @@
 // global memory, which returns when the kernel before it has completed and its writes are
 // visible (so buffers may be read and rewritten as after an ordinary launch), then
 // pdl_trigger(), which allows the kernel after it to be placed as soon as every block of this
-// one has started.  (The trigger comes after the wait, so that at most two grids overlap and
-// the L1 lines a grid cached of a buffer are dropped before a later grid reads it rewritten.)
+// one has started.  The trigger comes after the wait, so that at most two grids overlap.  What
+// the grids before it write is not read-only data for such a kernel, although it reads it only
+// after the wait: its loads are plain ones (__ldca), not ld.global.nc (__ldg).
 // Both are no-ops without the launch attribute.  What overlaps is the launch itself, 1 to
 // 2 us; us per window: 384 x 4 D2Q9 50 steps 320 -> 204, 64^2 FP64 20 steps of four stage
 // kernels 885 -> 694, 256^2 x 16 50 steps 2504 -> 2407, 75 x 50 x 61 D3Q27 20 steps 2041 -> 1950.

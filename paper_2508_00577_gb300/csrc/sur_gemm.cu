@@ -139,7 +139,7 @@ __device__ __forceinline__ void epilogue(const Epi &g, uint32_t tmem, long long 
         if ((reinterpret_cast<uintptr_t>(b) & 15) == 0) {
 #pragma unroll
             for (int j = 0; j < CS / 4; ++j) {
-                const float4 q = __ldg(reinterpret_cast<const float4 *>(b) + j);
+                const float4 q = __ldca(reinterpret_cast<const float4 *>(b) + j);
                 v[4 * j] += q.x;
                 v[4 * j + 1] += q.y;
                 v[4 * j + 2] += q.z;
@@ -147,7 +147,7 @@ __device__ __forceinline__ void epilogue(const Epi &g, uint32_t tmem, long long 
             }
         } else {
 #pragma unroll
-            for (int j = 0; j < CS; ++j) v[j] += __ldg(b + j);
+            for (int j = 0; j < CS; ++j) v[j] += __ldca(b + j);
         }
     };
 #pragma unroll 1
@@ -868,7 +868,7 @@ __global__ void __launch_bounds__(32 * (CfgR<C, N>::EW + 2), CfgR<C, N>::CTAS)
             uint32_t off = rbase - wbase + (uint32_t)(Cf::SLOTS * Cf::ROW + (i - 10 * N) * 16);
             if (i < 10 * N) {
                 const int tap = i / N, n = i % N;
-                if (tap < 9) v = __ldg(reinterpret_cast<const uint4 *>(g.w + (long long)n * g.wld + g.b_c0 + tap * 8));
+                if (tap < 9) v = __ldca(reinterpret_cast<const uint4 *>(g.w + (long long)n * g.wld + g.b_c0 + tap * 8));
                 off = (uint32_t)((tap * (N / 8) + n / 8) * 128 + n % 8 * 16);
             }
             *reinterpret_cast<uint4 *>(wp + off) = v;
