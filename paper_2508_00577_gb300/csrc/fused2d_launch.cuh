@@ -123,15 +123,24 @@ cudaError_t launch_w(const FusedArgs &A, int nz, bool balanced, bool follows, cu
         resident = per_sm * sms;
         attr = true;
     }
+    // Wall columns make the CTAs of a strip's two ends longer than the others (they solve for the
+    // wall's density).  Where about all slots are taken, the next grid's CTAs would fill them in the
+    // order in which this one's end, the long ones last and together: 512^2 x 4 layers 75.0 us a
+    // step overlapping and 72.9 apart, 1024^2 x 4 in strips of 128 and chunks of 128 rows 269 and
+    // 259; but 130 x 130 7.9 and 10.2, and 2048 CTAs (64 x 32) 232 and 235.
+    auto overlaps = [&](long long ctas) {
+        return follows && !(WALLS && 2 * ctas > resident && ctas < 2LL * resident);
+    };
     if (balanced) {
         const int S = (A.nx + W - 1) / W;
         const long long parts = min((long long)max(resident / S, 1), (long long)nz * ((A.ny + 1) / 2));
-        return launch_overlap(follows, k_fused2d_bal<W, THERMAL, WALLS, ST>, dim3((unsigned)(S * parts)),
+        return launch_overlap(overlaps(S * parts), k_fused2d_bal<W, THERMAL, WALLS, ST>, dim3((unsigned)(S * parts)),
                               threads_of<W>(), smem, st, A);
     }
     return in_layers(A, nz, [&](const FusedArgs &B, int layers) {
         const dim3 grid((B.nx + W - 1) / W, (B.ny + B.H - 1) / B.H, layers);
-        return launch_overlap(follows, k_fused2d<W, THERMAL, WALLS, ST>, grid, threads_of<W>(), smem, st, B);
+        return launch_overlap(overlaps((long long)grid.x * grid.y * grid.z), k_fused2d<W, THERMAL, WALLS, ST>, grid,
+                              threads_of<W>(), smem, st, B);
     });
 }
 
