@@ -612,7 +612,7 @@ int lbm_autotune(lbm_ctx *c, int probe_steps, int *tile_w, int *tile_h)
     for (int round = 0; round < kAutotuneRounds; ++round)
     for (int wi = 0; wi < evlbm::kFusedWidthCount && e == cudaSuccess; ++wi) {
         const int W = evlbm::kFusedWidths[wi];
-        if (W > 2 * c->P.nx && W != evlbm::kFusedWidths[0]) continue;
+        if (W > 2 * c->P.nx && W != evlbm::kFusedWidths[0] && W != dw) continue;
         for (int hi = 0; hi < kH && e == cudaSuccess; ++hi) {
             const int H = heights[hi] < c->P.ny ? heights[hi] : c->P.ny;    // the balanced grid stays -1
             if (hi == kH - 1 && (W != dw || dh == LBM_TILE_BALANCED)) continue;
