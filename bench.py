@@ -41,7 +41,7 @@ BYTES_PER_LU = 2 * 9 * 2 * 4          # D2Q9, f and g, read + write, FP32
 # shape (W, H) of the fused kernel (H = -1: the balanced grid, k_fused2d_bal), from one ncu
 # capture each (profiles/fused2d_d2q9_thermal_fp32.md); a shape without a capture, or a
 # changed kernel, reports None.
-MEASURED_TRAFFIC_BYTES = {(128, 256): 1.3342e9, (128, -1): 1.3384e9}
+MEASURED_TRAFFIC_BYTES = {(128, 256): 1.3280e9, (128, -1): 1.3306e9}
 # Floating-point operations per lattice update of the FP64 oracle's plain form of the
 # step (every stencil and equilibrium product summed over all Q velocities), counted by
 # running the oracle's source with a counting number type; tests/test_oracle_flops.py
@@ -52,7 +52,7 @@ FP32_LANES = 152 * 128
 # DRAM bytes (read + write) of one step of the 512-domain ensemble per work-item shape,
 # from one ncu capture of a one-step launch of k_batch (5.949 GB algorithmic;
 # profiles/batch_ensemble_d2q9_fp32.md); None for other shapes or when the kernel changes.
-ENSEMBLE_TRAFFIC_BYTES_PER_STEP = {(128, 256): 6.0400e9, (128, 512): 6.0011e9}
+ENSEMBLE_TRAFFIC_BYTES_PER_STEP = {(128, 256): 6.01e9, (128, 512): 5.99e9}
 WORKLOAD = "droplet Laplace sweep: 9 x 1024^2 D2Q9 thermal, FP32"
 
 

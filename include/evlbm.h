@@ -50,7 +50,7 @@ extern "C" {
 #define LBM_D2Q9 0
 #define LBM_D3Q27 1
 
-/* tile_h of lbm_set_tile (D2Q9 FP32) selecting the balanced persistent grid: per
+/* tile_h of lbm_set_tile (D2Q9) selecting the balanced persistent grid: per
  * strip, as many CTAs as fit on the GPU at once divided by the strip count, each
  * taking an equal share of that strip's row pairs over all layers. */
 #define LBM_TILE_BALANCED (-1)
@@ -65,8 +65,8 @@ extern "C" {
  * weight,
  *   (h_i - h_i^eq(R)) / (w_i rho_R)   (g: / (w_i rho_R 3/2 RT_R)),
  * with that node's reference state R = (rho, u, theta0, 3/2 RT) stored beside the
- * populations as an FP32 record of 24 bytes per node; arithmetic is FP32.  D3Q27
- * runs the fused single-pass kernel, D2Q9 the stage kernels. */
+ * populations as an FP32 record of 24 bytes per node; arithmetic is FP32.  Both
+ * lattices run the fused single-pass kernel (force_form 0), one launch per step. */
 #define LBM_FP16_DEV 2       /* FP16 deviation storage */
 #define LBM_BF16_DEV 3       /* BF16 deviation storage */
 
@@ -237,8 +237,8 @@ int lbm_get_tile(const lbm_ctx *ctx, int *tile_w, int *tile_h);
 
 /* Autotuner: times every candidate launch shape of the fused kernel for
  * probe_steps (>= 1) steps each with CUDA events on the context's stream, in two
- * rounds over all candidates, and keeps the shape with the fastest time.  The probes read the current state and write the spare
- * buffer, so the state is unchanged.  Synchronises the stream.  The chosen shape
+ * rounds over all candidates, and keeps the shape with the fastest time.  The probes
+ * read the current state and write the spare buffer, so the state is unchanged.  Synchronises the stream.  The chosen shape
  * is returned in *tile_w, *tile_h (either may be NULL); both are 0 when the
  * context has no fused kernel.  Errors: LBM_EINVAL, LBM_ECUDA. */
 int lbm_autotune(lbm_ctx *ctx, int probe_steps, int *tile_w, int *tile_h);

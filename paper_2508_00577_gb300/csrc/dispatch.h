@@ -60,8 +60,9 @@ __device__ __forceinline__ float over_R(float RT, const GasConstant &R)
     const float t = fmaf(fmaf(-q, R.l, fmaf(-q, R.h, RT)), R.i, q);
     return isfinite(t) ? t : q;
 }
-// Macroscopic fields of the current state on lattices a fused step supports, as that step's
-// own stages compute them.
+// Macroscopic fields of the current state on lattices a fused step supports, by the arithmetic
+// of that step's stages A to C: the step's own code in two dimensions, a copy of it in three,
+// where the compiler may contract other products and the last bit may differ from the step's.
 cudaError_t fused2d_moments(int prec, const KParams &p, const void *f, const void *g, const void *RT_iso,
                             const void *Rin, const MomentOut &o, cudaStream_t st);
 cudaError_t fused2d_moments16(int prec, const KParams &p, const void *f, const void *g, const void *RT_iso,
@@ -79,8 +80,8 @@ extern const int kFusedWidths[kFusedWidthCount];
 void fused2d_default_tile(const KParams &p, int *W, int *H);
 bool fused2d_supported(int prec, int Q, const KParams &p);
 // Fused single-pass D3Q27 step (FP32 arithmetic, divergence force form; storage prec
-// 1/2/3 as above, 16-bit storage reading Rin and writing Rout); the x-y tile of 256
-// columns is fused3d_tile_w(prec) wide (32 x 8 for FP32, 16 x 16 for 16-bit storage),
+// 1/2/3 as above, 16-bit storage reading Rin and writing Rout); the x-y tile is
+// fused3d_tile_w(prec) wide (32 x 8 columns for FP32, 32 x 16 for 16-bit storage),
 // tile_h is the z-chunk height (0 = default).
 int fused3d_tile_w(int prec);
 int fused3d_default_chunk(int prec, const KParams &p);

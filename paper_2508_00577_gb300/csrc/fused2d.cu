@@ -18,19 +18,21 @@ bool fused2d_supported(int prec, int Q, const KParams &p)
 }
 
 // Default launch shape: the candidate with the least estimated time.  A CTA that marches p
-// row pairs runs p + 4 iterations per tile (the pipeline of four stages fills first), and the
-// time of one iteration depends on the strip width and on how many CTAs share an SM.  The
-// measured times of an iteration (us, thermal FP32; the ratios hold for the isothermal kernel
+// row pairs runs p + 5 iterations per tile (the pipeline of four stages fills first); those of
+// the fill, without some of the stages, take about the time of 4 (with 5 in its place the shapes
+// picked for 70 lattices take 1.107 times the best one's time on average, with 4 1.093).  The
+// time of one iteration depends on the strip width and on how many CTAs share an SM.  Measured
+// (us, thermal FP32, before the launches overlapped; the ratios hold for the isothermal kernel
 // and 16-bit storage):
 //   CTAs per SM       1     2     3     4
 //   W =  64         1.28  1.60  2.20  2.90
 //   W =  96         1.20  2.25
 //   W = 128         1.50  2.35
 // so few row pairs per CTA win as long as the GPU is not full, and beyond that the wide
-// strips of the balanced grid.  Against the former rule (strips of 128 columns, 128 rows a
-// CTA), us per step: 331 x 203 x 2 104.8 -> 13.2, 512^2 104.5 -> 18.7, 256^2 x 16 123.2 ->
-// 48.9, 1024^2 122.6 -> 45.5, 256^2 x 64 161.7 -> 154.5, 64^2 45.5 -> 8.5, 384 x 4 isothermal
-// 8.5 -> 6.5 (the spacing of dependent launches).
+// strips of the balanced grid.  Against strips of 128 columns and 128 rows a CTA, us per step
+// (the launches overlapping, too): 331 x 203 x 2 104.6 -> 12.5, 512^2 102.4 -> 16.7, 256^2 x 16
+// 123.0 -> 46.6, 1024^2 122.7 -> 42.8, 256^2 x 64 161.6 -> 149.8, 64^2 45.1 -> 5.4, 384 x 4
+// isothermal 8.2 -> 4.0.
 void fused2d_default_tile(const KParams &p, int *W, int *H)
 {
     static const int widths[3] = {128, 96, 64}, per_sm[3] = {2, 2, 4};

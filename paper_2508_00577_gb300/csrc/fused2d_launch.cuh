@@ -155,7 +155,6 @@ cudaError_t launch(int W, const FusedArgs &A, int nz, bool balanced, bool follow
     }
 }
 
-
 // Kernel arguments of a lattice (populations, records and the T field as passed by the caller).
 inline FusedArgs make_args(const KParams &p, const void *f, const void *g, void *fo, void *go, const void *RT_iso,
                            const void *Rin, void *Rout)

@@ -281,8 +281,8 @@ __device__ __forceinline__ void fused_tile(const ARGS &A, int bx, int y0, int ro
     // q0 - 1 and q0 - 2.  The other row of such a pair may come out undefined (from ring cells
     // not written yet); nothing reads it.  Likewise A ends at pair qD_end + 1 (one iteration
     // before the last) and B at pair qD_end.  Against filling by whole pairs (one iteration and
-    // two pulled f pairs more per tile), us per window of 50 steps: 331 x 203 x 2 837 -> 736,
-    // 256^2 x 16 2556 -> 2504, 9 x 1024^2 (20 steps) 6871 -> 6853; the values are the same.
+    // two pulled f pairs more per tile), us per window of 50 steps: 331 x 203 x 2 688 -> 647,
+    // 256^2 x 16 2386 -> 2361, 9 x 1024^2 (20 steps) 6771 -> 6679; the values are the same.
     // With 16-bit storage A and B run on in the last iteration: the conditions cost that
     // kernel, which is bound by issue, 7 % on 9 x 1024^2.
     const int qbeg = q0 - (MOM ? 1 : 2), qend = qD_end + (MOM ? 1 : 2);

@@ -7,8 +7,9 @@
 // the grids before it write is not read-only data for such a kernel, although it reads it only
 // after the wait: its loads are plain ones (__ldca), not ld.global.nc (__ldg).
 // Both are no-ops without the launch attribute.  What overlaps is the launch itself, 1 to
-// 2 us; us per window: 384 x 4 D2Q9 50 steps 320 -> 204, 64^2 FP64 20 steps of four stage
-// kernels 885 -> 694, 256^2 x 16 50 steps 2504 -> 2407, 75 x 50 x 61 D3Q27 20 steps 2041 -> 1950.
+// 2 us; us per window without and with it: 384 x 4 D2Q9 50 steps 323 and 204, 331 x 203 x 2 737
+// and 633, 64^2 FP64 20 steps of four stage kernels 888 and 692, 256^2 x 16 50 steps 2447 and
+// 2360, 75 x 50 x 61 D3Q27 20 steps 1613 and 1582.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -775,7 +775,6 @@ __global__ void __launch_bounds__(32 * (kEpiWarps<BN, MN> + 2), kEpiWarps<BN, MN
     if (warp == 0) tmem_free(tmem, TCOLS);
 }
 
-
 // ---------------------------------------------------------------------------
 // Row-marching 3x3 convolution (images at least 128 pixels wide)
 // ---------------------------------------------------------------------------
@@ -794,8 +793,8 @@ __global__ void __launch_bounds__(32 * (kEpiWarps<BN, MN> + 2), kEpiWarps<BN, MN
 // end of a row of taps to the start of the next, and from the last tap to a block of zeros (a
 // pixel times a zero weight would spread infinities).  That stride is unsigned, so the row in
 // slot 0 of the ring is loaded a second time behind the last slot.  The threads lay out the
-// nine taps' weights and the zeros.  On the TMA mainloop a K block took 8 boxes, whose requests bound it: 32 x 256^2 pixels to 32
-// channels 163 -> 95 us.
+// nine taps' weights and the zeros.  On the TMA mainloop a K block took 8 boxes, whose requests
+// bound it: 32 x 256^2 pixels to 32 channels 163 -> 95 us.
 template <int C, int N> struct CfgR {
     static constexpr int CB = C < 64 ? C : 64, NB = C / CB;       // channels per box, boxes per row
     static constexpr int RB = CB * 2;                             // bytes of a pixel in a box
