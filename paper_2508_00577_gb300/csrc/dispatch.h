@@ -53,12 +53,12 @@ struct GasConstant {
     explicit GasConstant(double R = 1.0) : h(float(R)), l(float(R - double(h))), i(float(1.0 / R)) {}
 };
 // R T / R to within a rounding, exact for R = 1: the quotient by the reciprocal and its residual's
-// correction, which an infinite quotient does not have (inf - inf).
+// correction.  An infinite quotient has no residual (inf - inf); the minimum makes a number of it,
+// so that the sum stays infinite (256^3 FP16 4720 us; 4780 with a selection of the quotient).
 __device__ __forceinline__ float over_R(float RT, const GasConstant &R)
 {
     const float q = RT * R.i;
-    const float t = fmaf(fmaf(-q, R.l, fmaf(-q, R.h, RT)), R.i, q);
-    return isfinite(t) ? t : q;
+    return fmaf(fminf(fmaf(-q, R.l, fmaf(-q, R.h, RT)), 3.4028235e38f), R.i, q);
 }
 // Macroscopic fields of the current state on lattices a fused step supports, by the arithmetic
 // of that step's stages A to C: the step's own code in two dimensions, a copy of it in three,
