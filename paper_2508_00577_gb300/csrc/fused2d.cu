@@ -39,10 +39,7 @@ void fused2d_default_tile(const KParams &p, int *W, int *H)
     static const float iter_us[3][4] = {{1.50f, 2.35f, 0.f, 0.f}, {1.20f, 2.25f, 0.f, 0.f}, {1.28f, 1.60f, 2.20f, 2.90f}};
     static const int heights[] = {2, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 256};
     constexpr int kFill = 4;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-        sms = 152;
+    const int sms = sm_count();
     const long long P = (p.ny + 1) / 2;                      // row pairs of a layer
     double best = 1e300;
     for (int k = 0; k < 3; ++k) {

@@ -83,7 +83,7 @@ cudaError_t launch_moments(MomentArgs A, int nz, cudaStream_t st)
 {
     const int W = A.nx > 64 ? 128 : 64, S = (A.nx + W - 1) / W;
     A.H = 32;
-    while (A.H > 4 && (long long)S * ((A.ny + A.H - 1) / A.H) * nz < 456) A.H >>= 1;
+    while (A.H > 4 && (long long)S * ((A.ny + A.H - 1) / A.H) * nz < 3 * sm_count()) A.H >>= 1;
     return in_layers(A, nz, [&](const MomentArgs &B, int layers) {
         const dim3 grid(S, (B.ny + B.H - 1) / B.H, layers);
         return W == 64 ? launch_pdl(k_moments2d<64, THERMAL, WALLS, ST>, grid, threads_of<64>(), moments_smem_of<64>(), st, B)
@@ -112,15 +112,13 @@ cudaError_t launch_w(const FusedArgs &A, int nz, bool balanced, bool follows, cu
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_fused2d_bal<W, THERMAL, WALLS, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem);
-        int per_sm = 0, dev = 0, sms = 0;
+        int per_sm = 0;
         if (e == cudaSuccess)
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fused2d_bal<W, THERMAL, WALLS, ST>,
                                                               threads_of<W>(), smem);
-        if (e == cudaSuccess) e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
         if (per_sm < 1) return cudaErrorLaunchOutOfResources;
-        resident = per_sm * sms;
+        resident = per_sm * sm_count();
         attr = true;
     }
     // Wall columns make the CTAs of a strip's two ends longer than the others (they solve for the

@@ -1008,16 +1008,6 @@ __global__ void __launch_bounds__(MGeo::NT, 3) k_moments3d(const Args<S> A, cons
     }
 }
 
-int sm_count()
-{
-    static int sms = 0;
-    int dev = 0;
-    if (!sms && (cudaGetDevice(&dev) != cudaSuccess ||
-                 cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1))
-        sms = 152;
-    return sms;
-}
-
 template <bool THERMAL, typename S, bool ONE>
 cudaError_t launch_k(const Args<S> &A, dim3 grid, cudaStream_t st)
 {
@@ -1171,11 +1161,11 @@ cudaError_t moments_t(const KParams &p, const void *f, const void *g, const void
     M.F = o.F;
     M.R = GasConstant(o.R);
     // Chunks of 32 planes (after 4 that fill the pipeline), shorter while the grid would leave
-    // slots of the GPU (152 SMs x 3) empty.  The tiles run along the grid's x, which alone is
+    // slots of the GPU (three CTAs an SM) empty.  The tiles run along the grid's x, which alone is
     // not limited to 65535.
     const long long tiles = (long long)((p.nx + MGeo::TX - 1) / MGeo::TX) * ((p.ny + MGeo::TY - 1) / MGeo::TY);
     A.HZ = 32;
-    while (A.HZ > 2 && tiles * ((p.nz + A.HZ - 1) / A.HZ) < 456) A.HZ >>= 1;
+    while (A.HZ > 2 && tiles * ((p.nz + A.HZ - 1) / A.HZ) < 3 * sm_count()) A.HZ >>= 1;
     while ((p.nz + A.HZ - 1) / A.HZ > 65535) A.HZ <<= 1;
     const dim3 grid((unsigned)tiles, (p.nz + A.HZ - 1) / A.HZ);
     return p.thermal ? launch_pdl(k_moments3d<true, S>, grid, MGeo::NT, 0, st, A, M)

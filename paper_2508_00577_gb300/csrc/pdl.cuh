@@ -16,6 +16,18 @@
 
 namespace evlbm {
 
+// SMs of the device (152 where there is none to ask).
+inline int sm_count()
+{
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        const bool ok = cudaGetDevice(&dev) == cudaSuccess &&
+                        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+        return ok && n > 0 ? n : 152;
+    }();
+    return sms;
+}
+
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -37,7 +37,7 @@ inline RefFields<real> ref_fields(void *scratch, long long N, const void *RT_iso
 inline int node_block(long long N)
 {
     int b = 256;
-    while (b > 32 && N < 304LL * b) b >>= 1;
+    while (b > 32 && N < 2LL * sm_count() * b) b >>= 1;
     return b;
 }
 

@@ -25,12 +25,12 @@ inline int grid_1d(long long n)
 }
 
 // Grid of the activation kernels: what is resident at once (per_sm blocks of 256 threads, by
-// registers, on each of the 152 SMs), each block striding over the tensor.  Those that end in
-// per-channel atomics (block_colsum8) so add at most 152 per_sm values to each accumulator.
+// registers, on each SM), each block striding over the tensor.  Those that end in
+// per-channel atomics (block_colsum8) so add at most that many values to each accumulator.
 inline int grid_res(long long n, int per_sm)
 {
-    const int g = grid_1d(n);
-    return g > 152 * per_sm ? 152 * per_sm : g;
+    const int g = grid_1d(n), most = evlbm::sm_count() * per_sm;
+    return g > most ? most : g;
 }
 
 inline int log2i(int v)
